@@ -79,7 +79,6 @@ int choose_pcg_cta(mpcg_handle *h, const mpcg_dims &d, int B, PcgLaunch &L) {
     else return MPCG_EUNSUPPORTED;
     L.cta_mode = 1;
     L.C = 1;
-    L.mode = MODE_PTR;
     L.stage = 0;
     L.threads = kMaxThreads;
     L.vs = nx <= 16 ? 16 : ceil_div(nx, 4) * 4;
@@ -109,7 +108,6 @@ int choose_pcg_tile(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_schur 
         if (ptr && ((uintptr_t)ptr % 16) != 0) return MPCG_EUNSUPPORTED;
     L.cta_mode = 2;
     L.C = 1;
-    L.mode = MODE_PTR;
     L.stage = 0;
     L.lpk = nx <= 16 ? 16 : 32;
     L.rpt = nx <= 32 ? 1 : 2;
@@ -163,7 +161,61 @@ int choose_pcg_tile(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_schur 
     return MPCG_OK;
 }
 
-// Launch shape of the cluster PCG kernel for horizons up to Nmax.  `wide`
+// Launch shape of the register-resident cluster kernel (float32, nx = 14;
+// pcg_reg.cu): up to 32 knots per CTA.
+//  - opts.cluster given: that many CTAs per instance.
+//  - Every instance can have its own cluster at once: the largest cluster that
+//    still allows it, down to about 8 knots per CTA (fewer warps per CTA
+//    barrier; a single instance of 64 / 128 knots).
+//  - More instances than clusters: full CTAs, a power of two per cluster, and
+//    clusters that split into groups as the long horizons run out.
+inline int choose_pcg_reg(const mpcg_dims &d, int B, const mpcg_opts *o, PcgLaunch &L) {
+    constexpr int kpc_cap = 32, kpc_small = 8;
+    L.cta_mode = 0;
+    L.reg = 1;
+    L.lpk = 8;
+    L.rpt = 2;
+    L.vs = 16;
+    const int C_full = ceil_div(d.N, kpc_cap);
+    if (C_full > kMaxCluster) return MPCG_EUNSUPPORTED;
+    auto shape = [&](int C) {  // co-resident clusters of C CTAs (0: cannot run)
+        L.C = C;
+        L.kpc_max = ceil_div(d.N, C);
+        if (L.kpc_max > kpc_cap) return 0;
+        L.threads = std::max(32, ceil_div(L.kpc_max * L.lpk, 32) * 32);
+        L.smem = pcg_reg_smem_bytes(L.kpc_max);
+        return pcg_reg_max_clusters(L);
+    };
+    if (o && o->cluster > 0) {
+        if (o->cluster > kMaxCluster) return MPCG_EUNSUPPORTED;
+        const int n = shape(std::min(o->cluster, d.N));
+        if (n < 1) return MPCG_EUNSUPPORTED;
+        L.clusters = std::min(B, n);
+        return MPCG_OK;
+    }
+    for (int C = std::min(kMaxCluster, std::max(C_full, ceil_div(d.N, kpc_small))); C >= C_full; --C)
+        if (shape(C) >= B) {
+            L.clusters = B;
+            return MPCG_OK;
+        }
+    int C = 1;
+    while (C < C_full) C <<= 1;
+    for (; C >= C_full && C >= 1; C >>= 1) {
+        L.C = C;
+        L.kpc_max = C > 1 ? kpc_cap : d.N;
+        L.threads = std::max(32, ceil_div(L.kpc_max * L.lpk, 32) * 32);
+        L.smem = pcg_reg_smem_bytes(L.kpc_max);
+        const int n = pcg_reg_max_clusters(L);
+        if (n >= 1) {
+            L.split = C > 1 && n < B;
+            L.clusters = std::min(B, n);
+            return MPCG_OK;
+        }
+    }
+    return MPCG_EUNSUPPORTED;
+}
+
+// Launch shape of the cluster PCG kernels for horizons up to Nmax.  `wide`
 // (opts.mode = 4, nx <= 16): operators staged in shared memory, 8 lanes x 2
 // rows per knot, up to 64 knots per CTA -- half the SMs per instance of the
 // register-resident form, for throughput.
@@ -174,24 +226,18 @@ int choose_pcg_cluster(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opt
     L.dot = (std::is_same<T, float>::value && o && o->dot == 1) ? 1 : 0;
     const int nx = d.nx;
     if (wide && nx > 16) return MPCG_EUNSUPPORTED;
-    const bool reg = !wide && std::is_same<T, float>::value && nx == 14;
-    int max_threads = kMaxThreads;
-    if (reg) { L.lpk = 8; L.rpt = 2; max_threads = 256; }  // 2 register-resident rows per thread
-    else if (wide) { L.lpk = 8; L.rpt = 2; }
+    if (!wide && std::is_same<T, float>::value && nx == 14) return choose_pcg_reg(d, B, o, L);
+    if (wide) { L.lpk = 8; L.rpt = 2; }
     else if (nx <= 16) { L.lpk = 16; L.rpt = 1; }
     else if (nx <= 32) { L.lpk = 32; L.rpt = 1; }
     else if (nx <= 64) { L.lpk = 32; L.rpt = 2; }
     else return MPCG_EUNSUPPORTED;
-    const int kpc_cap = max_threads / L.lpk;  // knot slots per CTA
-    // A single instance runs fastest spread over more CTAs than it fills:
-    // register form (float32, nx = 14) at about 8 knots per CTA (fewer warps
-    // per CTA barrier and reduction tree; measured on GB300, N = 64 / 128:
-    // 402 / 697 us against 447 / 765 us with full 32-knot CTAs), the shared-
-    // memory form at the largest cluster (each lane's rows per iteration grow
-    // with the knots per CTA: FP64 N = 128 4.9 ms at 16 CTAs against 13.0 ms
-    // at 4; nx = 36 N = 64 2.0 against 4.3 ms).  Batches fill the CTAs (the
-    // autotuner tries the other packings).
-    const int kpc_pref = B > 1 ? kpc_cap : (reg ? std::min(kpc_cap, 8) : 1);
+    const int kpc_cap = kMaxThreads / L.lpk;  // knot slots per CTA
+    // A single instance runs fastest at the largest cluster (each lane's rows
+    // per iteration grow with the knots per CTA: FP64 N = 128 4.9 ms at 16
+    // CTAs against 13.0 ms at 4; nx = 36 N = 64 2.0 against 4.3 ms).  Batches
+    // fill the CTAs (the autotuner tries the other packings).
+    const int kpc_pref = B > 1 ? kpc_cap : 1;
     int C = (o && o->cluster > 0) ? o->cluster : std::min(kMaxCluster, ceil_div(d.N, kpc_pref));
     if (!(o && o->cluster > 0)) C = std::max(C, ceil_div(d.N, kpc_cap));
     if (C > kMaxCluster) return MPCG_EUNSUPPORTED;
@@ -201,14 +247,10 @@ int choose_pcg_cluster(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opt
         L.kpc_max = ceil_div(d.N, C);
         if (L.kpc_max > kpc_cap) return MPCG_EUNSUPPORTED;
         L.threads = std::max(32, ceil_div(L.kpc_max * L.lpk, 32) * 32);
-        L.mode = reg ? MODE_REG : MODE_PTR;
         L.vs = nx <= 16 ? 16 : ceil_div(nx, 4) * 4;
         const int W = L.threads / 32;
         L.stage = 0;
-        if (L.mode == MODE_PTR) {
-            size_t with = pcg_smem_bytes<T>(L.kpc_max, L.vs, C, W, nx, 1, L.dot);
-            if (with <= (size_t)h->smem_optin) L.stage = 1;
-        }
+        if (pcg_smem_bytes<T>(L.kpc_max, L.vs, C, W, nx, 1, L.dot) <= (size_t)h->smem_optin) L.stage = 1;
         L.smem = pcg_smem_bytes<T>(L.kpc_max, L.vs, C, W, nx, L.stage, L.dot);
         const int active = pcg_max_clusters<T>(L);
         if (active >= 1) {
@@ -345,11 +387,14 @@ int pcg_t(mpcg_handle *h, const mpcg_dims &d, int B, const int *knot_off, const 
     if (P.n_tickets > 1 && L.clusters < P.n_tickets) {
         if (!ws) return MPCG_EINVAL;
         P.queue = (int *)ws;
-        rc = err_cuda(cudaMemsetAsync(ws, 0, sizeof(int), st));
+        rc = err_cuda(cudaMemsetAsync(ws, 0, 8 * sizeof(int), st));  // one counter per group level
         if (rc) return rc;
     }
     if (L.cta_mode == 2) return err_cuda(pcg_tile_launch<T>(L, P, st));
     if (L.cta_mode == 1) return err_cuda(pcg_cta_launch<T>(L, P, st));
+    if constexpr (std::is_same<T, float>::value) {
+        if (L.reg) return err_cuda(pcg_reg_launch(L, P, st));
+    }
     return err_cuda(pcg_launch<T>(L, P, st));
 }
 
@@ -551,7 +596,7 @@ int mpcg_create(mpcg_handle **out) {
         delete h;
         return MPCG_ECUDA;
     }
-    if (pcg_prepare(h->smem_optin) != cudaSuccess || pcg_cta_prepare(h->smem_optin) != cudaSuccess ||
+    if (pcg_prepare(h->smem_optin) != cudaSuccess || pcg_reg_prepare() != cudaSuccess || pcg_cta_prepare(h->smem_optin) != cudaSuccess ||
         pcg_tile_prepare(h->smem_optin) != cudaSuccess ||
         form_prepare(h->smem_optin) != cudaSuccess) {
         cudaGetLastError();

@@ -16,8 +16,6 @@ struct SchurArgs {
     unsigned *info;
 };
 
-enum { MODE_REG = 0, MODE_PTR = 1 };
-
 template <typename T>
 struct PcgParams {
     int nx;
@@ -28,7 +26,8 @@ struct PcgParams {
     T *lam;
     const unsigned *info;
     mpcg_stats *stats;
-    int *queue;       // instance counter (nullptr: static round robin)
+    int *queue;       // instance counters, one per group level (nullptr: static round robin)
+    int split;        // pcg_reg_kernel: clusters split into groups for shorter horizons
     const int *inst_list;  // tickets -> instances (nullptr: ticket t is instance t)
     int n_tickets;         // instances to solve (B, or the list's length)
     double tol;
@@ -36,7 +35,7 @@ struct PcgParams {
     int max_iter;     // <= 0: 10 N nx
     int precon;       // 0: symmetric stair Phi^-1 (Pd, Po); 1: block Jacobi (Pd only)
     int kpc_max;      // knot slots per CTA (blockDim.x / LPK)
-    int stage_smem;   // PTR mode: stage blocks in shared memory
+    int stage_smem;   // pcg_cluster_kernel: stage blocks in shared memory
     int vs;           // shared vector stride (elements per knot)
     int depth;        // pcg_tile_kernel: steps each knot stream copies ahead
     const T *Sdp, *Pdp;  // pcg_tile_kernel: packed diagonal blocks (nullptr: full Sd, Pd)
@@ -44,13 +43,16 @@ struct PcgParams {
 };
 
 struct PcgLaunch {
-    int cta_mode;  // 0: cluster per instance; 1: one CTA per instance, blocks from L2
+    int cta_mode;  // 0: cluster per instance (pcg_reg_kernel when reg, else
+                   // pcg_cluster_kernel); 1: one CTA per instance, blocks from L2
                    // (pcg_cta_kernel); 2: one CTA per instance, blocks streamed as
                    // TMA tiles (pcg_tile_kernel)
     int C;         // CTAs per cluster
     int clusters;  // clusters in the grid
     int threads;   // threads per CTA
-    int lpk, rpt, mode, stage, vs, kpc_max;
+    int lpk, rpt, stage, vs, kpc_max;
+    int reg;       // cluster form with register-resident operators (float32, nx = 14)
+    int split;     // reg: one counter per group level, clusters split (see pcg_reg.cu)
     int vw;        // pcg_tile_kernel: elements per shared-memory row load (2 or 4)
     int depth;     // pcg_tile_kernel: steps each knot stream copies ahead (1..4)
     int nxc;       // pcg_tile_kernel: nx fixed at compile time (14, 36), else 0
@@ -94,6 +96,10 @@ __host__ __device__ __forceinline__ int packed_len(int nx) { return (nx * (nx + 
 template <typename T> cudaError_t pcg_launch(const PcgLaunch &, const PcgParams<T> &, cudaStream_t);
 template <typename T> int pcg_max_clusters(const PcgLaunch &);
 cudaError_t pcg_prepare(int smem_optin);
+cudaError_t pcg_reg_launch(const PcgLaunch &, const PcgParams<float> &, cudaStream_t);
+int pcg_reg_max_clusters(const PcgLaunch &);
+size_t pcg_reg_smem_bytes(int kpc_max);
+cudaError_t pcg_reg_prepare();
 cudaError_t pcg_cta_prepare(int smem_optin);
 cudaError_t pcg_tile_prepare(int smem_optin);
 template <typename T>

@@ -7,16 +7,11 @@
 // instance (KPC = ceil(N/C)); inside the CTA, LPK consecutive threads own
 // the rows of one knot, RPT rows per thread (rows li, li+LPK, ...).
 //
-// Data placement (GB300: 256 KB registers + 227 KB shared memory per SM):
-//  * REG mode (float32, nx = 14): each thread keeps its two rows of S+ and
-//    of Phi^-1 (row i of the diagonal block and of both neighbour blocks:
-//    168 floats) in registers for the whole solve; the matrices are read
-//    from global memory once per solve.
-//  * PTR mode (any dtype / nx): the instance's blocks are staged once into
-//    shared memory when they fit, else read from global memory (L2) each
-//    iteration.
-//  * p and r, with one halo knot on each side, live in shared memory; each
-//    thread's rows of lambda, r, p stay in registers.
+// Data placement (GB300: 256 KB registers + 227 KB shared memory per SM): the
+// instance's blocks are staged once into shared memory when they fit, else
+// read from global memory (L2) each iteration; p and r, with one halo knot on
+// each side, live in shared memory; each thread's rows of lambda, r, p stay
+// in registers.  (float32 at nx = 14 has a kernel of its own, pcg_reg.cu.)
 //
 // Communication: two exchanges per iteration, one per reduction of
 // Algorithm 1 (A: p^T S p; B: r^T r~ and ||r||^2).  Each warp reduces its
@@ -29,9 +24,8 @@
 // takes in the pushes of an exchange one after another (measured on GB300:
 // ~6.6 cycles each), and one push per warp (C*W = 128 at N = 512) made the
 // exchange ~1.5x longer.  The same exchanges carry the halo rows the next
-// phase needs (S p of the boundary knots with A, Phi^-1 r with B; in REG
-// mode four 16-byte pushes per side), so Algorithm 2's separate neighbour
-// loads of p and r cost nothing extra: a CTA updates its halo copies of r
+// phase needs (S p of the boundary knots with A, Phi^-1 r with B), so
+// Algorithm 2's separate neighbour loads of p and r cost nothing extra: a CTA updates its halo copies of r
 // and p with the same fused multiply-adds the owner uses (bit-identical).
 // Every CTA adds the C partials in the same butterfly order (the pair
 // additions are commutative), so all CTAs take identical scalar decisions
@@ -94,54 +88,6 @@ struct SmemLayout {
     }
 };
 
-constexpr int NXR = 14;  // REG-mode block size
-
-// Two rows of one block row times the halo'd vector (REG mode): the knot's
-// three 16-float vector slots are read once for both rows.
-__device__ __forceinline__ void rowdot_reg2(const float (&d)[2][NXR], const float (&l)[2][NXR],
-                                            const float (&u)[2][NXR], const float *vprev,
-                                            const float *vself, const float *vnext, float &y0,
-                                            float &y1) {
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, b0 = 0.f, b1 = 0.f, b2 = 0.f;
-    const float4 *s4 = reinterpret_cast<const float4 *>(vself);
-    const float4 *p4 = reinterpret_cast<const float4 *>(vprev);
-    const float4 *n4 = reinterpret_cast<const float4 *>(vnext);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const float4 xs = s4[q], xp = p4[q], xn = n4[q];
-        const float vs_[4] = {xs.x, xs.y, xs.z, xs.w};
-        const float vp_[4] = {xp.x, xp.y, xp.z, xp.w};
-        const float vn_[4] = {xn.x, xn.y, xn.z, xn.w};
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int j = 4 * q + t;
-            if (j < NXR) {
-                a0 = __fmaf_rn(d[0][j], vs_[t], a0);
-                b0 = __fmaf_rn(d[1][j], vs_[t], b0);
-                a1 = __fmaf_rn(l[0][j], vp_[t], a1);
-                b1 = __fmaf_rn(l[1][j], vp_[t], b1);
-                a2 = __fmaf_rn(u[0][j], vn_[t], a2);
-                b2 = __fmaf_rn(u[1][j], vn_[t], b2);
-            }
-        }
-    }
-    y0 = (a0 + a1) + a2;
-    y1 = (b0 + b1) + b2;
-}
-
-__device__ __forceinline__ float resid_reg(float b, const float (&d)[NXR], const float (&l)[NXR],
-                                           const float (&u)[NXR], const float *vprev,
-                                           const float *vself, const float *vnext) {
-    dfloat a{b, 0.f};
-#pragma unroll
-    for (int j = 0; j < NXR; ++j) {
-        a = df_add(a, df_prod(-d[j], vself[j]));
-        a = df_add(a, df_prod(-l[j], vprev[j]));
-        a = df_add(a, df_prod(-u[j], vnext[j]));
-    }
-    return __fadd_rn(a.hi, a.lo);
-}
-
 __device__ __forceinline__ dfloat acc_add_tree(dfloat a, dfloat b) { return df_add_lazy(a, b); }
 __device__ __forceinline__ double acc_add_tree(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ dfloat acc_shfl(dfloat a, int m) {
@@ -187,12 +133,8 @@ __device__ __forceinline__ void st_async_pay(uint32_t addr, const PayB<double> &
     st_async(addr + 8, v.rr, mbar);
 }
 
-// REG mode keeps 168 matrix floats per thread: at most 256 threads per CTA.
-template <int MODE>
-constexpr int pcg_max_threads() { return MODE == MODE_REG ? 256 : 512; }
-
-template <typename T, typename AT, int MODE, int LPK, int RPT>
-__global__ void __launch_bounds__(pcg_max_threads<MODE>(), 1) pcg_cluster_kernel(const PcgParams<T> P) {
+template <typename T, typename AT, int LPK, int RPT>
+__global__ void __launch_bounds__(512, 1) pcg_cluster_kernel(const PcgParams<T> P) {
     using A = typename AT::type;
     using PB = PayB<A>;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -240,9 +182,7 @@ __global__ void __launch_bounds__(pcg_max_threads<MODE>(), 1) pcg_cluster_kernel
     int wpow = 1, cpow = 1;
     while (wpow < W) wpow <<= 1;
     while (cpow < (int)C) cpow <<= 1;
-    // REG mode sends a boundary knot's 16-float slot (14 rows and 2 zeros) as
-    // four 16-byte pushes; PTR mode one push per row
-    const uint32_t side_bytes = MODE == MODE_REG ? 16u * (uint32_t)sizeof(float) : (uint32_t)(nx * sizeof(T));
+    const uint32_t side_bytes = (uint32_t)(nx * sizeof(T));  // one push per row
     const uint32_t halo_bytes = side_bytes * ((has_left ? 1u : 0u) + (has_right ? 1u : 0u));
 
     const uint32_t mbS = smem_u32(&mbar[2]);  // one arrival per peer that has stopped pushing
@@ -295,9 +235,7 @@ __global__ void __launch_bounds__(pcg_max_threads<MODE>(), 1) pcg_cluster_kernel
             rv[m] = active_knot && rows[m] < nx;
         }
 
-        // REG mode: the thread's rows of S+ and Phi^-1 in registers.
-        float sd[2][NXR], sl[2][NXR], su[2][NXR], qd[2][NXR], ql[2][NXR], qu[2][NXR];
-        // PTR mode: block pointers (shared or global).
+        // block pointers (shared or global)
         const T *pSd = nullptr, *pSl = nullptr, *pSu = nullptr;
         const T *pPd = nullptr, *pPl = nullptr, *pPu = nullptr;
         const int nx2 = nx * nx;
@@ -306,29 +244,7 @@ __global__ void __launch_bounds__(pcg_max_threads<MODE>(), 1) pcg_cluster_kernel
         // (precon 1), the even knots' rows for the stair preconditioner (2)
         const bool jac = P.precon == 1 || (P.precon == 2 && (k & 1) == 0);
         if (!bad) {
-            if constexpr (MODE == MODE_REG) {
-                const bool hl = active_knot && k >= 1, hu = active_knot && k + 1 < Nb;
-                const float *Sd = reinterpret_cast<const float *>(P.Sd) + (size_t)(k0 + k) * nx2;
-                const float *Pd = reinterpret_cast<const float *>(P.Pd) + (size_t)(k0 + k) * nx2;
-                const float *SoL = reinterpret_cast<const float *>(P.So) + (size_t)(c0 + k - 1) * nx2;
-                const float *PoL = reinterpret_cast<const float *>(P.Po) + (size_t)(c0 + k - 1) * nx2;
-                const float *SoU = reinterpret_cast<const float *>(P.So) + (size_t)(c0 + k) * nx2;
-                const float *PoU = reinterpret_cast<const float *>(P.Po) + (size_t)(c0 + k) * nx2;
-#pragma unroll
-                for (int m = 0; m < 2; ++m) {
-                    const int i = rows[m];
-                    const bool v = rv[m];
-#pragma unroll
-                    for (int j = 0; j < NXR; ++j) {
-                        sd[m][j] = v ? __ldg(Sd + j * NXR + i) : 0.f;
-                        qd[m][j] = v ? __ldg(Pd + j * NXR + i) : 0.f;
-                        sl[m][j] = (v && hl) ? __ldg(SoL + i * NXR + j) : 0.f;
-                        ql[m][j] = (v && hl && !jac) ? __ldg(PoL + i * NXR + j) : 0.f;
-                        su[m][j] = (v && hu) ? __ldg(SoU + j * NXR + i) : 0.f;
-                        qu[m][j] = (v && hu && !jac) ? __ldg(PoU + j * NXR + i) : 0.f;
-                    }
-                }
-            } else {
+            {
                 if (P.stage_smem) {
                     // own diagonal blocks and the KPC+1 neighbouring off-diagonal blocks
                     T *mSd = mats;
@@ -375,47 +291,15 @@ __global__ void __launch_bounds__(pcg_max_threads<MODE>(), 1) pcg_cluster_kernel
         // y[m] = (row rows[m] of S+ or Phi^-1) . vec (halo'd)
         auto matvec = [&](bool precon, const T *vec, T (&y)[RPT]) {
             const T *vp = vec + kl * vs, *vsf = vec + (kl + 1) * vs, *vn = vec + (kl + 2) * vs;
-            if constexpr (MODE == MODE_REG) {
-                float y0 = 0.f, y1 = 0.f;
-                if (active_knot) {
-                    if (precon) rowdot_reg2(qd, ql, qu, vp, vsf, vn, y0, y1);
-                    else rowdot_reg2(sd, sl, su, vp, vsf, vn, y0, y1);
-                }
-                y[0] = y0;
-                y[1] = y1;
-            } else {
 #pragma unroll
                 for (int m = 0; m < RPT; ++m)
                     y[m] = rv[m] ? (precon ? rowdot_ptr<T>(nx, rows[m], pPd, pPl, pPu, vp, vsf, vn)
                                            : rowdot_ptr<T>(nx, rows[m], pSd, pSl, pSu, vp, vsf, vn))
                                  : T(0);
-            }
         };
 
-        // the warps holding the first and last knot slot (warp-uniform)
-        const bool warp_left = has_left && warp == 0;
-        const bool warp_right = has_right && (int)warp == ((KPC - 1) * LPK) / 32;
         // Push this knot's boundary rows into the neighbours' halo slots.
         auto push_halo = [&](uint32_t h_l, uint32_t m_l, uint32_t h_r, uint32_t m_r, const T (&val)[RPT]) {
-            if constexpr (MODE == MODE_REG) {
-                // Rows 4j..4j+3 gathered into lane j (< 4) of the knot's group:
-                // row i sits in lane i % 8 as val[i / 8]; rows 14, 15 are zero.
-                if (!(warp_left || warp_right)) return;
-                const int base = (int)lane & ~(LPK - 1), j = (int)lane & (LPK - 1);
-                const int src0 = base + (j & 1) * 4;
-                float x[4];
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const float a = __shfl_sync(0xffffffffu, val[0], src0 + t);
-                    const float b = __shfl_sync(0xffffffffu, val[1], src0 + t);
-                    x[t] = (j & 2) ? b : a;
-                }
-                if (j < 4) {
-                    const uint32_t off = 16u * (uint32_t)j;
-                    if (send_left) st_async_v4(h_l + off, x[0], x[1], x[2], x[3], m_l);
-                    if (send_right) st_async_v4(h_r + off, x[0], x[1], x[2], x[3], m_r);
-                }
-            } else {
 #pragma unroll
                 for (int m = 0; m < RPT; ++m) {
                     if (!rx[m]) continue;
@@ -423,7 +307,6 @@ __global__ void __launch_bounds__(pcg_max_threads<MODE>(), 1) pcg_cluster_kernel
                     if (send_left) st_async(h_l + off, val[m], m_l);
                     if (send_right) st_async(h_r + off, val[m], m_r);
                 }
-            }
         };
 
         // Exchange A: cluster sum of one accumulator per thread.  Each warp
@@ -526,10 +409,7 @@ __global__ void __launch_bounds__(pcg_max_threads<MODE>(), 1) pcg_cluster_kernel
                 r_r[m] = T(0);
                 if (rv[m]) {
                     const T *vp = vecP + kl * vs, *vsf = vecP + (kl + 1) * vs, *vn = vecP + (kl + 2) * vs;
-                    if constexpr (MODE == MODE_REG)
-                        r_r[m] = resid_reg(bv[m], sd[m], sl[m], su[m], vp, vsf, vn);
-                    else
-                        r_r[m] = resid_ptr<T>(nx, rows[m], bv[m], pSd, pSl, pSu, vp, vsf, vn);
+                    r_r[m] = resid_ptr<T>(nx, rows[m], bv[m], pSd, pSl, pSu, vp, vsf, vn);
                 }
                 sb = AT::add(sb, AT::prod(bv[m], bv[m]));
                 if (rx[m]) vecR[(kl + 1) * vs + rows[m]] = r_r[m];
@@ -736,13 +616,10 @@ size_t pcg_smem_bytes(int kpc_max, int vs, int C, int W, int nx, int stage, int 
 
 template <typename T, typename AT>
 static void (*pcg_fn_acc(const PcgLaunch &L))(const PcgParams<T>) {
-    if constexpr (sizeof(T) == 4) {
-        if (L.mode == MODE_REG) return pcg_cluster_kernel<float, AT, MODE_REG, 8, 2>;
-    }
-    if (L.lpk == 8) return pcg_cluster_kernel<T, AT, MODE_PTR, 8, 2>;
-    if (L.lpk == 16) return pcg_cluster_kernel<T, AT, MODE_PTR, 16, 1>;
-    if (L.rpt == 1) return pcg_cluster_kernel<T, AT, MODE_PTR, 32, 1>;
-    return pcg_cluster_kernel<T, AT, MODE_PTR, 32, 2>;
+    if (L.lpk == 8) return pcg_cluster_kernel<T, AT, 8, 2>;
+    if (L.lpk == 16) return pcg_cluster_kernel<T, AT, 16, 1>;
+    if (L.rpt == 1) return pcg_cluster_kernel<T, AT, 32, 1>;
+    return pcg_cluster_kernel<T, AT, 32, 2>;
 }
 
 template <typename T>
@@ -794,13 +671,10 @@ static cudaError_t prepare_one(void (*fn)(const PcgParams<T>), int smem_optin) {
 template <typename T, typename AT>
 static cudaError_t prepare_acc(int smem_optin) {
     cudaError_t e;
-    if constexpr (sizeof(T) == 4) {
-        if ((e = prepare_one<T>(pcg_cluster_kernel<T, AT, MODE_REG, 8, 2>, smem_optin))) return e;
-    }
-    if ((e = prepare_one<T>(pcg_cluster_kernel<T, AT, MODE_PTR, 8, 2>, smem_optin))) return e;
-    if ((e = prepare_one<T>(pcg_cluster_kernel<T, AT, MODE_PTR, 16, 1>, smem_optin))) return e;
-    if ((e = prepare_one<T>(pcg_cluster_kernel<T, AT, MODE_PTR, 32, 1>, smem_optin))) return e;
-    return prepare_one<T>(pcg_cluster_kernel<T, AT, MODE_PTR, 32, 2>, smem_optin);
+    if ((e = prepare_one<T>(pcg_cluster_kernel<T, AT, 8, 2>, smem_optin))) return e;
+    if ((e = prepare_one<T>(pcg_cluster_kernel<T, AT, 16, 1>, smem_optin))) return e;
+    if ((e = prepare_one<T>(pcg_cluster_kernel<T, AT, 32, 1>, smem_optin))) return e;
+    return prepare_one<T>(pcg_cluster_kernel<T, AT, 32, 2>, smem_optin);
 }
 
 cudaError_t pcg_prepare(int smem_optin) {
