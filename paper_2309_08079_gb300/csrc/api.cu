@@ -16,6 +16,11 @@ namespace mpcg {
 template <typename T> cudaError_t launch_form_fused(const SchurArgs<T> &, T *Pd, T *Po, int sms,
                                                     cudaStream_t);
 template <typename T> size_t form_fused_smem_bytes(int nx, int nu, int Kgrid, int sms);
+// the same for float32 (14, 7) and (36, 12), tiled (csrc/form_tile.cu)
+bool form_tile_fits(const SchurArgs<float> &, const float *Pd, const float *Po);
+cudaError_t launch_form_tile(const SchurArgs<float> &, float *Pd, float *Po, float *Sdp, float *Pdp, int sms,
+                             cudaStream_t);
+cudaError_t form_tile_prepare(int smem_optin);
 }  // namespace mpcg
 
 using namespace mpcg;
@@ -476,14 +481,7 @@ int precon_t(const mpcg_dims &d, int B, const int *knot_off, mpcg_schur *s, cuda
 template <typename T>
 int form_all_t(mpcg_handle *h, const mpcg_dims &d, int B, const int *knot_off, const mpcg_lq *lq,
                mpcg_schur *s, cudaStream_t st) {
-    // Dense costs, and nx > 16 (one CTA per knot, where repeating D_{k+1}'s
-    // formation and inversion in every CTA costs more than the two launches
-    // it saves): the two separate launches.
     const int Kgrid = knot_off ? B * d.N : d.N;
-    if (lq->Q || d.nx > 16 || form_fused_smem_bytes<T>(d.nx, d.nu, Kgrid, h->sms) > (size_t)h->smem_optin) {
-        int rc = form_schur_t<T>(h, d, B, knot_off, lq, s, st);
-        return rc ? rc : precon_t<T>(d, B, knot_off, s, st);
-    }
     SchurArgs<T> a;
     a.nx = d.nx;
     a.nu = d.nu;
@@ -492,13 +490,32 @@ int form_all_t(mpcg_handle *h, const mpcg_dims &d, int B, const int *knot_off, c
     a.A = (const T *)lq->A; a.B = (const T *)lq->B; a.Qd = (const T *)lq->Qd;
     a.Rd = (const T *)lq->Rd; a.q = (const T *)lq->q; a.r = (const T *)lq->r;
     a.c = (const T *)lq->c;
-    a.Qf = nullptr;
-    a.Rf = nullptr;
+    a.Qf = (const T *)lq->Q;
+    a.Rf = (const T *)lq->R;
     a.Sd = (T *)s->Sd; a.So = (T *)s->So; a.gamma = (T *)s->gamma;
     a.info = s->info;
+    bool tile = false;
+    if constexpr (std::is_same<T, float>::value) tile = form_tile_fits(a, (const T *)s->Pd, (const T *)s->Po);
+    // Dense costs, and nx > 16 outside the tiled shapes (one CTA per knot,
+    // where repeating D_{k+1}'s formation and inversion in every CTA costs
+    // more than the two launches it saves): the two separate launches.
+    if (!tile && (lq->Q || d.nx > 16 || form_fused_smem_bytes<T>(d.nx, d.nu, Kgrid, h->sms) > (size_t)h->smem_optin)) {
+        int rc = form_schur_t<T>(h, d, B, knot_off, lq, s, st);
+        return rc ? rc : precon_t<T>(d, B, knot_off, s, st);
+    }
+    const bool packed = s->Sdp && s->Pdp;
+    if (tile && packed && ((uintptr_t)s->Sdp | (uintptr_t)s->Pdp) % 16 != 0) return MPCG_EINVAL;
     if (s->info) {
         int e = err_cuda(cudaMemsetAsync(s->info, 0, sizeof(unsigned) * B, st));
         if (e) return e;
+    }
+    if constexpr (std::is_same<T, float>::value) {
+        if (tile) {
+            const bool in_kernel = packed && d.nx == 36;
+            const int rc = err_cuda(launch_form_tile(a, (T *)s->Pd, (T *)s->Po, in_kernel ? (T *)s->Sdp : nullptr,
+                                                     in_kernel ? (T *)s->Pdp : nullptr, h->sms, st));
+            return rc || in_kernel ? rc : pack_t<T>(d, B, knot_off, s, st);
+        }
     }
     const int rc = err_cuda(launch_form_fused<T>(a, (T *)s->Pd, (T *)s->Po, h->sms, st));
     return rc ? rc : pack_t<T>(d, B, knot_off, s, st);
@@ -598,7 +615,7 @@ int mpcg_create(mpcg_handle **out) {
     }
     if (pcg_prepare(h->smem_optin) != cudaSuccess || pcg_reg_prepare() != cudaSuccess || pcg_cta_prepare(h->smem_optin) != cudaSuccess ||
         pcg_tile_prepare(h->smem_optin) != cudaSuccess ||
-        form_prepare(h->smem_optin) != cudaSuccess) {
+        form_prepare(h->smem_optin) != cudaSuccess || form_tile_prepare(h->smem_optin) != cudaSuccess) {
         cudaGetLastError();
         delete h;
         return MPCG_ECUDA;

@@ -257,6 +257,57 @@ recover_kernel(int nx, int nu, BatchView bv, const T *__restrict__ A,
     }
 }
 
+// The same for the measured shapes, one thread per output entry: thread
+// (knot, i) of a CTA's KN consecutive knots takes column i of A_k or column
+// i - NX of B_k, so a warp has no idle lanes (21 of 32 were used at nx = 14)
+// and both kinds of column run one instruction stream with every load of a
+// column in flight at once.  Same sums in the same order as recover_kernel.
+template <typename T, int NX, int NU>
+__global__ void __launch_bounds__(256)
+recover_flat_kernel(BatchView bv, const T *__restrict__ A, const T *__restrict__ B, const T *__restrict__ Qd,
+                    const T *__restrict__ Rd, const T *__restrict__ hx, const T *__restrict__ hu,
+                    const T *__restrict__ v, T *__restrict__ zx, T *__restrict__ zu) {
+    constexpr int NC = NX + NU, KN = 256 / NC;
+    __shared__ T vn[KN * NX];
+    __shared__ int own[KN];  // control index of the knot, or -1 - it for an instance's last knot
+    const int kg0 = blockIdx.x * KN, total = bv.total();
+    if (kg0 >= total) return;
+    if ((int)threadIdx.x < KN && kg0 + (int)threadIdx.x < total) {
+        const int kg = kg0 + threadIdx.x, b = bv.owner(kg);
+        int k0, Nb;
+        bv.range(b, k0, Nb);
+        own[threadIdx.x] = kg - k0 + 1 >= Nb ? -1 - (kg - b) : kg - b;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < KN * NX; e += 256)
+        vn[e] = kg0 + e / NX < total && own[e / NX] >= 0 ? v[(size_t)(kg0 + 1) * NX + e] : T(0);
+    __syncthreads();
+    const int kn = threadIdx.x / NC, i = threadIdx.x % NC, kg = kg0 + kn;
+    if (kn >= KN || kg >= total) return;
+    const int j = own[kn];
+    const bool last = j < 0, isx = i < NX;
+    if (last && !isx) return;
+    using AT = Acc<T>;
+    // entry of an x-shaped or u-shaped array, its column and weight
+    const size_t o = isx ? (size_t)kg * NX + i : (size_t)j * NU + (i - NX);
+    const T h = (isx ? hx : hu)[o], w = (isx ? Qd : Rd)[o];
+    typename AT::type s = isx ? AT::add(AT::from(v[o]), AT::from(-h)) : AT::from(-h);
+    if (!last) {
+        const T *col = isx ? A + (size_t)j * NX * NX + i : B + (size_t)j * NX * NU + (i - NX);
+        const int stride = isx ? NX : NU;
+        constexpr int CH = NX <= 16 ? NX : 12;
+#pragma unroll
+        for (int m0 = 0; m0 < NX; m0 += CH) {
+            T x[CH];
+#pragma unroll
+            for (int m = 0; m < CH; ++m) x[m] = __ldg(col + (m0 + m) * stride);
+#pragma unroll
+            for (int m = 0; m < CH; ++m) s = AT::add(s, AT::prod(-x[m], vn[kn * NX + m0 + m]));
+        }
+    }
+    (isx ? zx : zu)[o] = AT::to_T(AT::div_x(s, w));
+}
+
 // ---------------------------------------------------------------------------
 // Backward seed: out = w + C G^-1 (hx, hu), block row k:
 //   k = 0: w_0 + hx_0 / Qd_0
@@ -942,6 +993,14 @@ template <typename T>
 cudaError_t launch_recover(int nx, int nu, BatchView bv, int Kgrid, const T *A, const T *B,
                            const T *Qd, const T *Rd, const T *hx, const T *hu, const T *v, T *zx,
                            T *zu, cudaStream_t s) {
+    if (nx == 14 && nu == 7) {
+        recover_flat_kernel<T, 14, 7><<<ceil_div(Kgrid, 256 / 21), 256, 0, s>>>(bv, A, B, Qd, Rd, hx, hu, v, zx, zu);
+        return cudaGetLastError();
+    }
+    if (nx == 36 && nu == 12) {
+        recover_flat_kernel<T, 36, 12><<<ceil_div(Kgrid, 256 / 48), 256, 0, s>>>(bv, A, B, Qd, Rd, hx, hu, v, zx, zu);
+        return cudaGetLastError();
+    }
     const int groups = FORM_THREADS / group_size(nx);
     recover_kernel<T><<<form_grid(nx, Kgrid), FORM_THREADS, sizeof(T) * nx * groups, s>>>(
         nx, nu, bv, A, B, Qd, Rd, hx, hu, v, zx, zu);
