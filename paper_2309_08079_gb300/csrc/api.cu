@@ -173,7 +173,12 @@ int choose_pcg_tile(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_schur 
 //    still allows it, down to about 8 knots per CTA (fewer warps per CTA
 //    barrier; a single instance of 64 / 128 knots).
 //  - More instances than clusters: full CTAs, a power of two per cluster, and
-//    clusters that split into groups as the long horizons run out.
+//    clusters that split into groups as the long horizons run out.  With two
+//    waves or more at that residency, two CTAs share an SM (Phi^-1 in shared
+//    memory): each iterates 1.84 times slower, and twice as many run, or more
+//    (36 clusters of 8 in place of 15, 14 of 16 in place of 7).  Measured: 256
+//    instances of 32..512 knots 25.3 against 27.5 ms, 150 of 100..250 6.2
+//    against 7.6; but 20 of 300..512, less than two waves, 4.4 against 3.9.
 inline int choose_pcg_reg(const mpcg_dims &d, int B, const mpcg_opts *o, PcgLaunch &L) {
     constexpr int kpc_cap = 32, kpc_small = 8;
     L.cta_mode = 0;
@@ -183,34 +188,35 @@ inline int choose_pcg_reg(const mpcg_dims &d, int B, const mpcg_opts *o, PcgLaun
     L.vs = 16;
     const int C_full = ceil_div(d.N, kpc_cap);
     if (C_full > kMaxCluster) return MPCG_EUNSUPPORTED;
-    auto shape = [&](int C) {  // co-resident clusters of C CTAs (0: cannot run)
+    // co-resident clusters of C CTAs (0: cannot run)
+    auto shape = [&](int C, int reg, int kpc) {
+        L.reg = reg;
         L.C = C;
-        L.kpc_max = ceil_div(d.N, C);
-        if (L.kpc_max > kpc_cap) return 0;
-        L.threads = std::max(32, ceil_div(L.kpc_max * L.lpk, 32) * 32);
-        L.smem = pcg_reg_smem_bytes(L.kpc_max);
+        L.kpc_max = kpc;
+        if (kpc > kpc_cap) return 0;
+        L.threads = std::max(32, ceil_div(kpc * L.lpk, 32) * 32);
+        L.smem = pcg_reg_smem_bytes(L);
         return pcg_reg_max_clusters(L);
     };
     if (o && o->cluster > 0) {
         if (o->cluster > kMaxCluster) return MPCG_EUNSUPPORTED;
-        const int n = shape(std::min(o->cluster, d.N));
+        const int C = std::min(o->cluster, d.N), n = shape(C, 1, ceil_div(d.N, C));
         if (n < 1) return MPCG_EUNSUPPORTED;
         L.clusters = std::min(B, n);
         return MPCG_OK;
     }
-    for (int C = std::min(kMaxCluster, std::max(C_full, ceil_div(d.N, kpc_small))); C >= C_full; --C)
-        if (shape(C) >= B) {
+    const int C_small = std::min(kMaxCluster, std::max(C_full, ceil_div(d.N, kpc_small)));
+    for (int C = C_small; C >= C_full; --C)
+        if (shape(C, 1, ceil_div(d.N, C)) >= B) {
             L.clusters = B;
             return MPCG_OK;
         }
     int C = 1;
     while (C < C_full) C <<= 1;
     for (; C >= C_full && C >= 1; C >>= 1) {
-        L.C = C;
-        L.kpc_max = C > 1 ? kpc_cap : d.N;
-        L.threads = std::max(32, ceil_div(L.kpc_max * L.lpk, 32) * 32);
-        L.smem = pcg_reg_smem_bytes(L.kpc_max);
-        const int n = pcg_reg_max_clusters(L);
+        const int kpc = C > 1 ? kpc_cap : d.N;
+        int n = shape(C, 2, kpc);
+        if (n < 1 || B < 2 * n) n = shape(C, 1, kpc);
         if (n >= 1) {
             L.split = C > 1 && n < B;
             L.clusters = std::min(B, n);
@@ -613,7 +619,7 @@ int mpcg_create(mpcg_handle **out) {
         delete h;
         return MPCG_ECUDA;
     }
-    if (pcg_prepare(h->smem_optin) != cudaSuccess || pcg_reg_prepare() != cudaSuccess || pcg_cta_prepare(h->smem_optin) != cudaSuccess ||
+    if (pcg_prepare(h->smem_optin) != cudaSuccess || pcg_reg_prepare(h->smem_optin) != cudaSuccess || pcg_cta_prepare(h->smem_optin) != cudaSuccess ||
         pcg_tile_prepare(h->smem_optin) != cudaSuccess ||
         form_prepare(h->smem_optin) != cudaSuccess || form_tile_prepare(h->smem_optin) != cudaSuccess) {
         cudaGetLastError();

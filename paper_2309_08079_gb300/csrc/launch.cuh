@@ -51,7 +51,8 @@ struct PcgLaunch {
     int clusters;  // clusters in the grid
     int threads;   // threads per CTA
     int lpk, rpt, stage, vs, kpc_max;
-    int reg;       // cluster form with register-resident operators (float32, nx = 14)
+    int reg;       // cluster form with resident operators (float32, nx = 14): 1 both in
+                   // registers, 2 Phi^-1 in shared memory, two CTAs per SM
     int split;     // reg: one counter per group level, clusters split (see pcg_reg.cu)
     int vw;        // pcg_tile_kernel: elements per shared-memory row load (2 or 4)
     int depth;     // pcg_tile_kernel: steps each knot stream copies ahead (1..4)
@@ -98,8 +99,8 @@ template <typename T> int pcg_max_clusters(const PcgLaunch &);
 cudaError_t pcg_prepare(int smem_optin);
 cudaError_t pcg_reg_launch(const PcgLaunch &, const PcgParams<float> &, cudaStream_t);
 int pcg_reg_max_clusters(const PcgLaunch &);
-size_t pcg_reg_smem_bytes(int kpc_max);
-cudaError_t pcg_reg_prepare();
+size_t pcg_reg_smem_bytes(const PcgLaunch &);
+cudaError_t pcg_reg_prepare(int smem_optin);
 cudaError_t pcg_cta_prepare(int smem_optin);
 cudaError_t pcg_tile_prepare(int smem_optin);
 template <typename T>

@@ -35,13 +35,19 @@
 // Phi^-1 (2 x 84 floats) in registers for the whole solve.  r, p, r~ (with
 // one halo knot on each side) live in shared memory.
 //
+// PS form: with many instances the exchanges of one leave the SM idle two
+// thirds of the time, and one 16-CTA cluster per GPC leaves SMs unused, so two
+// CTAs share an SM: 128 registers a thread hold the rows of S+, the rows of
+// Phi^-1 lie in shared memory (same products in the same order).  The shared-
+// memory reads then bound it: an iteration takes 1.84 times as long.
+//
 // Groups: a launch with more instances than clusters splits its clusters as
 // the long instances run out.  At level l a group of C >> l CTAs takes only
 // instances that need more than half of it at 32 knots per CTA; when that
 // class is exhausted the group splits in two.  A ragged batch then runs its
 // long horizons first, and short ones do not occupy a whole cluster (256
 // instances of 32..512 knots: 42.8 ms with a 16-CTA cluster for each and two
-// reductions, 27.5 ms now).
+// reductions, 27.5 ms split, 25.3 with two CTAs per SM).
 //
 // Exchanges (st.async pushes completing transaction bytes on the receiver's
 // mbarriers, no cluster barrier in the loop): per iteration the boundary rows
@@ -64,12 +70,14 @@ constexpr int VSR = 16;   // floats per knot slot of a shared vector
 constexpr int LPR = 8;    // lanes per knot
 constexpr int CMAX = 16;  // CTAs per cluster
 constexpr int WMAX = 8;   // warps per CTA
+constexpr int PROWS = 3 * 2 * NXR;  // a thread's entries of one operator
 constexpr int LEVELS = 5; // group sizes C, C/2, ..., C/16
 
 // Shared-memory carve-up, in bytes; the same on host and device.
 struct RegLayout {
-    size_t vecR, vecP, vecZ, halo, slot, wpart, mbar, mail, misc, total;
-    __host__ __device__ explicit RegLayout(int kpc_max) {
+    size_t vecR, vecP, vecZ, halo, slot, wpart, mbar, mail, misc, mats, total;
+    // threads > 0: the rows of Phi^-1 of so many threads too
+    __host__ __device__ RegLayout(int kpc_max, int threads) {
         size_t o = 0;
         auto take = [&o](size_t bytes) {
             const size_t at = o;
@@ -86,6 +94,7 @@ struct RegLayout {
         mbar = take(sizeof(uint64_t) * (4 + LEVELS));  // R0, R1, Z, peers stopped, instance mail
         mail = take(sizeof(int) * LEVELS);
         misc = take(16);
+        mats = take(sizeof(float) * (size_t)PROWS * threads);
         total = o;
     }
 };
@@ -120,6 +129,41 @@ __device__ __forceinline__ void rowdot2(const float (&d)[2][NXR], const float (&
     }
     y[0] = (a0 + a1) + a2;
     y[1] = (b0 + b1) + b2;
+}
+
+// The same with the thread's rows in shared memory (PS form): 21 four-entry
+// words per thread, word c of all threads side by side, so a warp's load is
+// conflict-free; per block seven words, the two rows' entries 4 q .. 4 q + 3
+// in turn (the last word: entries 12 and 13 of both).
+__device__ __forceinline__ void rowdot2_ps(const float4 *m, int stride, const float *vprev,
+                                           const float *vself, const float *vnext, float (&y)[2]) {
+    float sum[3][2];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const float4 *v4 = reinterpret_cast<const float4 *>(b == 0 ? vself : b == 1 ? vprev : vnext);
+        const float4 *w = m + (size_t)7 * b * stride;
+        float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const float4 x = v4[q], r0 = w[2 * q * stride], r1 = w[(2 * q + 1) * stride];
+            a0 = __fmaf_rn(r0.x, x.x, a0);
+            a1 = __fmaf_rn(r1.x, x.x, a1);
+            a0 = __fmaf_rn(r0.y, x.y, a0);
+            a1 = __fmaf_rn(r1.y, x.y, a1);
+            a0 = __fmaf_rn(r0.z, x.z, a0);
+            a1 = __fmaf_rn(r1.z, x.z, a1);
+            a0 = __fmaf_rn(r0.w, x.w, a0);
+            a1 = __fmaf_rn(r1.w, x.w, a1);
+        }
+        const float2 x = *reinterpret_cast<const float2 *>(v4 + 3);
+        const float4 r = w[6 * stride];
+        a0 = __fmaf_rn(r.x, x.x, a0);
+        a1 = __fmaf_rn(r.z, x.x, a1);
+        sum[b][0] = __fmaf_rn(r.y, x.y, a0);
+        sum[b][1] = __fmaf_rn(r.w, x.y, a1);
+    }
+    y[0] = (sum[0][0] + sum[1][0]) + sum[2][0];
+    y[1] = (sum[0][1] + sum[1][1]) + sum[2][1];
 }
 
 __device__ __forceinline__ float resid_row(float b, const float (&d)[NXR], const float (&l)[NXR],
@@ -175,8 +219,8 @@ __device__ __forceinline__ bool warp_wait(uint32_t mbar, uint32_t parity, const 
 
 }  // namespace
 
-template <typename AT>
-__global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<float> P) {
+template <typename AT, bool PS>
+__global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const PcgParams<float> P) {
     using A = typename AT::type;
     static_assert(sizeof(A) == 8, "sums travel in pairs of 8 bytes");
     extern __shared__ __align__(16) unsigned char smem[];
@@ -190,7 +234,7 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const int kl = tid / LPR, li = tid % LPR;
 
-    const RegLayout L(P.kpc_max);
+    const RegLayout L(P.kpc_max, PS ? blockDim.x : 0);
     float *vecR = reinterpret_cast<float *>(smem + L.vecR);
     float *vecP = reinterpret_cast<float *>(smem + L.vecP);
     float *vecZ = reinterpret_cast<float *>(smem + L.vecZ);
@@ -315,7 +359,10 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
         const uint32_t nb_mbar = nb + (uint32_t)L.mbar;
 
         // ---- rows of S+ and Phi^-1 into registers -----------------------------
-        float sd[2][NXR], sl[2][NXR], su[2][NXR], qd[2][NXR], ql[2][NXR], qu[2][NXR];
+        float sd[2][NXR], sl[2][NXR], su[2][NXR];
+        constexpr int NQ = PS ? 1 : NXR;
+        float qd[2][NQ], ql[2][NQ], qu[2][NQ];  // (PS: in shared memory)
+        float4 *mq = reinterpret_cast<float4 *>(smem + L.mats) + tid;
         {
             // Phi^-1 rows without off-diagonal blocks: every row for block
             // Jacobi (precon 1), the even knots' rows for the stair (2)
@@ -325,19 +372,40 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
             const float *Sd = P.Sd + (size_t)(k0 + k) * n2, *Pd = P.Pd + (size_t)(k0 + k) * n2;
             const float *SoL = P.So + (ptrdiff_t)(c0 + k - 1) * n2, *PoL = P.Po + (ptrdiff_t)(c0 + k - 1) * n2;
             const float *SoU = P.So + (size_t)(c0 + k) * n2, *PoU = P.Po + (size_t)(c0 + k) * n2;
+            // rows 2 li, 2 li + 1 of a block: down its columns (the diagonal
+            // blocks are symmetric), or along its rows
+            auto rows_of = [&](const float *M, bool on, bool along, auto &out) {
 #pragma unroll
-            for (int m = 0; m < 2; ++m) {
-                const int i = 2 * li + m;
-                const bool v = rv;
+                for (int m = 0; m < 2; ++m)
 #pragma unroll
-                for (int j = 0; j < NXR; ++j) {
-                    sd[m][j] = v ? __ldg(Sd + j * NXR + i) : 0.f;
-                    qd[m][j] = v ? __ldg(Pd + j * NXR + i) : 0.f;
-                    sl[m][j] = (v && hl) ? __ldg(SoL + i * NXR + j) : 0.f;
-                    ql[m][j] = (v && hl && !jac) ? __ldg(PoL + i * NXR + j) : 0.f;
-                    su[m][j] = (v && hu) ? __ldg(SoU + j * NXR + i) : 0.f;
-                    qu[m][j] = (v && hu && !jac) ? __ldg(PoU + j * NXR + i) : 0.f;
-                }
+                    for (int j = 0; j < NXR; ++j) {
+                        const int i = 2 * li + m;
+                        out[m][j] = on && rv ? __ldg(M + (along ? i * NXR + j : j * NXR + i)) : 0.f;
+                    }
+            };
+            rows_of(Sd, true, false, sd);
+            rows_of(SoL, hl, true, sl);
+            rows_of(SoU, hu, false, su);
+            if constexpr (PS) {
+                auto stash = [&](int b, const float (&x)[2][NXR]) {
+#pragma unroll
+                    for (int q = 0; q < 3; ++q)
+#pragma unroll
+                        for (int m = 0; m < 2; ++m)
+                            mq[(7 * b + 2 * q + m) * nthreads] = make_float4(x[m][4 * q], x[m][4 * q + 1], x[m][4 * q + 2], x[m][4 * q + 3]);
+                    mq[(7 * b + 6) * nthreads] = make_float4(x[0][12], x[0][13], x[1][12], x[1][13]);
+                };
+                float x[2][NXR];
+                rows_of(Pd, true, false, x);
+                stash(0, x);
+                rows_of(PoL, hl && !jac, true, x);
+                stash(1, x);
+                rows_of(PoU, hu && !jac, false, x);
+                stash(2, x);
+            } else {
+                rows_of(Pd, true, false, qd);
+                rows_of(PoL, hl && !jac, true, ql);
+                rows_of(PoU, hu && !jac, false, qu);
             }
         }
 
@@ -476,7 +544,8 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
             float z[2] = {0.f, 0.f}, q[2] = {0.f, 0.f}, t[2] = {0.f, 0.f};
             if (active_knot) {
                 const float *vp = vecR + kl * VSR;
-                rowdot2(qd, ql, qu, vp, vp + VSR, vp + 2 * VSR, z);
+                if constexpr (PS) rowdot2_ps(mq, nthreads, vp, vp + VSR, vp + 2 * VSR, z);
+                else rowdot2(qd, ql, qu, vp, vp + VSR, vp + 2 * VSR, z);
             }
             push_halo(0, zpar, 16, z);
             if (st) *reinterpret_cast<float2 *>(vecZ + own) = make_float2(z[0], z[1]);
@@ -626,10 +695,11 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
     cluster_sync_all();  // peers may push into this CTA's shared memory until they leave too
 }
 
-size_t pcg_reg_smem_bytes(int kpc_max) { return RegLayout(kpc_max).total; }
+size_t pcg_reg_smem_bytes(const PcgLaunch &L) { return RegLayout(L.kpc_max, L.reg == 2 ? L.threads : 0).total; }
 
 static void (*reg_fn(const PcgLaunch &L))(const PcgParams<float>) {
-    return L.dot ? pcg_reg_kernel<AccF64> : pcg_reg_kernel<Acc<float>>;
+    if (L.reg == 2) return L.dot ? pcg_reg_kernel<AccF64, true> : pcg_reg_kernel<Acc<float>, true>;
+    return L.dot ? pcg_reg_kernel<AccF64, false> : pcg_reg_kernel<Acc<float>, false>;
 }
 
 static cudaLaunchConfig_t reg_config(const PcgLaunch &L, int clusters, cudaLaunchAttribute *attr, cudaStream_t s) {
@@ -668,10 +738,14 @@ int pcg_reg_max_clusters(const PcgLaunch &L) {
     return n;
 }
 
-cudaError_t pcg_reg_prepare() {
-    cudaError_t e = cudaFuncSetAttribute(pcg_reg_kernel<Acc<float>>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(pcg_reg_kernel<AccF64>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+cudaError_t pcg_reg_prepare(int smem_optin) {
+    for (auto *fn : {pcg_reg_kernel<Acc<float>, false>, pcg_reg_kernel<AccF64, false>, pcg_reg_kernel<Acc<float>, true>,
+                     pcg_reg_kernel<AccF64, true>}) {
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin)) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace mpcg

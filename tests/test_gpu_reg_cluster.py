@@ -63,10 +63,11 @@ def test_direct_sum_when_the_identity_cancels():
     assert oracle.relerr(lam.cpu().double().numpy().ravel(), lo) < 1e-3
 
 
-@pytest.mark.parametrize("B,N_lo,N_hi", [(60, 1, 512), (200, 30, 70), (90, 120, 130)])
+@pytest.mark.parametrize("B,N_lo,N_hi", [(60, 1, 512), (200, 30, 70), (90, 120, 130), (20, 33, 512)])
 def test_more_instances_than_clusters(B, N_lo, N_hi):
     """A queue of instances longer than the co-resident clusters: every group
-    size down to one CTA, and instances at the ends of a class.  Against the
+    size down to one CTA, instances at the ends of a class, with one CTA per
+    SM (20 instances) and two.  Against the
     exact solution of the S+ that was formed: its rounding alone takes the KKT
     solution of a long horizon to the bar."""
     import torch
