@@ -964,6 +964,8 @@ template <typename T>
 cudaError_t launch_recover_dense(int nx, int nu, BatchView bv, int Kgrid, const T *A, const T *B,
                                  const T *Qf, const T *Rf, const T *hx, const T *hu, const T *v,
                                  T *zx, T *zu, cudaStream_t s) {
+    if constexpr (sizeof(T) == 4)
+        if (nx == 14 && nu == 7) return launch_recover_dense_14(bv, Kgrid, A, B, Qf, Rf, hx, hu, v, zx, zu, s);
     const int groups = FORM_THREADS / group_size(nx);
     const size_t smem = sizeof(T) * ((size_t)nx * nx + nu * nu + 2 * nx + nu) * groups;
     recover_dense_kernel<T><<<form_grid(nx, Kgrid), FORM_THREADS, smem, s>>>(

@@ -74,6 +74,10 @@ template <typename T>
 cudaError_t launch_recover_dense(int nx, int nu, BatchView bv, int Kgrid, const T *A, const T *B,
                                  const T *Qf, const T *Rf, const T *hx, const T *hu, const T *v,
                                  T *zx, T *zu, cudaStream_t s);
+// the same for float32 nx = 14, nu = 7 (form_tile.cu)
+cudaError_t launch_recover_dense_14(BatchView bv, int Kgrid, const float *A, const float *B, const float *Qf,
+                                    const float *Rf, const float *hx, const float *hu, const float *v, float *zx,
+                                    float *zu, cudaStream_t s);
 template <typename T>
 cudaError_t launch_cgh(int nx, int nu, BatchView bv, int Kgrid, const T *A, const T *B,
                        const T *Qd, const T *Rd, const T *hx, const T *hu, const T *w, T *out,

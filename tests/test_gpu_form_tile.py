@@ -92,3 +92,45 @@ def test_flat_recovery(nx, nu, Ns, dtype):
         big = np.abs(L[k0:k0 + it.N]).max() * nx
         for got, ref in ((dx[k0:k0 + it.N], x / it.Qd), (du[j0:j0 + it.N - 1], u / it.Rd)):
             assert np.all(np.abs(got - ref) <= eps * np.abs(ref) + 2.0 ** -40 * big / 0.01)
+
+
+@pytest.mark.parametrize("Ns", [[1], [6], [300], [1, 15, 16, 14, 2, 31] * 10])
+def test_dense_costs_equal_the_separate_calls(Ns):
+    """Dense SPD cost blocks at nx = 14: the tiled formation against the two
+    general launches, and the recovery against float64 (bars as above; the
+    inverse cost blocks add their condition to S+'s rounding)."""
+    import torch
+    from paper_2309_08079_gb300.solver import LQTensors
+    s = solver()
+    b = gen.kuka_batch(14, 7, Ns, 7200, dense=True).astype(np.float32)
+    lt = LQTensors.from_batch(b) if len(Ns) > 1 else LQTensors.from_numpy(b.items[0])
+    one, two = s.alloc_schur(lt), s.alloc_schur(lt)
+    s.form(lt, one)
+    s.form_schur(lt, two)
+    s.form_precon(lt, two)
+    K, J = lt.total, lt.total - lt.nb
+    for f, n in (("Sd", K), ("So", J), ("gamma", K), ("Pd", K), ("Po", J)):
+        x, y = getattr(one, f)[:n], getattr(two, f)[:n]
+        assert torch.isfinite(x).all() and _rel(x, y) < 1e-5, (f, _rel(x, y))
+    lam = torch.as_tensor(np.cumsum(np.random.default_rng(5).normal(size=(K, 14)), 0), dtype=torch.float32, device="cuda")
+    dx, du = (x.cpu().double().numpy() for x in s.recover_step(lt, lam))
+    L = lam.cpu().double().numpy()
+    for i, it in enumerate(b.items):
+        it = it.astype(np.float64)
+        k0, j0 = b.knot_off[i], b.knot_off[i] - i
+        x, u = L[k0:k0 + it.N] - it.q, -it.r
+        x[:-1] -= np.einsum("kij,ki->kj", it.A, L[k0 + 1:k0 + it.N])
+        u = u - np.einsum("kij,ki->kj", it.B, L[k0 + 1:k0 + it.N])
+        for got, M, rhs in ((dx[k0:k0 + it.N], it.Q, x), (du[j0:j0 + it.N - 1], it.R, u)):
+            ref = np.linalg.solve(M, rhs[..., None])[..., 0]
+            assert np.linalg.norm(got - ref) <= 1e-5 * np.linalg.norm(ref)
+
+
+def test_dense_block_that_is_not_spd_is_flagged():
+    from paper_2309_08079_gb300.solver import LQTensors
+    s = solver()
+    items = [gen.kuka_lq(14, 7, n, 50 + n, dense=True) for n in (5, 20, 9)]
+    items[1].R[7] = -items[1].R[7]
+    items[2].Q[8] = np.nan
+    lt = LQTensors.from_batch(gen.concat_batch(items).astype(np.float32))
+    assert s.form(lt, s.alloc_schur(lt)).info.tolist() == [0, 1, 1]
