@@ -16,7 +16,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libmpcg.so")
-UNITS = ("api", "form", "form_tile", "pcg", "pcg_reg", "pcg_cta", "nmpc", "diag")
+UNITS = ("api", "form", "form_tile", "pcg", "pcg_reg", "pcg_split", "pcg_cta", "nmpc", "diag")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-I", os.path.join(ROOT, "include")]

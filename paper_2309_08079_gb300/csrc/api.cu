@@ -238,6 +238,23 @@ int choose_pcg_cluster(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opt
     const int nx = d.nx;
     if (wide && nx > 16) return MPCG_EUNSUPPORTED;
     if (!wide && std::is_same<T, float>::value && nx == 14) return choose_pcg_reg(d, B, o, L);
+    // float32 nx = 36 and float64 nx = 14 while the operators stay on chip and
+    // every instance has its own cluster (pcg_split.cu), as many CTAs as that
+    // leaves (the products of a CTA shrink with its knots: N = 64 1.90 us per
+    // iteration at 4 knots per CTA, N = 128 2.94 at 8); float64 accumulation of float32 sums stays with the general form
+    if (!wide && !L.dot) {
+        const int fixed = o && o->cluster > 0 ? std::min(o->cluster, d.N) : 0;
+        for (int C = fixed ? fixed : std::min(kMaxCluster, d.N); C >= (fixed ? fixed : 1) && C <= kMaxCluster; --C) {
+            PcgLaunch Ls{};
+            const int n = pcg_split_shape<T>(nx, d.N, C, Ls);
+            if (n < 1 && !fixed && Ls.C == 0) break;  // not its shape at this many knots per CTA, nor below
+            if (n >= B || (fixed && n >= 1)) {
+                L = Ls;
+                L.clusters = std::min(B, n);
+                return MPCG_OK;
+            }
+        }
+    }
     if (wide) { L.lpk = 8; L.rpt = 2; }
     else if (nx <= 16) { L.lpk = 16; L.rpt = 1; }
     else if (nx <= 32) { L.lpk = 32; L.rpt = 1; }
@@ -406,6 +423,7 @@ int pcg_t(mpcg_handle *h, const mpcg_dims &d, int B, const int *knot_off, const 
     if constexpr (std::is_same<T, float>::value) {
         if (L.reg) return err_cuda(pcg_reg_launch(L, P, st));
     }
+    if (L.split_rows) return err_cuda(pcg_split_launch<T>(L, P, st));
     return err_cuda(pcg_launch<T>(L, P, st));
 }
 
@@ -619,7 +637,8 @@ int mpcg_create(mpcg_handle **out) {
         delete h;
         return MPCG_ECUDA;
     }
-    if (pcg_prepare(h->smem_optin) != cudaSuccess || pcg_reg_prepare(h->smem_optin) != cudaSuccess || pcg_cta_prepare(h->smem_optin) != cudaSuccess ||
+    if (pcg_prepare(h->smem_optin) != cudaSuccess || pcg_reg_prepare(h->smem_optin) != cudaSuccess ||
+        pcg_split_prepare(h->smem_optin) != cudaSuccess || pcg_cta_prepare(h->smem_optin) != cudaSuccess ||
         pcg_tile_prepare(h->smem_optin) != cudaSuccess ||
         form_prepare(h->smem_optin) != cudaSuccess || form_tile_prepare(h->smem_optin) != cudaSuccess) {
         cudaGetLastError();

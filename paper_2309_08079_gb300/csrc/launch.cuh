@@ -53,6 +53,7 @@ struct PcgLaunch {
     int lpk, rpt, stage, vs, kpc_max;
     int reg;       // cluster form with resident operators (float32, nx = 14): 1 both in
                    // registers, 2 Phi^-1 in shared memory, two CTAs per SM
+    int split_rows; // cluster form with rows split over lanes (pcg_split.cu): its variant, 0 none
     int split;     // reg: one counter per group level, clusters split (see pcg_reg.cu)
     int vw;        // pcg_tile_kernel: elements per shared-memory row load (2 or 4)
     int depth;     // pcg_tile_kernel: steps each knot stream copies ahead (1..4)
@@ -105,6 +106,10 @@ cudaError_t pcg_reg_launch(const PcgLaunch &, const PcgParams<float> &, cudaStre
 int pcg_reg_max_clusters(const PcgLaunch &);
 size_t pcg_reg_smem_bytes(const PcgLaunch &);
 cudaError_t pcg_reg_prepare(int smem_optin);
+// sets L to pcg_split.cu's shape for C CTAs; co-resident clusters (0: not its shape)
+template <typename T> int pcg_split_shape(int nx, int N, int C, PcgLaunch &L);
+template <typename T> cudaError_t pcg_split_launch(const PcgLaunch &, const PcgParams<T> &, cudaStream_t);
+cudaError_t pcg_split_prepare(int smem_optin);
 cudaError_t pcg_cta_prepare(int smem_optin);
 cudaError_t pcg_tile_prepare(int smem_optin);
 template <typename T>

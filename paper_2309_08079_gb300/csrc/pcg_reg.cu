@@ -59,7 +59,7 @@
 // halo copies of r and p are updated with the owner's own multiply-adds.
 #include <type_traits>
 
-#include "pcg_rows.cuh"
+#include "pcg_sums.cuh"
 
 namespace mpcg {
 
@@ -177,44 +177,6 @@ __device__ __forceinline__ float resid_row(float b, const float (&d)[NXR], const
         a = df_add(a, df_prod(-u[j], vnext[j]));
     }
     return __fadd_rn(a.hi, a.lo);
-}
-
-// ||r||^2 term in the accumulator's precision (the exit test alone uses it)
-__device__ __forceinline__ dfloat sq_sum(float a, float b, dfloat) { return dfloat{__fmaf_rn(b, b, __fmul_rn(a, a)), 0.f}; }
-__device__ __forceinline__ double sq_sum(float a, float b, double) {
-    return __fma_rn((double)b, (double)b, __dmul_rn((double)a, (double)a));
-}
-
-__device__ __forceinline__ dfloat bcast(dfloat a, int lane) {
-    return dfloat{__shfl_sync(0xffffffffu, a.hi, lane), __shfl_sync(0xffffffffu, a.lo, lane)};
-}
-__device__ __forceinline__ double bcast(double a, int lane) { return __shfl_sync(0xffffffffu, a, lane); }
-
-// two accumulators as one 16-byte push
-__device__ __forceinline__ void push_pair(uint32_t addr, dfloat a, dfloat b, uint32_t mbar) {
-    st_async_v4(addr, a.hi, a.lo, b.hi, b.lo, mbar);
-}
-__device__ __forceinline__ void push_pair(uint32_t addr, double a, double b, uint32_t mbar) {
-    st_async_v4(addr, __int_as_float(__double2loint(a)), __int_as_float(__double2hiint(a)),
-                __int_as_float(__double2loint(b)), __int_as_float(__double2hiint(b)), mbar);
-}
-
-__device__ __forceinline__ void load_pair(const dfloat *p, dfloat &a, dfloat &b) {
-    const float4 v = *reinterpret_cast<const float4 *>(p);
-    a = dfloat{v.x, v.y};
-    b = dfloat{v.z, v.w};
-}
-__device__ __forceinline__ void load_pair(const double *p, double &a, double &b) {
-    const double2 v = *reinterpret_cast<const double2 *>(p);
-    a = v.x;
-    b = v.y;
-}
-
-// Every lane of a warp waits (bounded) for the phase of `parity`; true in all
-// lanes if any of them gave up.
-__device__ __forceinline__ bool warp_wait(uint32_t mbar, uint32_t parity, const volatile int *abort_flag) {
-    const bool ok = mbar_wait_bounded_abort(mbar, parity, WAIT_LIMIT_NS, abort_flag);
-    return __any_sync(0xffffffffu, !ok) != 0;
 }
 
 }  // namespace
@@ -539,7 +501,7 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
         int it = 0;
         for (;; ++it) {
             // ---- r~ = Phi^-1 r, boundary rows to the neighbours -----------------
-            const uint32_t zpar = xz & 1u, rpar = xr & 1u;
+            const uint32_t zpar = xz & 1u, rpar = xr & 1u;  // halo rows alternate once per iteration
             const int failed = *s_fail;  // before the barrier: as every warp saw it
             float z[2] = {0.f, 0.f}, q[2] = {0.f, 0.f}, t[2] = {0.f, 0.f};
             if (active_knot) {
@@ -556,7 +518,7 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
                 const float *vp = vecP + kl * VSR;
                 rowdot2(sd, sl, su, vp, vp + VSR, vp + 2 * VSR, t);
             }
-            push_halo(2, rpar, 8 * rpar, t);
+            push_halo(2, zpar, 8 * rpar, t);
             const A s_eta = AT::add(AT::prod(r[0], z[0]), AT::prod(r[1], z[1]));
             const A s_rr = sq_sum(r[0], r[1], A{});
             const A s_eps = AT::add(AT::prod(z[0], s[0]), AT::prod(z[1], s[1]));
@@ -574,7 +536,7 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
                 rowdot2(sd, sl, su, kl == 0 && has_left ? halo + halo_off(0, zpar, 0) : vp, vp + VSR,
                         kl == KPC - 1 && has_right ? halo + halo_off(0, zpar, 1) : vp + 2 * VSR, q);
             }
-            push_halo(1, rpar, 8 * rpar, q);
+            push_halo(1, zpar, 8 * rpar, q);
             // the boundary lanes' halo operands are loaded before alpha and beta are formed
             float2 hz, hq, ht, hp, hr;
             hz = hq = ht = hp = hr = make_float2(0.f, 0.f);
@@ -586,8 +548,8 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
             }
             const Sums S = exchange(s_eta, s_rr, AT::add(AT::prod(z[0], q[0]), AT::prod(z[1], q[1])), s_eps);
             if (hany) {
-                hq = *reinterpret_cast<const float2 *>(hsrc + halo_off(1, rpar, 0));
-                ht = *reinterpret_cast<const float2 *>(hsrc + halo_off(2, rpar, 0));
+                hq = *reinterpret_cast<const float2 *>(hsrc + halo_off(1, zpar, 0));
+                ht = *reinterpret_cast<const float2 *>(hsrc + halo_off(2, zpar, 0));
             }
             eta = S.eta;
             rr = S.rr;
@@ -627,7 +589,7 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
                     const float *h = halo + halo_off(0, 0, 1) + 2 * li;
                     for (int m = 0; m < 2; ++m) {
                         float *vr = vecR + 2 * VSR + 2 * li + m, *vp = vecP + 2 * VSR + 2 * li + m;
-                        *vr = fma_rn(-alpha, fma_rn(beta, h[halo_off(2, rpar, 0) + m], h[halo_off(1, rpar, 0) + m]), *vr);
+                        *vr = fma_rn(-alpha, fma_rn(beta, h[halo_off(2, zpar, 0) + m], h[halo_off(1, zpar, 0) + m]), *vr);
                         *vp = fma_rn(beta, *vp, h[halo_off(0, zpar, 0) + m]);
                     }
                 }
