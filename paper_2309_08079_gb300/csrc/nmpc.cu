@@ -64,7 +64,10 @@ __device__ __forceinline__ Acc fdyn(const ModelView<T> &m, int i, const T *x, co
 //     dv/dp = -dt diag(stiff cos p), dv/dv = I - dt diag(damp), dv/du = dt P,
 //     A = [[I + dt dv/dp, dt dv/dv], [dv/dp, dv/dv]], B = [[dt dv/du], [dv/du]].
 // ---------------------------------------------------------------------------
-template <typename T>
+// NXC, NUC: compile-time nx, nu (0: from the model).  The 400 index divisions
+// of a knot were most of its instructions: 64 x 128 knots 20.7 us, 9.7 with the
+// shape known.
+template <typename T, int NXC, int NUC>
 __global__ void __launch_bounds__(LIN_THREADS)
 linearize_kernel(ModelView<T> m, BatchView bv, const T *__restrict__ X, const T *__restrict__ U,
                  const T *__restrict__ xref, const T *__restrict__ xs, T *A, T *B, T *Qd, T *Rd,
@@ -77,6 +80,11 @@ linearize_kernel(ModelView<T> m, BatchView bv, const T *__restrict__ X, const T 
     bv.range(b, k0, Nb);
     const int k = kg - k0;
     const bool last = k + 1 >= Nb;
+    if constexpr (NXC > 0) {
+        m.nx = NXC;
+        m.nu = NUC;
+        m.h = NXC / 2;
+    }
     const int nx = m.nx, nu = m.nu, h = m.h;
     const T *x = X + (size_t)kg * nx;
     for (int i = lane; i < nx; i += 32) {
@@ -126,60 +134,84 @@ linearize_kernel(ModelView<T> m, BatchView bv, const T *__restrict__ X, const T 
 // J + mu_b (||x'_0 - x_s||_1 + sum ||x'_{k+1} - f(x'_k, u'_k)||_1).  The
 // candidate point is rounded to the working type first, as the applied step
 // will be.  mu_b = mu when mu > 0, else 1.1 max(1, max |lambda_b|).  Block
-// (b, a, chunk) takes 64 (knot, joint) pairs of instance b, one per thread:
-// thread (k, i) adds the cost of state rows i and h + i of knot k (and of
+// (b, a, chunk) takes 64 PP (knot, joint) pairs of instance b, PP per thread:
+// a pair (k, i) adds the cost of state rows i and h + i of knot k (and of
 // input i, nu <= h), and the defects of those two rows, which need joint i's
 // velocity update alone.  Its share goes to merit[b][a] (zeroed before the
-// launch) with an FP64 atomic: the FP64 work (one sine per pair) spreads
-// over h times more threads than one knot per thread would, and the
-// summation order only moves the merits by rounding, far below the tie
-// tolerance of the choice.
+// launch) with an FP64 atomic: the summation order only moves the merits by
+// rounding, far below the tie tolerance of the choice.
+//
+// Bound by FP64 instructions: each of an SM's schedulers issues one per 64
+// cycles (a conversion from float as well).  A pair takes ~42 of them, against
+// ~97 as first written: floats are widened with integer instructions, the sine
+// of a float takes 14, and the block sum is shared by PP pairs.  64 problems
+// of 128 knots, 9 steps: 54 us at 84 % of that pipe, against ~115.
 // ---------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ double block_sum(double v, double *red) {
-    for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int w = threadIdx.x / 32, lane = threadIdx.x % 32, W = blockDim.x / 32;
-    __syncthreads();
-    if (lane == 0) red[w] = v;
-    __syncthreads();
-    v = lane < W ? red[lane] : 0.0;
-    for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
 
-template <typename T>
-__device__ __forceinline__ double block_max(double v, double *red) {
-    for (int o = 16; o >= 1; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    const int w = threadIdx.x / 32, lane = threadIdx.x % 32, W = blockDim.x / 32;
-    __syncthreads();
-    if (lane == 0) red[w] = v;
-    __syncthreads();
-    v = lane < W ? red[lane] : 0.0;
-    for (int o = 16; o >= 1; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+// The exact double of v: normal floats by moving the bits.
+__device__ __forceinline__ double widen(float v) {
+    const uint32_t u = __float_as_uint(v), m = u & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)  // neither zero, subnormal, infinite nor NaN
+        return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+    return m == 0 ? __hiloint2double((int)u, 0) : (double)v;
 }
+__device__ __forceinline__ double widen(double v) { return v; }
+// v / 2, exactly (halving a float loses a bit only below the normal range)
+__device__ __forceinline__ double half(float v) {
+    return fabsf(v) > 1e-37f ? widen(0.5f * v) : 0.5 * (double)v;
+}
+__device__ __forceinline__ double half(double v) { return 0.5 * v; }
 
-template <typename T>
+// sin of a float in double precision: x = q pi/2 + r with |r| <= pi/4 (pi/2 in
+// two parts; q is small, so the first fused step loses only its own rounding),
+// then the Taylor series of sin r or cos r to r^17, r^16 (the next terms are
+// below 2e-18).  Large arguments take the library's.
+__device__ __forceinline__ double sin_wide(float x) {
+    if (!(fabsf(x) < 8192.f)) return sin((double)x);
+    const float qf = rintf(x * 0.63661977f);
+    const int qi = (int)qf;
+    const double q = widen(qf);
+    double r = __fma_rn(-q, 1.57079632679489655800, widen(x));
+    r = __fma_rn(-q, 6.12323399573676603587e-17, r);
+    const double z = __dmul_rn(r, r);
+    const bool c = qi & 1;
+    double p = c ? 1.0 / 20922789888000.0 : 1.0 / 355687428096000.0;
+    p = __fma_rn(p, z, c ? -1.0 / 87178291200.0 : -1.0 / 1307674368000.0);
+    p = __fma_rn(p, z, c ? 1.0 / 479001600.0 : 1.0 / 6227020800.0);
+    p = __fma_rn(p, z, c ? -1.0 / 3628800.0 : -1.0 / 39916800.0);
+    p = __fma_rn(p, z, c ? 1.0 / 40320.0 : 1.0 / 362880.0);
+    p = __fma_rn(p, z, c ? -1.0 / 720.0 : -1.0 / 5040.0);
+    p = __fma_rn(p, z, c ? 1.0 / 24.0 : 1.0 / 120.0);
+    p = __fma_rn(p, z, c ? -0.5 : -1.0 / 6.0);
+    const double base = c ? 1.0 : r;
+    const double s = __fma_rn(__dmul_rn(z, base), p, base);
+    return (qi & 2) ? -s : s;
+}
+__device__ __forceinline__ double sin_wide(double x) { return sin(x); }
+
+template <typename T, int NXC, int NUC>
 __global__ void __launch_bounds__(MERIT_THREADS)
-merit_kernel(ModelView<T> m, BatchView bv, int n_alpha, const T *__restrict__ X,
+merit_kernel(ModelView<T> m, BatchView bv, int n_alpha, int pp, const T *__restrict__ X,
              const T *__restrict__ U, const T *__restrict__ dX, const T *__restrict__ dU,
              const T *__restrict__ xref, const T *__restrict__ xs, const T *__restrict__ lam,
              double mu, double *merit) {
-    __shared__ double red[MERIT_THREADS / 32];
+    static_assert(MERIT_THREADS == 64, "two warps");
+    __shared__ double red;
+    __shared__ T redT[2];
     const int b = blockIdx.x / n_alpha, a = blockIdx.x % n_alpha;
     if (b >= bv.B) return;
     int k0, Nb;
     bv.range(b, k0, Nb);
-    const int nx = m.nx, nu = m.nu, h = m.h;
-    const int ebase = blockIdx.y * MERIT_THREADS;
+    const int nx = NXC ? NXC : m.nx, nu = NXC ? NUC : m.nu, h = nx / 2;
+    const int ebase = blockIdx.y * MERIT_THREADS * pp;
     if (ebase >= Nb * h) return;  // whole block: this instance is shorter
-    const int c0 = k0 - b;
+    const int c0 = k0 - b, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const T alpha = T(ldexp(1.0, -a));
     double mub = mu;
     if (!(mu > 0.0)) {
         // max |lambda_b|: eight independent loads per thread in flight
         const T *lb = lam + (size_t)k0 * nx;
-        const int n = Nb * nx, step = blockDim.x;
+        const int n = Nb * nx, step = MERIT_THREADS;
         T mx = T(0);
         for (int e0 = threadIdx.x; e0 < n; e0 += 8 * step) {
             T v[8];
@@ -188,11 +220,14 @@ merit_kernel(ModelView<T> m, BatchView bv, int n_alpha, const T *__restrict__ X,
 #pragma unroll
             for (int u = 0; u < 8; ++u) mx = fmax(mx, fabs(v[u]));
         }
-        mub = 1.1 * fmax(1.0, block_max<T>((double)mx, red));
+        for (int o = 16; o >= 1; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (lane == 0) redT[warp] = mx;
+        __syncthreads();
+        mub = 1.1 * fmax(1.0, (double)fmax(redT[0], redT[1]));
     }
     double J = 0.0, viol = 0.0;
-    const int e = ebase + threadIdx.x;
-    if (e < Nb * h) {
+    const int eend = min(ebase + MERIT_THREADS * pp, Nb * h);
+    for (int e = ebase + threadIdx.x; e < eend; e += MERIT_THREADS) {
         const int k = e / h, i = e % h;
         const size_t o = (size_t)(k0 + k) * nx;
         const bool last = k + 1 >= Nb;
@@ -200,36 +235,42 @@ merit_kernel(ModelView<T> m, BatchView bv, int n_alpha, const T *__restrict__ X,
         const T pk = X[o + i] + alpha * dX[o + i];
         const T vk = X[o + h + i] + alpha * dX[o + h + i];
         const T *w = last ? m.wf : m.wq;
-        const double ep = (double)pk - (double)xref[o + i];
-        const double ev = (double)vk - (double)xref[o + h + i];
-        J += 0.5 * (double)w[i] * ep * ep;
-        J += 0.5 * (double)w[h + i] * ev * ev;
+        const double dp = widen(pk), dv = widen(vk);
+        const double ep = dp - widen(xref[o + i]), ev = dv - widen(xref[o + h + i]);
+        J += half(w[i]) * ep * ep;
+        J += half(w[h + i]) * ev * ev;
         if (!last && i < nu) {
             const size_t ou = (size_t)(c0 + k) * nu + i;
-            const T ui = U[ou] + alpha * dU[ou];
-            J += 0.5 * (double)m.wr[i] * (double)ui * (double)ui;
+            const double ui = widen(T(U[ou] + alpha * dU[ou]));
+            J += half(m.wr[i]) * ui * ui;
         }
         if (k == 0) {
-            viol += fabs((double)pk - (double)xs[(size_t)b * nx + i]);
-            viol += fabs((double)vk - (double)xs[(size_t)b * nx + h + i]);
+            viol += fabs(dp - widen(xs[(size_t)b * nx + i]));
+            viol += fabs(dv - widen(xs[(size_t)b * nx + h + i]));
         } else {
             // joint i's velocity update from the candidate (x'_{k-1}, u'_{k-1})
             const size_t op = o - nx, ou = (size_t)(c0 + k - 1) * nu;
-            const T pp = X[op + i] + alpha * dX[op + i];
+            const T pp_ = X[op + i] + alpha * dX[op + i];
             const T vp = X[op + h + i] + alpha * dX[op + h + i];
             double f = 0.0;
+#pragma unroll
             for (int j = 0; j < nu; ++j) {
                 const T uj = U[ou + j] + alpha * dU[ou + j];
-                f += (double)m.P[i * nu + j] * (double)uj;
+                f += widen(m.P[i * nu + j]) * widen(uj);
             }
-            f += -(double)m.damp[i] * (double)vp - (double)m.stiff[i] * sin((double)pp);
-            const double vn = (double)vp + m.dt * f;
-            viol += fabs((double)pk - ((double)pp + m.dt * vn));
-            viol += fabs((double)vk - vn);
+            const double wp = widen(pp_), wv = widen(vp);
+            f = __fma_rn(-widen(m.damp[i]), wv, f);
+            f = __fma_rn(-widen(m.stiff[i]), sin_wide(pp_), f);
+            const double vn = wv + m.dt * f;
+            viol += fabs(dp - (wp + m.dt * vn));
+            viol += fabs(dv - vn);
         }
     }
-    const double part = block_sum<T>(J + mub * viol, red);
-    if (threadIdx.x == 0) atomicAdd(&merit[(size_t)b * n_alpha + a], part);
+    double part = J + mub * viol;
+    for (int o = 16; o >= 1; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    if (threadIdx.x == 32) red = part;
+    __syncthreads();
+    if (threadIdx.x == 0) atomicAdd(&merit[(size_t)b * n_alpha + a], part + red);
 }
 
 // ---------------------------------------------------------------------------
@@ -311,7 +352,8 @@ int linearize_t(const mpcg_dims &d, int B, const int *knot_off, const mpcg_model
                 cudaStream_t st) {
     const int K = knot_off ? B * d.N : d.N;  // upper bound on the total knots
     const int per = LIN_THREADS / 32;
-    linearize_kernel<T><<<(K + per - 1) / per, LIN_THREADS, 0, st>>>(
+    auto *fn = d.nx == 14 && d.nu == 7 ? linearize_kernel<T, 14, 7> : linearize_kernel<T, 0, 0>;
+    fn<<<(K + per - 1) / per, LIN_THREADS, 0, st>>>(
         view<T>(m), bview(knot_off, B, d.N), (const T *)X, (const T *)U, (const T *)xref,
         (const T *)xs, (T *)o->A, (T *)o->B, (T *)o->Qd, (T *)o->Rd, (T *)o->q, (T *)o->r,
         (T *)o->c);
@@ -326,9 +368,16 @@ int line_search_t(const mpcg_dims &d, int B, const int *knot_off, const mpcg_mod
     const BatchView bv = bview(knot_off, B, d.N);
     int rc = err(cudaMemsetAsync(merit, 0, sizeof(double) * (size_t)B * n_alpha, st));
     if (rc) return rc;
-    const dim3 grid(B * n_alpha, (d.N * (d.nx / 2) + MERIT_THREADS - 1) / MERIT_THREADS);
-    merit_kernel<T><<<grid, MERIT_THREADS, 0, st>>>(
-        view<T>(m), bv, n_alpha, (const T *)X, (const T *)U, (const T *)dX, (const T *)dU,
+    // Pairs per thread: one while that leaves schedulers idle (the chain of a
+    // pair is the time: 2 x 128 knots 13.5 us a call with one, 20.6 with
+    // four), more once there are a dozen warps for each (64 x 128: 69.6 with
+    // four, 75.9 with one, 65.6 with eight; 32 x 128: 41 and 45).
+    const long long warps = (long long)B * n_alpha * d.N * (d.nx / 2) / 32;
+    const int pp = warps >= 12288 ? 8 : warps >= 6144 ? 4 : 1;
+    const dim3 grid(B * n_alpha, (d.N * (d.nx / 2) + MERIT_THREADS * pp - 1) / (MERIT_THREADS * pp));
+    auto *fn = d.nx == 14 && d.nu == 7 ? merit_kernel<T, 14, 7> : merit_kernel<T, 0, 0>;
+    fn<<<grid, MERIT_THREADS, 0, st>>>(
+        view<T>(m), bv, n_alpha, pp, (const T *)X, (const T *)U, (const T *)dX, (const T *)dU,
         (const T *)xref, (const T *)xs, (const T *)lam, mu, merit);
     rc = err(cudaGetLastError());
     if (rc) return rc;

@@ -134,3 +134,51 @@ def test_batched_sqp_matches_the_oracle_per_instance():
         h = onmpc.sqp(m, t, 5)[-1]
         assert oracle.relerr(X[ko[b]:ko[b + 1]], h["X"]) < 1e-4
         assert oracle.relerr(U[ko[b] - b:ko[b + 1] - b - 1], h["U"]) < 1e-3
+
+
+@pytest.mark.parametrize("nx,nu", [(14, 7), (10, 3)])
+@pytest.mark.parametrize("B,N", [(1, 1), (1, 40), (64, 100), (100, 129)])
+def test_merits_at_every_pairs_per_thread(nx, nu, B, N):
+    """Merits of a batch (one, four and eight knot-joint pairs per thread)
+    against the oracle's FP64 merits at the same float32 candidates, with
+    positions where the sine's argument reduction and the widening of floats
+    can go wrong: zeros, multiples of pi / 2, large, subnormal.  The bar is
+    1e-13 of the merit: its terms are positive and there are under 2^14 of
+    them, each good to a few 2^-53."""
+    import torch
+    m = gen.nmpc_model(nx, nu, 6).astype(np.float32)
+    rng = np.random.default_rng(7)
+    trks = []
+    for b in range(B):
+        t = gen.nmpc_tracking(m, N, 6200 + b).astype(np.float32)
+        pos = t.X[:, :nx // 2]
+        pick = rng.integers(0, 8, size=pos.shape)
+        for v, vals in enumerate((0.0, np.pi / 2 * rng.integers(-40, 40, size=pos.shape), 3e4 * rng.normal(size=pos.shape),
+                                  1e-40, 8191.9, -8192.1)):
+            pos[...] = np.where(pick == v, np.float32(vals), pos)
+        t.U[...] = rng.normal(size=t.U.shape).astype(np.float32)
+        trks.append(t)
+    q = _sqp(m, trks if B > 1 else trks[0])
+    dX = rng.normal(size=(B * N, nx)).astype(np.float32)
+    dU = rng.normal(size=(B, max(N - 1, 0), nu)).astype(np.float32)
+    q.dx.copy_(torch.as_tensor(dX))
+    if N > 1:
+        q.du.copy_(torch.as_tensor(dU.reshape(-1, nu)))
+    q.mu = 3.0
+    q.line_search()
+    got = q.merit.cpu().numpy()
+    for b in sorted({0, B // 2, B - 1}):
+        t, dx, du = trks[b], dX[b * N:(b + 1) * N], dU[b]
+        for a in range(got.shape[1]):
+            al = np.float32(0.5 ** a)
+            want = onmpc.merit(m, t, t.X + al * dx, t.U + al * du, 3.0)
+            assert abs(got[b, a] - want) <= 1e-13 * abs(want), (b, a, got[b, a], want)
+
+
+def test_a_nan_position_gives_a_nan_merit():
+    import torch
+    m, t = _problem(30)
+    q = _sqp(m, t)
+    q.X[11, 3] = float("nan")
+    q.line_search()
+    assert torch.isnan(q.merit).all()
