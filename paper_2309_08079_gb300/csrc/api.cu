@@ -96,7 +96,7 @@ int choose_pcg_cta(mpcg_handle *h, const mpcg_dims &d, int B, PcgLaunch &L) {
     return MPCG_OK;
 }
 
-// Launch shape of the tiled CTA-per-instance kernel; MPCG_EUNSUPPORTED when
+// Launch shape of the tiled kernel, one CTA per instance or (`clusters`) more; MPCG_EUNSUPPORTED when
 // its TMA tiles cannot be used (odd nx: a block is not a 16-byte multiple;
 // a block array not 16-byte aligned; nx > 64) or nothing fits in shared
 // memory.  Each knot stream's steps are bound by their own instruction
@@ -105,14 +105,13 @@ int choose_pcg_cta(mpcg_handle *h, const mpcg_dims &d, int B, PcgLaunch &L) {
 // (at most one per four knots of the longest horizon, at most 16 warps) and
 // then the deepest pipeline (up to 2 steps ahead) that still fits.
 template <typename T>
-int choose_pcg_tile(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_schur *s, PcgLaunch &L) {
+int choose_pcg_tile(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_schur *s, bool clusters, PcgLaunch &L) {
     const int nx = d.nx;
     if (nx > 64 || nx % 2 != 0) return MPCG_EUNSUPPORTED;
     if ((sizeof(T) * (size_t)nx * nx) % 16 != 0) return MPCG_EUNSUPPORTED;
     for (const void *ptr : {s->Sd, s->So, s->Pd, s->Po})
         if (ptr && ((uintptr_t)ptr % 16) != 0) return MPCG_EUNSUPPORTED;
     L.cta_mode = 2;
-    L.C = 1;
     L.stage = 0;
     L.lpk = nx <= 16 ? 16 : 32;
     L.rpt = nx <= 32 ? 1 : 2;
@@ -121,48 +120,82 @@ int choose_pcg_tile(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_schur 
     // vector slots padded only to the load width (nx = 14: 14, not 16;
     // measured 3 % faster on 64-knot batches)
     L.vs = ceil_div(nx, L.vw) * L.vw;
-    L.kpc_max = d.N;
+    L.n_long = d.N;
     const int SW = 32 / L.lpk;
-    const int ns_want = std::max(1, std::min(32, ceil_div(d.N, 4)));
     const int wmax = L.nxc == 36 ? 8 : 16;  // the nx = 36 form is compiled for <= 256 threads
-    // the most streams (then the deepest ring) that fit, with diagonal slots
-    // of npk entries (0: full tiles)
-    auto fit = [&](int npk_, int &W_, int &D_) {
-        W_ = D_ = 0;
-        for (int W = std::min(wmax, ceil_div(ns_want, SW)); W >= 1 && !W_; --W)
-            for (int dep = 2; dep >= 1; --dep)
-                if (pcg_tile_smem_bytes<T>(d.N, L.vs, W, W * SW, nx, dep, npk_) <= (size_t)h->smem_optin) {
-                    W_ = W;
-                    D_ = dep;
-                    break;
-                }
-    };
-    int bestW = 0, bestD = 0;
-    fit(0, bestW, bestD);
-    // Packed diagonal blocks (nx = 36, when the caller formed them) cut the
-    // bytes per step by a quarter but add a scalar load per entry: taken
-    // only when their smaller slots fit more knot streams (long horizons,
-    // where the kernel is bound by bytes in flight; measured 1.16-1.21x at
-    // N = 160-256, 5 % slower at N = 64 where the streams are capped anyway).
-    L.pk = 0;
-    int npk = 0;
-    if (L.nxc == 36 && s->Sdp && s->Pdp && (((uintptr_t)s->Sdp | (uintptr_t)s->Pdp) % 16) == 0) {
-        int pW = 0, pD = 0;
-        fit(packed_len(nx), pW, pD);
-        if (pW > bestW) {
-            L.pk = 1;
-            npk = packed_len(nx);
-            bestW = pW;
-            bestD = pD;
+    // shape with C CTAs per instance: co-resident clusters (0: does not fit)
+    auto shape = [&](int C) -> int {
+        L.C = C;
+        L.kpc_max = ceil_div(d.N, C);
+        const int ns_want = std::max(1, std::min(32, ceil_div(L.kpc_max, 4)));
+        auto bytes = [&](int W, int dep, int npk) {
+            return pcg_tile_smem_bytes<T>(L.kpc_max, L.vs, W, W * SW, nx, dep, npk, C > 1);
+        };
+        // the most streams (then the deepest ring) that fit, with diagonal
+        // slots of npk entries (0: full tiles)
+        auto fit = [&](int npk_, int &W_, int &D_) {
+            W_ = D_ = 0;
+            for (int W = std::min(wmax, ceil_div(ns_want, SW)); W >= 1 && !W_; --W)
+                for (int dep = 2; dep >= 1; --dep)
+                    if (bytes(W, dep, npk_) <= (size_t)h->smem_optin) {
+                        W_ = W;
+                        D_ = dep;
+                        break;
+                    }
+        };
+        int bestW = 0, bestD = 0;
+        fit(0, bestW, bestD);
+        // Packed diagonal blocks (nx = 36, when the caller formed them) cut the
+        // bytes per step by a quarter but add a scalar load per entry: taken
+        // only when their smaller slots fit more knot streams (long horizons,
+        // where the kernel is bound by bytes in flight; measured 1.16-1.21x at
+        // N = 160-256, 5 % slower at N = 64 where the streams are capped anyway;
+        // clusters have the room).
+        L.pk = 0;
+        int npk = 0;
+        if (C == 1 && L.nxc == 36 && s->Sdp && s->Pdp && (((uintptr_t)s->Sdp | (uintptr_t)s->Pdp) % 16) == 0) {
+            int pW = 0, pD = 0;
+            fit(packed_len(nx), pW, pD);
+            if (pW > bestW) {
+                L.pk = 1;
+                npk = packed_len(nx);
+                bestW = pW;
+                bestD = pD;
+            }
         }
+        if (!bestW) return 0;
+        L.depth = bestD;
+        L.smem = bytes(bestW, bestD, npk);
+        L.threads = 32 * bestW;
+        return pcg_tile_max_clusters<T>(L, h->sms);
+    };
+    int n = shape(1);  // what one CTA cannot hold stays refused
+    if (n < 1) return MPCG_EUNSUPPORTED;
+    L.n_cta = n;
+    // `clusters` (float32 nx = 36): as many CTAs per instance as pays.  One
+    // iteration of an instance takes about 6 us + 0.35 us per knot of a CTA
+    // (measured alone at 16..224 knots: 12.1, 15.7 at 32, 25 at 64, 51 at 128,
+    // 84), and the batch as many times that as it has waves; the horizons of a
+    // ragged batch, longest first, count 0.6 of the longest.  Within a fifth of
+    // the best the most CTAs: fewer instances at a time, which the L2 holds.
+    // Measured, 1 / 2 / 4 / 8 / 16 CTAs, ms: 160 instances of 64..256 knots
+    // 238 / 152 / 136 / 208 / 336; 24 of 64..256 219 / 121 / 59 / 45 / 65; 300 of
+    // 64..128 119 / 108 / 130 / 236 / 186; 60 of 20..60 20.7 / 14.0 / 11.0 / 10.6 / 12.6.
+    if (clusters && L.nxc == 36) {
+        double cost[5], best = 0.0;
+        int levels = 0;
+        for (int C = 1; C <= kMaxCluster && (C == 1 || d.N >= 8 * C); C *= 2) {
+            const int m = shape(C);
+            const double t = m < 1 ? 1e30 : (6.0 + 0.35 * L.kpc_max) * std::max(1.0, 0.6 * B / m);
+            cost[levels++] = t;
+            if (C == 1 || t < best) best = t;
+        }
+        while (cost[levels - 1] > 1.2 * best) --levels;
+        n = shape(1 << (levels - 1));
     }
-    if (!bestW) return MPCG_EUNSUPPORTED;
-    L.depth = bestD;
-    L.smem = pcg_tile_smem_bytes<T>(d.N, L.vs, bestW, bestW * SW, nx, bestD, npk);
-    L.threads = 32 * bestW;
-    const int per_sm = pcg_tile_max_blocks<T>(L);
-    if (per_sm < 1) return MPCG_EUNSUPPORTED;
-    L.clusters = std::max(1, std::min(B, per_sm * h->sms));
+    L.clusters = std::max(1, std::min(B, n));
+    // a batch of more than one wave starts its long horizons first
+    L.split = L.clusters < B;
     return MPCG_OK;
 }
 
@@ -306,7 +339,7 @@ int choose_pcg(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opts *o, co
     // the L2 CTA kernel has none
     const int dot = (std::is_same<T, float>::value && o && o->dot == 1) ? 1 : 0;
     auto tile = [&](PcgLaunch &Lt) -> int {
-        const int r = choose_pcg_tile<T>(h, d, B, s, Lt);
+        const int r = choose_pcg_tile<T>(h, d, B, s, mode == 0 && !dot, Lt);
         if (r != MPCG_OK || !dot) return r;
         if (Lt.nxc == 0) return MPCG_EUNSUPPORTED;
         Lt.dot = 1;
@@ -320,12 +353,14 @@ int choose_pcg(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opts *o, co
     if (mode == 1) return choose_pcg_cluster<T>(h, d, B, o, L);
     if (mode == 4) return choose_pcg_cluster<T>(h, d, B, o, L, true);
     int rc = choose_pcg_cluster<T>(h, d, B, o, L);
-    // A batch that needs more than one wave of clusters, with operators the
-    // cluster kernel cannot keep in registers (anything but float32 nx = 14),
-    // goes to the tiled kernel: measured 1.25 s vs 3.16 s per solve of the
-    // 1024-instance nx = 36 batch.
+    // Operators the cluster kernels cannot keep on chip go to the tiled kernel:
+    // a batch that needs more than one wave of clusters (measured 1.25 s vs
+    // 3.16 s per solve of the 1024-instance nx = 36 batch), and float32 nx = 36
+    // always, with several CTAs per instance (N = 256 alone 28.6 vs 41.2 ms).
     const bool reg = std::is_same<T, float>::value && d.nx == 14;
-    if (!reg && !(o && o->cluster > 0) && (rc != MPCG_OK || (long)B * L.C > h->sms)) {
+    const bool tiled36 = std::is_same<T, float>::value && d.nx == 36 && !dot;
+    if (!reg && !(o && o->cluster > 0) &&
+        (rc != MPCG_OK || (!L.split_rows && (tiled36 || (long)B * L.C > h->sms)))) {
         PcgLaunch Lt{};
         if (tile(Lt) == MPCG_OK) {
             L = Lt;
@@ -413,10 +448,13 @@ int pcg_t(mpcg_handle *h, const mpcg_dims &d, int B, const int *knot_off, const 
     P.npk = packed_len(d.nx);
     if (P.inst_list && !knot_off) return MPCG_EINVAL;
     if (P.n_tickets > 1 && L.clusters < P.n_tickets) {
-        if (!ws) return MPCG_EINVAL;
+        // (a batch that needs none with a CTA per instance is dealt out in turn)
+        if (!ws && P.n_tickets > L.n_cta) return MPCG_EINVAL;
         P.queue = (int *)ws;
-        rc = err_cuda(cudaMemsetAsync(ws, 0, 8 * sizeof(int), st));  // one counter per group level
-        if (rc) return rc;
+        if (ws) {
+            rc = err_cuda(cudaMemsetAsync(ws, 0, 8 * sizeof(int), st));  // one counter per group level
+            if (rc) return rc;
+        }
     }
     if (L.cta_mode == 2) return err_cuda(pcg_tile_launch<T>(L, P, st));
     if (L.cta_mode == 1) return err_cuda(pcg_cta_launch<T>(L, P, st));

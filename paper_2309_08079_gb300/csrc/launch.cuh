@@ -27,7 +27,9 @@ struct PcgParams {
     const unsigned *info;
     mpcg_stats *stats;
     int *queue;       // instance counters, one per group level (nullptr: static round robin)
-    int split;        // pcg_reg_kernel: clusters split into groups for shorter horizons
+    int split;        // pcg_reg_kernel: clusters split into groups for shorter horizons;
+                      // pcg_tile_kernel: instances by quarters of n_long, long ones first
+    int n_long;       // pcg_tile_kernel: the longest horizon of the launch
     const int *inst_list;  // tickets -> instances (nullptr: ticket t is instance t)
     int n_tickets;         // instances to solve (B, or the list's length)
     double tol;
@@ -54,7 +56,10 @@ struct PcgLaunch {
     int reg;       // cluster form with resident operators (float32, nx = 14): 1 both in
                    // registers, 2 Phi^-1 in shared memory, two CTAs per SM
     int split_rows; // cluster form with rows split over lanes (pcg_split.cu): its variant, 0 none
-    int split;     // reg: one counter per group level, clusters split (see pcg_reg.cu)
+    int n_cta;     // tiled: instances that one CTA each takes at a time
+    int split;     // reg: one counter per group level, clusters split (see pcg_reg.cu);
+                   // tiled: long horizons first (one counter per quarter of n_long)
+    int n_long;    // tiled: the longest horizon the launch is sized for
     int vw;        // pcg_tile_kernel: elements per shared-memory row load (2 or 4)
     int depth;     // pcg_tile_kernel: steps each knot stream copies ahead (1..4)
     int nxc;       // pcg_tile_kernel: nx fixed at compile time (14, 36), else 0
@@ -113,9 +118,9 @@ cudaError_t pcg_split_prepare(int smem_optin);
 cudaError_t pcg_cta_prepare(int smem_optin);
 cudaError_t pcg_tile_prepare(int smem_optin);
 template <typename T>
-size_t pcg_tile_smem_bytes(int nmax, int vs, int W, int NS, int nx, int depth, int npk);
+size_t pcg_tile_smem_bytes(int nmax, int vs, int W, int NS, int nx, int depth, int npk, bool cluster);
 template <typename T> cudaError_t pcg_tile_launch(const PcgLaunch &, const PcgParams<T> &, cudaStream_t);
-template <typename T> int pcg_tile_max_blocks(const PcgLaunch &);
+template <typename T> int pcg_tile_max_clusters(const PcgLaunch &, int sms);
 template <typename T> size_t pcg_cta_smem_bytes(int nmax, int vs, int W);
 template <typename T> cudaError_t pcg_cta_launch(const PcgLaunch &, const PcgParams<T> &, cudaStream_t);
 template <typename T> int pcg_cta_max_blocks(const PcgLaunch &);

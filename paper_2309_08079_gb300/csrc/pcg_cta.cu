@@ -4,7 +4,7 @@
 // one pipeline per knot stream.
 #include <type_traits>
 
-#include "pcg_rows.cuh"
+#include "pcg_sums.cuh"
 
 namespace mpcg {
 
@@ -281,11 +281,13 @@ __global__ void __launch_bounds__(512, 1) pcg_cta_kernel(const PcgParams<T> P) {
 // Per knot stream and pipeline depth d: a ring of d+1 diagonal-block slots
 // (full or packed blocks), d+1 off-diagonal tiles and d+1 mbarriers.
 
+// nmax: knots per CTA.  Clusters (below) add exchange buffers.
+constexpr int TILE_CMAX = 16;
 template <typename T>
 struct TileLayout {
-    size_t r, p, w, tiles, tile_bytes, dtile_bytes, stream_bytes, mbar, wpart, misc, total;
+    size_t r, p, w, tiles, tile_bytes, dtile_bytes, stream_bytes, mbar, wpart, misc, xmbar, slot, halo, total;
     // npk > 0: the diagonal slots hold packed blocks of npk entries
-    __host__ __device__ TileLayout(int nmax, int vs, int W, int NS, int nx, int depth, int npk) {
+    __host__ __device__ TileLayout(int nmax, int vs, int W, int NS, int nx, int depth, int npk, bool cluster) {
         using A = typename std::conditional<sizeof(T) == 4, dfloat, double>::type;
         auto al = [](size_t x) { return (x + 127) & ~size_t(127); };
         size_t o = 0;
@@ -305,6 +307,12 @@ struct TileLayout {
         mbar = o; o = al(o + (size_t)NS * (depth + 1) * sizeof(uint64_t));
         wpart = o; o = al(o + 2 * sizeof(A) * W);
         misc = o; o = al(o + 16);
+        xmbar = slot = halo = o;
+        if (cluster) {
+            xmbar = o; o = al(o + 2 * sizeof(uint64_t));  // exchange A, exchange B
+            slot = o; o = al(o + 2 * TILE_CMAX * 16);     // exchange x source CTA
+            halo = o; o = al(o + 2 * 2 * sizeof(T) * vs);  // exchange x side
+        }
         total = o;
     }
 };
@@ -483,7 +491,18 @@ constexpr int tile_max_threads() { return NXC == 36 ? 256 : 512; }
 // AT: accumulator of the dot products (Acc<T>; AccF64 for float32 with
 // mpcg_opts.dot = 1, where the few FP64 operations per row and step cost
 // little beside the tile products)
-template <typename T, int LPK, int RPT, int VW, int NXC = 0, typename AT = Acc<T>, bool PK = false>
+// CL: a cluster of CTAs per instance, each with its share of the knots.  The
+// sums and the boundary rows travel as in pcg.cu: exchange A after an S+ pass
+// (p^T S p; rows of S p), exchange B after a Phi^-1 pass (r^T r~, ||r||^2; rows of
+// r~).  A CTA alone is bound by the steps of its longest stream (about 1.3 us
+// each), and a batch by its longest instance.  With its share of the knots a
+// CTA's passes shorten and its vectors leave room for more streams, fewer
+// instances at a time fit the L2, and a small batch fills the GPU.  nx = 36, one
+// CTA per instance -> as chosen: 160 instances of 64..256 knots 238 -> 136 ms, 24
+// of 64..256 219 -> 45, 24 of 64..128 62 -> 22; alone at N = 256 41.2 (pcg.cu, 16
+// CTAs) -> 28.6.  Packed diagonal blocks cost more loads than they save here
+// (136 -> 192), a ring of three steps ahead gives nothing.
+template <typename T, int LPK, int RPT, int VW, int NXC = 0, typename AT = Acc<T>, bool PK = false, bool CL = false>
 __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(const PcgParams<T> P) {
     // PK: the diagonal blocks arrive packed (upper triangle by columns) and
     // are read in place, each lane through its row's 36 offsets
@@ -507,7 +526,7 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
     const uint32_t nxb = (uint32_t)(nx2 * sizeof(T));
     const int depth = P.depth;       // steps copied ahead
     const int RD = depth + 1, RO = depth + 1, RM = depth + 1;  // ring sizes
-    TileLayout<T> Lo(P.kpc_max, vs, W, NS, nx, depth, PK ? P.npk : 0);
+    TileLayout<T> Lo(P.kpc_max, vs, W, NS, nx, depth, PK ? P.npk : 0, CL);
     T *vr = reinterpret_cast<T *>(smem + Lo.r);
     T *vp = reinterpret_cast<T *>(smem + Lo.p);
     T *vw = reinterpret_cast<T *>(smem + Lo.w);
@@ -521,8 +540,27 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
     if (tid == 0) fence_mbar_init();
     __syncthreads();
     uint32_t ph = 0u;  // bit x: next phase parity of this stream's barrier x
+    const int C = CL ? (int)cluster_size() : 1, rank = CL ? (int)cluster_rank() : 0;
+    const uint32_t xmb = smem_u32(smem + Lo.xmbar);
+    uint32_t xph = 0u;         // bits 0, 1: next phase parity of exchanges A, B
+    T *xhalo = reinterpret_cast<T *>(smem + Lo.halo);
+    int *s_abort = s_misc + 1;  // set by a peer that gave up waiting
+    bool has_left = false, has_right = false;  // neighbours in this instance
+    if constexpr (CL) {
+        if (tid == 0) {
+            mbar_init(xmb, 1);
+            mbar_init(xmb + 8, 1);
+            *s_abort = 0;
+            fence_mbar_init();
+        }
+        cluster_sync_all();
+    }
 
-    auto reduce2 = [&](A &x, A &y) {
+    // Sums of x and y over the CTA (CL: over the cluster; exchange ex, 0 = A, 1 =
+    // B, which takes the boundary rows of the knot vector `edge`, Nl knots, to
+    // the neighbours' halo rows).  The exchanges alternate, so a peer can be
+    // in the next one only after this CTA has read the last.
+    auto reduce2 = [&](A &x, A &y, int ex, const T *edge, int Nl) -> bool {
 #pragma unroll
         for (int m = 16; m >= 1; m >>= 1) {
             x = AT::add_tree(x, AT::shfl_xor(x, m));
@@ -540,33 +578,94 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
             x = AT::add_tree(x, AT::shfl_xor(x, m));
             y = AT::add_tree(y, AT::shfl_xor(y, m));
         }
+        bool gave_up = false;
+        if constexpr (CL) {
+            const uint32_t bar = xmb + 8 * ex, s0 = smem_u32(smem);
+            if (warp == 0) {
+                if (lane == 0)
+                    mbar_arrive_expect(bar, (uint32_t)C * 16u + (uint32_t)(nx * sizeof(T)) * ((has_left ? 1u : 0u) + (has_right ? 1u : 0u)));
+                if (lane < C) {
+                    const uint32_t pb = map_rank(s0, lane);
+                    push_pair(pb + (uint32_t)Lo.slot + (uint32_t)(ex * TILE_CMAX + rank) * 16u, x, y, pb + (uint32_t)Lo.xmbar + 8 * ex);
+                }
+#pragma unroll
+                for (int side = 0; side < 2; ++side) {  // to the left: the receiver's right halo
+                    if (!(side ? has_right : has_left)) continue;
+                    const uint32_t pb = map_rank(s0, side ? rank + 1 : rank - 1);
+                    const uint32_t dst = pb + (uint32_t)Lo.halo + (uint32_t)((ex * 2 + (1 - side)) * vs * (int)sizeof(T));
+                    for (int i = lane; i < nx; i += 32)
+                        st_async(dst + (uint32_t)(i * sizeof(T)), edge[(side ? Nl : 1) * vs + i], pb + (uint32_t)Lo.xmbar + 8 * ex);
+                }
+                gave_up = warp_wait(bar, (xph >> ex) & 1u, s_abort);
+            }
+            xph ^= 1u << ex;
+            __syncthreads();
+            int cpow = 1;
+            while (cpow < C) cpow <<= 1;
+            const int q = lane & (cpow - 1);
+            x = y = AT::zero();
+            if (q < C) load_pair(reinterpret_cast<const A *>(smem + Lo.slot) + 2 * (ex * TILE_CMAX + q), x, y);
+            for (int m = cpow >> 1; m >= 1; m >>= 1) {
+                x = AT::add_tree(x, AT::shfl_xor(x, m));
+                y = AT::add_tree(y, AT::shfl_xor(y, m));
+            }
+        }
+        return gave_up;
     };
 
-    int served = 0;
+    int served = 0, level = 0;
     bool failed = false;
     for (;;) {
-        if (tid == 0) {
-            int t = P.queue ? atomicAdd(P.queue, 1) : (int)(blockIdx.x + served * gridDim.x);
-            s_misc[0] = t >= P.n_tickets ? -1 : (P.inst_list ? P.inst_list[t] : t);
+        if (tid == 0 && rank == 0) {
+            int b;
+            for (;;) {
+                const int t = P.queue ? atomicAdd(P.queue + level, 1) : (int)(blockIdx.x / C + served * (gridDim.x / C));
+                if (t >= P.n_tickets) {
+                    b = -1;
+                    if (!P.split || level == 3) break;
+                    ++level;  // the next quarter of horizons
+                    continue;
+                }
+                b = P.inst_list ? P.inst_list[t] : t;
+                if (!P.split || b < 0) break;
+                int k0, Nb;
+                P.bv.range(b, k0, Nb);
+                if (min(3, max(0, 3 - (4 * Nb - 1) / P.n_long)) == level) break;
+            }
+            if constexpr (CL) {
+                for (int q = 0; q < C; ++q) st_cluster(map_rank(smem_u32(s_misc), q), b);
+            } else {
+                s_misc[0] = b;
+            }
         }
-        __syncthreads();
+        if constexpr (CL) cluster_sync_all();
+        else __syncthreads();
         const int b = s_misc[0];
         ++served;
         if (b < 0 || failed) break;
         int k0, Nb;
         P.bv.range(b, k0, Nb);
         const int c0 = k0 - b;
-        const bool bad = Nb < 1 || (P.info && P.info[b] != 0u) || Nb > P.kpc_max;
+        const bool bad = Nb < 1 || (P.info && P.info[b] != 0u) || ceil_div(Nb, C) > P.kpc_max;
+        // this CTA's knots [kf, kf + Nl); an instance shorter than the cluster
+        // leaves its last CTAs without any
+        const int Ce = CL ? min(C, max(Nb, 1)) : 1;
+        const int kf = CL ? (rank < Ce ? rank * Nb / Ce : Nb) : 0;
+        const int Nl = CL ? (rank < Ce ? (rank + 1) * Nb / Ce : Nb) - kf : Nb;
+        if constexpr (CL) {
+            has_left = rank > 0 && rank < Ce;
+            has_right = rank + 1 < Ce;
+        }
         const int max_iter = P.max_iter > 0 ? P.max_iter : 10 * Nb * nx;
         int iters = 0, status = MPCG_CONVERGED;
         A eta = AT::zero(), bb = AT::zero();
         T rr_t = T(0);
 
-        // this stream's knots [ks0, ks0 + len); every stream runs Lmax steps
-        // per pass so the two streams of a warp stay converged
-        const int ks0 = bad ? 0 : (int)(((long long)s * Nb) / NS);
-        const int len = bad ? 0 : (int)(((long long)(s + 1) * Nb) / NS) - ks0;
-        const int Lmax = bad ? 0 : ceil_div(Nb, NS);
+        // this stream's knots [ks0, ks0 + len) of the CTA's; every stream runs
+        // Lmax steps per pass so the two streams of a warp stay converged
+        const int ks0 = bad ? 0 : (int)(((long long)s * Nl) / NS);
+        const int len = bad ? 0 : (int)(((long long)(s + 1) * Nl) / NS) - ks0;
+        const int Lmax = bad ? 0 : ceil_div(Nl, NS);
         // Pipeline state of this stream (identical in all its lanes).  Steps
         // are numbered across passes; ring positions advance by one per step
         // (no divisions in the loop).
@@ -582,7 +681,7 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
         // the copies of the next step to issue (leader lane; len > 0): even
         // passes read S+, odd passes Phi^-1
         auto issue_next = [&]() {
-            const int k = ks0 + i_t;
+            const int k = kf + ks0 + i_t;
             const T *Md = (i_ps & 1) ? P.Pd : P.Sd;
             const T *Mo = (i_ps & 1) ? P.Po : P.So;
             const uint32_t bar = mbs + (uint32_t)(i_m * sizeof(uint64_t));
@@ -649,7 +748,7 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
                 T lv[RPT];
                 T *lrow = nullptr;
                 if (lam_upd && act) {
-                    lrow = P.lam + (size_t)(k0 + ks0 + t) * nx;
+                    lrow = P.lam + (size_t)(k0 + kf + ks0 + t) * nx;
 #pragma unroll
                     for (int m = 0; m < RPT; ++m) {
                         const int i = li + m * LPK;
@@ -669,7 +768,7 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
                     break;
                 }
                 if (act) {
-                    const int k = ks0 + t;
+                    const int kv = ks0 + t, k = kf + kv;  // within the CTA's vectors, the instance
                     const bool off = offd(k);
                     const T *D = dslot(c_d);
                     // O_k was copied when some row uses it (as in issue_next)
@@ -685,8 +784,8 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
                             const int i = li + m * LPK;
                             if (i < nx) {
                                 const T bi = P.rhs_sign * P.rhs[(size_t)(k0 + k) * nx + i];
-                                out[(k + 1) * vs + i] = tile_resid<T>(nx, i, bi, D, PK, Lg, hu ? O : nullptr, v + k * vs,
-                                                                      v + (k + 1) * vs, v + (k + 2) * vs);
+                                out[(kv + 1) * vs + i] = tile_resid<T>(nx, i, bi, D, PK, Lg, hu ? O : nullptr, v + kv * vs,
+                                                                       v + (kv + 1) * vs, v + (kv + 2) * vs);
                                 dot = AT::add(dot, AT::prod(bi, bi));
                             }
                         }
@@ -698,14 +797,14 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
                         // row k+1's, for this stream's next step
                         const bool hn = t + 1 < len && k + 1 < Nb && offd(k + 1);
                         T y[RPT];
-                        tile_rows<T, VW, RPT, LPK, NXC, PK, ND>(nx, li, D, O, hu, hn, Lg, lc, v + k * vs,
-                                                                v + (k + 1) * vs, v + (k + 2) * vs, y, cl, dl,
+                        tile_rows<T, VW, RPT, LPK, NXC, PK, ND>(nx, li, D, O, hu, hn, Lg, lc, v + kv * vs,
+                                                                v + (kv + 1) * vs, v + (kv + 2) * vs, y, cl, dl,
                                                                 ts, doff);
 #pragma unroll
                         for (int m = 0; m < RPT; ++m) {
                             const int i = li + m * LPK;
                             if (i < nx) {
-                                const int o = (k + 1) * vs + i;
+                                const int o = (kv + 1) * vs + i;
                                 out[o] = y[m];
                                 const T vi = v[o];
                                 dot = AT::add(dot, AT::prod(vi, y[m]));
@@ -721,15 +820,28 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
         if (bad) {
             status = MPCG_BADINPUT;
         } else {
-            const int nv = (Nb + 2) * vs;
+            const int nv = (Nl + 2) * vs;
             for (int e = tid; e < nv; e += nthreads) {
                 vr[e] = T(0); vp[e] = T(0); vw[e] = T(0);
             }
             __syncthreads();
-            for (int e = tid; e < Nb * nx; e += nthreads) {  // lambda0 into w (halo'd)
-                const int k = e / nx, i = e % nx;
-                vw[(k + 1) * vs + i] = P.lam[(size_t)(k0 + k) * nx + i];
+            // lambda0 into w, with the neighbours' knots beside the CTA's
+            const int lo = has_left ? -1 : 0, hi = Nl + (has_right ? 1 : 0);
+            for (int e = tid; e < (hi - lo) * nx; e += nthreads) {
+                const int k = lo + e / nx, i = e % nx;
+                vw[(k + 1) * vs + i] = P.lam[(size_t)(k0 + kf + k) * nx + i];
             }
+            // a vector's halo rows from exchange ex: fn(vector entry, pushed row's entry)
+            auto halo_rows = [&](T *vec, int ex, auto fn) {
+                if constexpr (CL) {
+                    for (int e = tid; e < 2 * nx; e += nthreads) {
+                        const int side = e / nx, i = e % nx;
+                        if (!(side ? has_right : has_left)) continue;
+                        T &x = vec[(side ? Nl + 1 : 0) * vs + i];
+                        x = fn(x, xhalo[(ex * 2 + side) * vs + i]);
+                    }
+                }
+            };
             // prime each stream's pipeline with its first `depth` steps
             if (len > 0)
                 for (int g = 0; g < depth; ++g) {
@@ -741,18 +853,20 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
             A sbb = AT::zero(), dummy = AT::zero();
             T sq0 = T(0);
             run_pass(0, 0, vw, vr, sbb, sq0);
-            reduce2(sbb, dummy);
+            failed |= reduce2(sbb, dummy, 0, vr, Nl);
             bb = sbb;
+            halo_rows(vr, 0, [](T, T h) { return h; });
             if (__syncthreads_or(failed)) failed = true;  // r complete, wpart read
             A s_eta = AT::zero();
             T sq = T(0);
             if (!failed) run_pass(1, 1, vr, vw, s_eta, sq);
             A s_rr = AT::prod(sq, T(1));
-            reduce2(s_eta, s_rr);
+            failed |= reduce2(s_eta, s_rr, 1, vw, Nl);
             eta = s_eta;
             rr_t = AT::to_T(s_rr);
             if (__syncthreads_or(failed)) failed = true;
-            for (int e = tid; e < nv; e += nthreads) vp[e] = vw[e];
+            for (int e = tid + (CL ? vs : 0); e < nv - (CL ? vs : 0); e += nthreads) vp[e] = vw[e];
+            halo_rows(vp, 1, [](T, T h) { return h; });
             __syncthreads();
 
             const double tol = P.tol > 0 ? P.tol : 1e-6;
@@ -774,7 +888,7 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
                     A s1 = AT::zero(), s1b = AT::zero();
                     T sq1 = T(0);
                     run_pass(1, ps++, vp, vw, s1, sq1);  // S p and p^T S p
-                    reduce2(s1, s1b);
+                    failed |= reduce2(s1, s1b, 0, vw, Nl);
                     iters = it;
                     if (__syncthreads_or(failed)) {
                         failed = true;
@@ -789,17 +903,18 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
                     const T alpha = AT::div(eta_t, ups);
                     // r -= alpha S p (shared memory); lambda += alpha p rides
                     // on the next pass, step by step
-                    for (int e = tid; e < Nb * nx; e += nthreads) {
+                    for (int e = tid; e < Nl * nx; e += nthreads) {
                         const int o = (e / nx + 1) * vs + e % nx;
                         vr[o] = fma_rn(-alpha, vw[o], vr[o]);
                     }
+                    halo_rows(vr, 0, [&](T x, T h) { return fma_rn(-alpha, h, x); });
                     __syncthreads();
                     A s2 = AT::zero();
                     T sq2 = T(0);
                     // r~ = Phi^-1 r, r^T r~, ||r||^2; lambda += alpha p
                     run_pass(1, ps++, vr, vw, s2, sq2, alpha);
                     A s2b = AT::prod(sq2, T(1));
-                    reduce2(s2, s2b);
+                    failed |= reduce2(s2, s2b, 1, vw, Nl);
                     if (__syncthreads_or(failed)) {
                         failed = true;
                         status = MPCG_TIMEOUT;
@@ -818,11 +933,12 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
                     }
                     const T beta = AT::div(etan, eta_t);
                     eta_t = etan;
-                    for (int e = tid; e < Nb * nx; e += nthreads) {
+                    for (int e = tid; e < Nl * nx; e += nthreads) {
                         const int k = e / nx, i = e % nx;
                         const int o = (k + 1) * vs + i;
                         vp[o] = fma_rn(beta, vp[o], vw[o]);
                     }
+                    halo_rows(vp, 1, [&](T x, T h) { return fma_rn(beta, x, h); });
                     __syncthreads();
                 }
             }
@@ -838,7 +954,21 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
             }
             if (__syncthreads_or(failed)) failed = true;
         }
-        if (tid == 0 && P.stats && b < P.bv.B) {
+        bool stop = false;
+        if constexpr (CL) {
+            // Every wait above is bounded, so every CTA arrives here.  One that
+            // gave up says so to all; the whole cluster then leaves, after the
+            // pushes still under way to a CTA that no longer waited.
+            if (failed && tid == 0)
+                for (int q = 0; q < C; ++q) st_cluster(map_rank(smem_u32(s_abort), q), 1);
+            cluster_sync_all();  // and every CTA has read this instance's id
+            stop = *(volatile int *)s_abort != 0;
+            if (stop) {
+                status = MPCG_TIMEOUT;
+                spin_ns(DRAIN_GRACE_NS);
+            }
+        }
+        if (tid == 0 && rank == 0 && P.stats && b < P.bv.B) {
             mpcg_stats st;
             st.iters = iters;
             st.status = status;
@@ -847,8 +977,13 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
             st.relres = bbd > 0.0 ? sqrt(rrd / bbd) : sqrt(rrd);
             P.stats[b] = st;
         }
-        __syncthreads();
+        if constexpr (CL) {
+            if (stop) break;
+        } else {
+            __syncthreads();
+        }
     }
+    if constexpr (CL) cluster_sync_all();
 }
 
 template <typename T>
@@ -898,6 +1033,7 @@ template <typename T>
 static void (*pcg_tile_fn(const PcgLaunch &L))(const PcgParams<T>) {
     if constexpr (sizeof(T) == 4) {
         // the measured shapes with nx fixed at compile time
+        if (L.C > 1) return pcg_tile_kernel<T, 32, 2, 4, 36, Acc<T>, false, true>;
         if (L.nxc == 36 && L.pk)
             return L.dot ? pcg_tile_kernel<T, 32, 2, 4, 36, AccF64, true>
                          : pcg_tile_kernel<T, 32, 2, 4, 36, Acc<T>, true>;
@@ -919,8 +1055,23 @@ static void (*pcg_tile_fn(const PcgLaunch &L))(const PcgParams<T>) {
 }
 
 template <typename T>
-size_t pcg_tile_smem_bytes(int nmax, int vs, int W, int NS, int nx, int depth, int npk) {
-    return TileLayout<T>(nmax, vs, W, NS, nx, depth, npk).total;
+size_t pcg_tile_smem_bytes(int nmax, int vs, int W, int NS, int nx, int depth, int npk, bool cluster) {
+    return TileLayout<T>(nmax, vs, W, NS, nx, depth, npk, cluster).total;
+}
+
+static cudaLaunchConfig_t tile_config(const PcgLaunch &L, int clusters, cudaLaunchAttribute *attr, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(L.C * clusters, 1, 1);
+    cfg.blockDim = dim3(L.threads, 1, 1);
+    cfg.dynamicSmemBytes = L.smem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = L.C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = L.C > 1 ? 1 : 0;
+    return cfg;
 }
 
 template <typename T>
@@ -930,14 +1081,27 @@ cudaError_t pcg_tile_launch(const PcgLaunch &L, const PcgParams<T> &P0, cudaStre
     P.stage_smem = 0;
     P.vs = L.vs;
     P.depth = L.depth;
-    pcg_tile_fn<T>(L)<<<L.clusters, L.threads, L.smem, s>>>(P);
-    return cudaGetLastError();
+    P.split = P.queue ? L.split : 0;
+    P.n_long = L.n_long;
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = tile_config(L, L.clusters, attr, s);
+    return cudaLaunchKernelEx(&cfg, pcg_tile_fn<T>(L), P);
 }
 
+// Co-resident clusters (CTAs when L.C == 1) on the device (0: cannot run).
 template <typename T>
-int pcg_tile_max_blocks(const PcgLaunch &L) {
+int pcg_tile_max_clusters(const PcgLaunch &L, int sms) {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pcg_tile_fn<T>(L), L.threads, L.smem) != cudaSuccess) {
+    cudaError_t e;
+    if (L.C > 1) {
+        cudaLaunchAttribute attr[1];
+        const cudaLaunchConfig_t cfg = tile_config(L, 1, attr, nullptr);
+        e = cudaOccupancyMaxActiveClusters(&n, pcg_tile_fn<T>(L), &cfg);
+    } else {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pcg_tile_fn<T>(L), L.threads, L.smem);
+        n *= sms;
+    }
+    if (e != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -953,6 +1117,9 @@ cudaError_t pcg_tile_prepare(int smem_optin) {
     if ((e = cudaFuncSetAttribute(pcg_tile_kernel<float, 32, 2, 4, 36, AccF64>, a, smem_optin))) return e;
     if ((e = cudaFuncSetAttribute(pcg_tile_kernel<float, 32, 2, 4, 36, Acc<float>, true>, a, smem_optin))) return e;
     if ((e = cudaFuncSetAttribute(pcg_tile_kernel<float, 32, 2, 4, 36, AccF64, true>, a, smem_optin))) return e;
+    const auto clustered = pcg_tile_kernel<float, 32, 2, 4, 36, Acc<float>, false, true>;
+    if ((e = cudaFuncSetAttribute(clustered, a, smem_optin))) return e;
+    if ((e = cudaFuncSetAttribute(clustered, cudaFuncAttributeNonPortableClusterSizeAllowed, 1))) return e;
     if ((e = cudaFuncSetAttribute(pcg_tile_kernel<float, 16, 1, 4>, a, smem_optin))) return e;
     if ((e = cudaFuncSetAttribute(pcg_tile_kernel<float, 32, 1, 4>, a, smem_optin))) return e;
     if ((e = cudaFuncSetAttribute(pcg_tile_kernel<float, 32, 2, 4>, a, smem_optin))) return e;
@@ -964,12 +1131,12 @@ cudaError_t pcg_tile_prepare(int smem_optin) {
     return cudaFuncSetAttribute(pcg_tile_kernel<double, 32, 2, 2>, a, smem_optin);
 }
 
-template size_t pcg_tile_smem_bytes<float>(int, int, int, int, int, int, int);
-template size_t pcg_tile_smem_bytes<double>(int, int, int, int, int, int, int);
+template size_t pcg_tile_smem_bytes<float>(int, int, int, int, int, int, int, bool);
+template size_t pcg_tile_smem_bytes<double>(int, int, int, int, int, int, int, bool);
 template cudaError_t pcg_tile_launch<float>(const PcgLaunch &, const PcgParams<float> &, cudaStream_t);
 template cudaError_t pcg_tile_launch<double>(const PcgLaunch &, const PcgParams<double> &, cudaStream_t);
-template int pcg_tile_max_blocks<float>(const PcgLaunch &);
-template int pcg_tile_max_blocks<double>(const PcgLaunch &);
+template int pcg_tile_max_clusters<float>(const PcgLaunch &, int);
+template int pcg_tile_max_clusters<double>(const PcgLaunch &, int);
 template size_t pcg_cta_smem_bytes<float>(int, int, int);
 template size_t pcg_cta_smem_bytes<double>(int, int, int);
 template cudaError_t pcg_cta_launch<float>(const PcgLaunch &, const PcgParams<float> &, cudaStream_t);
