@@ -253,6 +253,19 @@ inline int choose_pcg_reg(const mpcg_dims &d, int B, const mpcg_opts *o, PcgLaun
         if (n >= 1) {
             L.split = C > 1 && n < B;
             L.clusters = std::min(B, n);
+            // later stages for shorter horizons; the first takes what 3/4 of the
+            // size cannot hold, if there can be such
+            if (L.split && C >= 4) {
+                L.n_low = std::min(B, shape(C / 2, L.reg, kpc));
+                L.n_mid = std::min(B, shape(3 * C / 4, L.reg, kpc));
+                L.C = C;
+                if (L.n_low < 1 || L.n_mid < 1) {
+                    L.n_low = L.n_mid = 0;
+                } else if (C_full <= 3 * C / 4) {
+                    L.C = 3 * C / 4;
+                    L.clusters = L.n_mid;
+                }
+            }
             return MPCG_OK;
         }
     }
@@ -452,7 +465,7 @@ int pcg_t(mpcg_handle *h, const mpcg_dims &d, int B, const int *knot_off, const 
         if (!ws && P.n_tickets > L.n_cta) return MPCG_EINVAL;
         P.queue = (int *)ws;
         if (ws) {
-            rc = err_cuda(cudaMemsetAsync(ws, 0, 8 * sizeof(int), st));  // one counter per group level
+            rc = err_cuda(cudaMemsetAsync(ws, 0, 3 * QUEUE_LEVELS * sizeof(int), st));  // a counter per stage and level
             if (rc) return rc;
         }
     }

@@ -377,6 +377,12 @@ __device__ __forceinline__ void st_async_v4(uint32_t addr, float a, float b, flo
         : "memory");
 }
 
+// Programmatic dependent launch: lets the next launch of the stream begin once
+// every CTA has said so; waits until the launches before this one are complete
+// (and their writes visible).
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Bulk (TMA, 1-D) copy of `bytes` from global to this CTA's shared memory,
 // completing on `mbar`.  Both addresses 16-byte aligned, bytes % 16 == 0.
 // Orders this thread's (and, after a warp or CTA barrier, its peers')

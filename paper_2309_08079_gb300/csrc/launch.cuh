@@ -27,6 +27,7 @@ struct PcgParams {
     const unsigned *info;
     mpcg_stats *stats;
     int *queue;       // instance counters, one per group level (nullptr: static round robin)
+    int n_above, n_upto;  // pcg_reg_kernel: the horizons this launch takes, (n_above, n_upto]
     int split;        // pcg_reg_kernel: clusters split into groups for shorter horizons;
                       // pcg_tile_kernel: instances by quarters of n_long, long ones first
     int n_long;       // pcg_tile_kernel: the longest horizon of the launch
@@ -44,6 +45,9 @@ struct PcgParams {
     int npk;             // entries per packed diagonal block
 };
 
+// Instance counters of one launch (int each): a level per group size
+constexpr int QUEUE_LEVELS = 8;
+
 struct PcgLaunch {
     int cta_mode;  // 0: cluster per instance (pcg_reg_kernel when reg, else
                    // pcg_cluster_kernel); 1: one CTA per instance, blocks from L2
@@ -56,6 +60,8 @@ struct PcgLaunch {
     int reg;       // cluster form with resident operators (float32, nx = 14): 1 both in
                    // registers, 2 Phi^-1 in shared memory, two CTAs per SM
     int split_rows; // cluster form with rows split over lanes (pcg_split.cu): its variant, 0 none
+    int n_mid, n_low;  // reg: clusters of the later stages, 3/4 and 1/2 of the full
+                   // size (0: one launch; see pcg_reg.cu)
     int n_cta;     // tiled: instances that one CTA each takes at a time
     int split;     // reg: one counter per group level, clusters split (see pcg_reg.cu);
                    // tiled: long horizons first (one counter per quarter of n_long)

@@ -49,6 +49,16 @@
 // instances of 32..512 knots: 42.8 ms with a 16-CTA cluster for each and two
 // reductions, 27.5 ms split, 25.3 with two CTAs per SM).
 //
+// Stages: a GPC holds one or two clusters of 16 and then has SMs to spare (14
+// clusters, 224 of 304 CTAs, with two CTAs per SM), and 257..384 knots need no
+// 16.  So a batch of more than one wave takes up to three launches, for the
+// horizons that need full clusters (16, 8 or 4 CTAs), those that 3/4 hold and those
+// that half holds (which split); each may begin in the SMs that the one before
+// leaves free.  One launch -> stages: 256 instances of 32..512 knots 25.5 -> 19.9
+// ms, 64 of 150 3.69 -> 2.27, 40 of 260..384 6.37 -> 4.45, 64 of 65..96 0.95 -> 0.91;
+// where all instances need the full size, nothing (256 of 120..128: 4.90 -> 5.03).
+// 13 CTAs for the middle stage fit the GPU worse (20.9).
+//
 // Exchanges (st.async pushes completing transaction bytes on the receiver's
 // mbarriers, no cluster barrier in the loop): per iteration the boundary rows
 // of r~ go to the neighbour CTAs (barrier Z), then each CTA's four sums go to
@@ -57,6 +67,7 @@
 // one reduction ahead, since the next one needs this CTA's sums.  All CTAs
 // add the partial sums in the same order, so they take identical decisions;
 // halo copies of r and p are updated with the owner's own multiply-adds.
+#include <climits>
 #include <type_traits>
 
 #include "pcg_sums.cuh"
@@ -230,6 +241,12 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
     int level = 0, g0 = 0, G = C;   // this CTA's group: ranks [g0, g0 + G)
     uint32_t mail_phase = 0;
     int served = 0;
+    grid_dep_launch();
+    // the next stage overlaps this one, so the last must outlive them all: one
+    // thread of each stage leaves only when the stage before it is complete
+    auto leave = [&]() {
+        if (blockIdx.x == 0 && tid == 0) grid_dep_wait();
+    };
 
     for (;;) {
         const int gr = rank - g0;  // rank in the group
@@ -249,6 +266,10 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
                 }
                 int k0, Nb;
                 P.bv.range(b, k0, Nb);
+                if (Nb <= P.n_above || Nb > P.n_upto) {  // another stage's instance
+                    b = -1;
+                    continue;
+                }
                 const bool fits = Nb >= 1 && ceil_div(Nb, C) <= P.kpc_max;
                 if (P.split) {  // another level's instance?
                     int need = C, l = 0;
@@ -283,6 +304,7 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
         if (timed_out) {
             if (tid == 0) cluster_drain(rank, C, smem_u32(s_abort), mbS, DRAIN_LIMIT_NS, DRAIN_GRACE_NS);
             __syncthreads();
+            leave();
             return;
         }
         if (b < 0) {
@@ -648,6 +670,7 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
         if (timed_out) {
             if (tid == 0) cluster_drain(rank, C, smem_u32(s_abort), mbS, DRAIN_LIMIT_NS, DRAIN_GRACE_NS);
             __syncthreads();
+            leave();
             return;
         }
         // No barrier between instances: a peer that is already at the next
@@ -655,6 +678,7 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
         // before this CTA's sums for it arrive.
     }
     cluster_sync_all();  // peers may push into this CTA's shared memory until they leave too
+    leave();
 }
 
 size_t pcg_reg_smem_bytes(const PcgLaunch &L) { return RegLayout(L.kpc_max, L.reg == 2 ? L.threads : 0).total; }
@@ -674,6 +698,8 @@ static cudaLaunchConfig_t reg_config(const PcgLaunch &L, int clusters, cudaLaunc
     attr[0].val.clusterDim.x = L.C;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cfg;
@@ -683,14 +709,29 @@ cudaError_t pcg_reg_launch(const PcgLaunch &L, const PcgParams<float> &P0, cudaS
     PcgParams<float> P = P0;
     P.kpc_max = L.kpc_max;
     P.vs = VSR;
-    P.split = L.split;
-    cudaLaunchAttribute attr[1];
-    const cudaLaunchConfig_t cfg = reg_config(L, L.clusters, attr, s);
-    return cudaLaunchKernelEx(&cfg, reg_fn(L), P);
+    cudaLaunchAttribute attr[2];
+    PcgLaunch S = L;
+    P.n_upto = INT_MAX;
+    int full = 1;  // sizes of the stages: full, 3/4 full, 1/2 full
+    while (full < L.C) full *= 2;
+    const int mid = 3 * full / 4, low = full / 2;
+    for (int stage = 0;; ++stage) {
+        const bool to_mid = P.queue && L.n_mid > 0 && S.C > mid, to_low = P.queue && L.n_mid > 0 && S.C == mid;
+        P.n_above = to_mid ? mid * L.kpc_max : to_low ? low * L.kpc_max : INT_MIN;
+        P.split = to_mid || to_low ? 0 : L.split;
+        cudaLaunchConfig_t cfg = reg_config(S, S.clusters, attr, s);
+        if (stage) cfg.numAttrs = 2;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, reg_fn(S), P);
+        if (e != cudaSuccess || !(to_mid || to_low)) return e;
+        P.n_upto = P.n_above;
+        P.queue += QUEUE_LEVELS;
+        S.C = to_mid ? mid : low;
+        S.clusters = to_mid ? L.n_mid : L.n_low;
+    }
 }
 
 int pcg_reg_max_clusters(const PcgLaunch &L) {
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = reg_config(L, 1, attr, nullptr);
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, reg_fn(L), &cfg) != cudaSuccess) {

@@ -128,3 +128,48 @@ def test_more_instances_than_clusters(B, N_lo, N_hi):
         S = oracle.block_tridiag_sparse(Sd[k0:k1], So[k0 - b:k1 - b - 1]).tocsc()
         ref = spla.spsolve(S, -g[k0:k1].ravel()).reshape(n, 14)
         assert oracle.relerr(lam[k0:k1], ref) < TOL_F32 and knot_err(lam[k0:k1], ref) < TOL_KNOT_F32, (b, n)
+
+
+@pytest.mark.parametrize("B,top,C", [(60, 512, 16), (60, 384, 12), (20, 257, 12), (70, 256, 8), (60, 192, 6),
+                                     (90, 128, 4), (90, 96, 3)])
+def test_stages_of_a_ragged_batch(B, top, C):
+    """Horizons at the ends of every stage's range, one instance flagged, one
+    longer than a cluster of the launch holds; the launches of a captured graph give
+    the same lambda, bit for bit."""
+    import torch
+    from paper_2309_08079_gb300.solver import LQTensors, make_opts, read_stats
+    s = solver()
+    edges = [n for n in (top, 385, 384, 257, 256, 193, 192, 129, 128, 97, 96, 65, 64, 48, 33, 32, 1) if n <= top]
+    Ns = edges + gen.batch_horizons(B - 1 - len(edges), 2, min(top, 130), 12).tolist() + [32 * C + 1]
+    items = [gen.kuka_lq(14, 7, int(n), 3500 + i) for i, n in enumerate(Ns)]
+    items[2].Qd[0, 0] = 0.0
+    batch = gen.concat_batch(items).astype(np.float32)
+    lt = LQTensors.from_batch(batch)
+    sch, stats, ws = s.alloc_schur(lt), s.alloc_stats(lt.nb), s.alloc_workspace(lt)
+    s.form(lt, sch)
+    o = make_opts()
+    sh = s.pcg_shape(lt, sch, o, N=top)
+    assert sh["C"] == C and sh["clusters"] < B, sh
+    lam = torch.full((lt.total, 14), 0.25, device="cuda")
+    s.pcg_solve(lt, sch, lam, o, stats, ws, N=top)
+    torch.cuda.synchronize()
+    st = read_stats(stats)
+    again = torch.empty_like(lam)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        again.fill_(0.25)
+        s.pcg_solve(lt, sch, again, o, stats, ws, N=top)
+        after = again + 0.0  # ordered behind every stage
+    for _ in range(3):
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(again, lam) and torch.equal(after, lam)
+    lam, Sd, So, gam = (t.cpu().double().numpy() for t in (lam, sch.Sd, sch.So, sch.gamma))
+    for b, n in enumerate(Ns):
+        k0, k1 = batch.knot_off[b], batch.knot_off[b + 1]
+        if b in (2, B - 1):
+            assert st["status"][b] == 4 and np.all(lam[k0:k1] == 0.25), (b, n)
+            continue
+        S = oracle.block_tridiag_sparse(Sd[k0:k1], So[k0 - b:k1 - b - 1]).tocsc()
+        ref = spla.spsolve(S, -gam[k0:k1].ravel()).reshape(n, 14)
+        assert st["status"][b] == 0 and oracle.relerr(lam[k0:k1], ref) < TOL_F32, (b, n)
