@@ -1,6 +1,6 @@
 // Cluster PCG with one reduction per iteration (the recurrence, the exchanges
 // and the parities are those of pcg_reg.cu) for float32 nx = 36 and float64
-// nx = 14: a lane per row, and one warp of each CTA that only forms the sums.
+// nx = 14: a lane (or Q lanes) per row, and one warp of each CTA that only forms the sums.
 //
 // What bounds it.  float32, nx = 36: the exchanges and barriers, and the
 // shared-memory reads (108 words of vector a row and product, 108 of Phi^-1).
@@ -17,14 +17,14 @@
 //    others update.
 // Measured per iteration, against the general cluster kernel (pcg.cu, blocks in
 // shared memory, two reductions): float32 nx = 36, N = 64: 1.90 against 8.4 us
-// (N = 128: 2.94); float64 nx = 14, N = 101: 6.0 against 8.2 us, of which the
+// (N = 128: 2.94); float64 nx = 14, N = 101: 5.9 against 8.2 us, of which the
 // three products' FP64 instructions are 3.9.
-// Rows split over two or four lanes measured slower at nx = 36 (N = 64, refined
-// solve: 3.3 and 4.4 ms against 2.8: more warps read the vectors), and no
-// faster in float64 (N = 101: 7.5 us, the sums repeated in twice the warps).
+// Rows split over two or four lanes: slower at nx = 36 (N = 64, refined solve:
+// 3.3 and 4.4 ms against 2.8: more warps read the vectors); in float64 faster
+// while that fills schedulers without rows (N = 20: 4.0 against 6.1 us).
 //
 // Layout: CTA r of an instance's C <= 16 CTAs owns KPC = ceil(N/C) knots, thread
-// kl NX + i row i of its knot kl.  The row's 3 nx columns (blocks k-1, k, k+1)
+// (kl NX + i) Q + q part q of row i of its knot kl.  The row's 3 nx columns (blocks k-1, k, k+1)
 // are consecutive words of a vector stored knot after knot.  The rows of S+ lie
 // in registers; those of Phi^-1 too (float64) or in shared memory (float32, as
 // 16-byte words, word w of all threads side by side).
@@ -79,14 +79,17 @@ __device__ __forceinline__ double quot(double a, double b) { return a / b; }
 
 }  // namespace
 
-template <typename T, int NX, int MAXT>
+// Q: lanes per row (float64), each with every Q-th pair of the columns
+template <typename T, int NX, int MAXT, int Q = 1>
 __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P) {
     using AT = Acc<T>;
     using A = typename AT::type;
     constexpr bool PS = sizeof(T) == 4;                   // Phi^-1 in shared memory
     constexpr int ROW = 3 * NX, VW = 16 / (int)sizeof(T);  // a row, entries per 16-byte load
     constexpr int NCH = PS ? VW : 1;                       // chains of a product
+    constexpr int WORDS = ROW / VW, WQ = (WORDS + Q - 1) / Q;  // 16-byte words of a row, of a lane
     static_assert(NX % VW == 0, "16-byte vector slots");
+    static_assert(!PS || Q == 1, "whole rows");
     constexpr uint32_t R0 = 0, Z = 16, TT = 24, STOP = 32, MAIL = 40;  // mbarriers
     extern __shared__ __align__(16) unsigned char smem[];
     struct Sums {
@@ -97,7 +100,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
     const int nthreads = blockDim.x, W = nthreads / 32 - 1;  // row warps
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const bool sums = warp == W;  // the warp without rows
-    const int kl = tid / NX, i = tid % NX;
+    const int kl = tid / (NX * Q), i = tid / Q % NX, q = tid % Q;
 
     const SplitLayout L(P.kpc_max, NX, sizeof(T), nthreads, PS ? ROW * (int)sizeof(T) : 0);
     T *vecR = reinterpret_cast<T *>(smem + L.vecR), *vecP = reinterpret_cast<T *>(smem + L.vecP);
@@ -177,9 +180,10 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
         const int max_iter = P.max_iter > 0 ? P.max_iter : 10 * Nb * NX;
         const int at = (kl + 1) * NX + i;  // this thread's row in a shared vector
         // the warps with a row of the first or last knot wait for the neighbours' rows
-        const bool warp_edge = !sums && ((has_left && warp * 32 < NX) ||
-                                         (has_right && warp * 32 + 31 >= (KPC - 1) * NX && warp * 32 < KPC * NX));
-        const bool hleft = own && kl == 0 && has_left, hright = own && kl == KPC - 1 && has_right;
+        const bool warp_edge = !sums && ((has_left && warp * 32 < NX * Q) ||
+                                         (has_right && warp * 32 + 31 >= (KPC - 1) * NX * Q && warp * 32 < KPC * NX * Q));
+        const bool one = own && q == 0;  // this row's only lane that writes or adds it
+        const bool hleft = one && kl == 0 && has_left, hright = one && kl == KPC - 1 && has_right;
         const bool hany = hleft || hright, hboth = hleft && hright;
         const int side = hleft ? 0 : 1, hat = (side ? (KPC + 1) * NX : 0) + i;
         const uint32_t nb = map_rank(smem_u32(smem), hleft ? rank - 1 : (hright ? rank + 1 : rank));
@@ -197,10 +201,15 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
             if (blk == 0) return k >= 1 ? __ldg(Mo + (size_t)(c0 + k - 1) * n2 + i * NX + j) : T(0);
             return k + 1 < Nb ? __ldg(Mo + (size_t)(c0 + k) * n2 + j * NX + i) : T(0);
         };
-        T sreg[ROW], preg[PS ? 1 : ROW];
+        T sreg[WQ * VW], preg[PS ? 1 : WQ * VW];
+        // entry e of this lane's part of the row is column col(e)
+        auto col = [&](int e) { return ((e / VW) * Q + q) * VW + e % VW; };
+        auto part = [&](const T *Md, const T *Mo, bool off, int e) -> T {
+            return col(e) < ROW ? entry(Md, Mo, off, col(e)) : T(0);
+        };
         float4 *mats = reinterpret_cast<float4 *>(smem + L.mats) + tid;
 #pragma unroll
-        for (int e = 0; e < ROW; ++e) sreg[e] = entry(P.Sd, P.So, true, e);
+        for (int e = 0; e < WQ * VW; ++e) sreg[e] = part(P.Sd, P.So, true, e);
         if constexpr (PS) {
 #pragma unroll
             for (int e = 0; e < ROW; e += 4)
@@ -208,28 +217,33 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
                                                        entry(P.Pd, P.Po, !jac, e + 2), entry(P.Pd, P.Po, !jac, e + 3));
         } else {
 #pragma unroll
-            for (int e = 0; e < ROW; ++e) preg[e] = entry(P.Pd, P.Po, !jac, e);
+            for (int e = 0; e < WQ * VW; ++e) preg[e] = part(P.Pd, P.Po, !jac, e);
         }
 
         // row . vec; float32 sums four chains, float64 one (its latency is
         // hardly above its issue interval)
         auto rowdot = [&](bool precon, const T *vec) -> T {
-            if (!active) return T(0);
             T acc[NCH];
 #pragma unroll
             for (int m = 0; m < NCH; ++m) acc[m] = T(0);
             const T *v = vec + kl * NX;
+            if (active) {
 #pragma unroll
-            for (int e = 0; e < ROW; e += VW) {
-                T x[VW], w[VW];
-                vec_load(v + e, x);
-                if (PS && precon) vec_load(reinterpret_cast<const T *>(mats + (e / VW) * nthreads), w);
+                for (int j = 0; j < WQ; ++j) {
+                    T x[VW], w[VW];
+                    if ((j + 1) * Q > WORDS && j * Q + q >= WORDS) continue;  // past the row
+                    vec_load(v + (j * Q + q) * VW, x);
+                    if (PS && precon) vec_load(reinterpret_cast<const T *>(mats + j * nthreads), w);
 #pragma unroll
-                for (int m = 0; m < VW; ++m)
-                    acc[m % NCH] = fma_rn(precon ? (PS ? w[m] : preg[PS ? 0 : e + m]) : sreg[e + m], x[m], acc[m % NCH]);
+                    for (int m = 0; m < VW; ++m)
+                        acc[m % NCH] = fma_rn(precon ? (PS ? w[m] : preg[PS ? 0 : j * VW + m]) : sreg[j * VW + m], x[m], acc[m % NCH]);
+                }
             }
             if constexpr (PS) return (acc[0] + acc[1]) + (acc[2] + acc[3]);
-            else return acc[0];
+            T y = acc[0];
+#pragma unroll
+            for (int m = 1; m < Q; m *= 2) y += __shfl_xor_sync(0xffffffffu, y, m);
+            return y;
         };
         // Boundary rows to offset off_l (off_r) of the left (right) neighbour's
         // shared memory; float32 rows leave in fours.
@@ -324,11 +338,11 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
         if (active) {
             lam = P.lam[(size_t)(k0 + k) * NX + i];
             bv = P.rhs_sign * P.rhs[(size_t)(k0 + k) * NX + i];
-            v0[at] = lam;
+            if (one) v0[at] = lam;
         }
         // lambda0 halo straight from global memory
-        if (own && kl == 0 && kfirst >= 1 && kfirst - 1 < Nb) v0[i] = P.lam[(size_t)(k0 + kfirst - 1) * NX + i];
-        if (own && kl == KPC - 1 && kfirst + KPC < Nb) v0[(KPC + 1) * NX + i] = P.lam[(size_t)(k0 + kfirst + KPC) * NX + i];
+        if (one && kl == 0 && kfirst >= 1 && kfirst - 1 < Nb) v0[i] = P.lam[(size_t)(k0 + kfirst - 1) * NX + i];
+        if (one && kl == KPC - 1 && kfirst + KPC < Nb) v0[(KPC + 1) * NX + i] = P.lam[(size_t)(k0 + kfirst + KPC) * NX + i];
         __syncthreads();
         if (active) {
             A a = AT::from(bv);
@@ -338,7 +352,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
             for (int e = 0; e < ROW; ++e) a = AT::add(a, AT::prod(-entry(P.Sd, P.So, true, e), v0[kl * NX + e]));
             r = AT::to_T(a);
         }
-        if (own) vecR[at] = r;
+        if (one) vecR[at] = r;
         __syncthreads();
         for (int e = tid; e < (int)(L.vec_bytes / sizeof(T)); e += nthreads) v0[e] = T(0);
         const bool mode1 = P.tol_mode == 1;
@@ -351,7 +365,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
             tol_t = mode1 ? (T)tol : (T)(tol * tol * AT::to_double(bb));
         } else {
             push_halo(0, ipar, r, R0 + 8 * ipar);
-            contribute(AT::prod(bv, bv), AT::zero(), AT::zero(), AT::zero());
+            contribute(one ? AT::prod(bv, bv) : AT::zero(), AT::zero(), AT::zero(), AT::zero());
         }
         ++xr;
         __syncthreads();
@@ -374,10 +388,12 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
             if (!sums) {
                 z = rowdot(true, vecR);
                 push(z, (uint32_t)(L.vecZ + zpar * L.vec_bytes + sizeof(T) * (KPC + 1) * NX), (uint32_t)(L.vecZ + zpar * L.vec_bytes), Z);
-                if (own) vz[at] = z;
-                s_eta = AT::prod(r, z);
-                s_rr = sq_sum(r, T(0), A{});
-                s_eps = AT::prod(z, s);
+                if (one) vz[at] = z;
+                if (Q == 1 || one) {
+                    s_eta = AT::prod(r, z);
+                    s_rr = sq_sum(r, T(0), A{});
+                    s_eps = AT::prod(z, s);
+                }
             } else {
                 if (C > 1 && lane == 0) {
                     mbar_arrive_expect(mb + Z, halo_bytes);
@@ -392,7 +408,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
                     if (warp_wait(mb + Z, xz & 1u, s_abort)) *s_fail = 1;
                 qv = rowdot(false, vz);
                 push_halo(0, zpar, qv, R0 + 8 * rpar);
-                contribute(s_eta, s_rr, AT::prod(z, qv), s_eps);
+                contribute(s_eta, s_rr, Q == 1 || one ? AT::prod(z, qv) : AT::zero(), s_eps);
                 t = rowdot(false, vecP);
                 push_halo(1, zpar, t, TT);
                 if (hany) {
@@ -443,7 +459,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
                     }
                     ups = ud;
                 } else {
-                    contribute(AT::prod(p, s), AT::zero(), AT::zero(), AT::zero());
+                    contribute(Q == 1 || one ? AT::prod(p, s) : AT::zero(), AT::zero(), AT::zero(), AT::zero());
                 }
                 ++xr;
                 __syncthreads();
@@ -461,7 +477,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
             if (!sums) {
                 r = fma_rn(-alpha, s, r);
                 lam = fma_rn(alpha, p, lam);
-                if (own) {
+                if (one) {
                     vecR[at] = r;
                     vecP[at] = p;
                 }
@@ -487,7 +503,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
             ++xz;
         }
         // ---- write back --------------------------------------------------------------
-        if (active) P.lam[(size_t)(k0 + k) * NX + i] = lam;
+        if (active && one) P.lam[(size_t)(k0 + k) * NX + i] = lam;
         if (rank == 0 && sums && lane == 0 && P.stats) {
             const T etan = AT::to_T(eta);
             mpcg_stats st;
@@ -521,14 +537,22 @@ struct SplitForm;
 template <>
 struct SplitForm<float> {
     static constexpr int NX = 36, KPC_MAX = 8, ROW_BYTES = 3 * 36 * 4;
+    static int lanes(int) { return 1; }
     static int variant(int kpc) { return kpc <= 6 ? 1 : 2; }
     static auto fn(int v) { return v == 1 ? pcg_split_kernel<float, 36, 256> : pcg_split_kernel<float, 36, 320>; }
 };
 template <>
 struct SplitForm<double> {
     static constexpr int NX = 14, KPC_MAX = 16, ROW_BYTES = 0;
-    static int variant(int) { return 1; }
-    static auto fn(int) { return pcg_split_kernel<double, 14, 256>; }
+    // Lanes per row, so that a product's instructions spread over the four
+    // schedulers (8 knots x 2 lanes: 7 warps).  Per iteration with 1 lane -> as
+    // chosen: N = 20 6.1 -> 4.0 us, 50 6.0 -> 4.6, 64 5.9 -> 4.5, 96 5.9 -> 5.4, 101
+    // 6.0 -> 5.9 (4 lanes at 3-4 knots: 4.5-4.8, 1 at 5: no gain over 6.0).
+    static int lanes(int kpc) { return kpc <= 2 ? 4 : kpc <= 8 ? 2 : 1; }
+    static int variant(int kpc) { return lanes(kpc); }
+    static auto fn(int v) {
+        return v == 4 ? pcg_split_kernel<double, 14, 256, 4> : v == 2 ? pcg_split_kernel<double, 14, 256, 2> : pcg_split_kernel<double, 14, 256>;
+    }
 };
 
 cudaLaunchConfig_t split_config(const PcgLaunch &L, int clusters, cudaLaunchAttribute *attr, cudaStream_t s) {
@@ -557,7 +581,7 @@ int pcg_split_shape(int nx, int N, int C, PcgLaunch &L) {
     L.split_rows = F::variant(kpc);
     L.C = C;
     L.kpc_max = kpc;
-    L.threads = 32 * (ceil_div(kpc * F::NX, 32) + 1);
+    L.threads = 32 * (ceil_div(kpc * F::NX * F::lanes(kpc), 32) + 1);
     L.smem = SplitLayout(kpc, nx, sizeof(T), L.threads, F::ROW_BYTES).total;
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = split_config(L, 1, attr, nullptr);
@@ -585,7 +609,9 @@ cudaError_t pcg_split_prepare(int smem_optin) {
     };
     cudaError_t e = one(SplitForm<float>::fn(1));
     if (e == cudaSuccess) e = one(SplitForm<float>::fn(2));
-    return e != cudaSuccess ? e : one(SplitForm<double>::fn(1));
+    for (int v : {1, 2, 4})
+        if (e == cudaSuccess) e = one(SplitForm<double>::fn(v));
+    return e;
 }
 
 template int pcg_split_shape<float>(int, int, int, PcgLaunch &);

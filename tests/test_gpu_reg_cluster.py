@@ -35,6 +35,12 @@ def test_capped_iterate_at_every_packing(nx, nu, dtype, N, C):
     assert oracle.relerr(lam, lo.reshape(lam.shape)) < (1e-3 if dtype == "float32" else 1e-9)
 
 
+@pytest.mark.parametrize("N,C", [(2, 1), (3, 2), (4, 1), (20, 16), (31, 16), (64, 16), (65, 16), (8, 1), (9, 1), (115, 16), (128, 16)])
+def test_capped_iterate_with_lanes_per_row(N, C):
+    """float64: four lanes a row up to 2 knots per CTA, two up to 8."""
+    test_capped_iterate_at_every_packing(14, 7, "float64", N, C)
+
+
 @pytest.mark.parametrize("nx,nu,dtype", [(14, 7, "float32"), (36, 12, "float32"), (14, 7, "float64")])
 @pytest.mark.parametrize("N", [16, 48])
 def test_direct_sum_when_the_identity_cancels(nx, nu, dtype, N):
