@@ -205,19 +205,14 @@ int choose_pcg_tile(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_schur 
 //  - Every instance can have its own cluster at once: the largest cluster that
 //    still allows it, down to about 8 knots per CTA (fewer warps per CTA
 //    barrier; a single instance of 64 / 128 knots).
-//  - More instances than clusters: full CTAs, a power of two per cluster, and
-//    clusters that split into groups as the long horizons run out.  With two
-//    waves or more at that residency, two CTAs share an SM (Phi^-1 in shared
-//    memory): each iterates 1.84 times slower, and twice as many run, or more
-//    (36 clusters of 8 in place of 15, 14 of 16 in place of 7).  Measured: 256
-//    instances of 32..512 knots 25.3 against 27.5 ms, 150 of 100..250 6.2
-//    against 7.6; but 20 of 300..512, less than two waves, 4.4 against 3.9.
+//  - More instances than clusters: full CTAs, a power of two (or 3/4 of one)
+//    per cluster, in stages and groups (pcg_reg.cu), two CTAs per SM with Phi^-1
+//    in shared memory; up to four waves by count the form with both operators
+//    in registers beside it, and the device takes the one that the horizons
+//    favour.
 inline int choose_pcg_reg(const mpcg_dims &d, int B, const mpcg_opts *o, PcgLaunch &L) {
-    constexpr int kpc_cap = 32, kpc_small = 8;
+    constexpr int kpc_cap = 32, kpc_cap_ps = 64, kpc_small = 8;
     L.cta_mode = 0;
-    L.reg = 1;
-    L.lpk = 8;
-    L.rpt = 2;
     L.vs = 16;
     const int C_full = ceil_div(d.N, kpc_cap);
     if (C_full > kMaxCluster) return MPCG_EUNSUPPORTED;
@@ -226,7 +221,9 @@ inline int choose_pcg_reg(const mpcg_dims &d, int B, const mpcg_opts *o, PcgLaun
         L.reg = reg;
         L.C = C;
         L.kpc_max = kpc;
-        if (kpc > kpc_cap) return 0;
+        if (kpc > (reg == 2 ? kpc_cap_ps : kpc_cap)) return 0;
+        L.lpk = reg == 2 ? 4 : 8;
+        L.rpt = 16 / L.lpk;
         L.threads = std::max(32, ceil_div(kpc * L.lpk, 32) * 32);
         L.smem = pcg_reg_smem_bytes(L);
         return pcg_reg_max_clusters(L);
@@ -244,32 +241,43 @@ inline int choose_pcg_reg(const mpcg_dims &d, int B, const mpcg_opts *o, PcgLaun
             L.clusters = B;
             return MPCG_OK;
         }
-    int C = 1;
-    while (C < C_full) C <<= 1;
-    for (; C >= C_full && C >= 1; C >>= 1) {
-        const int kpc = C > 1 ? kpc_cap : d.N;
-        int n = shape(C, 2, kpc);
-        if (n < 1 || B < 2 * n) n = shape(C, 1, kpc);
-        if (n >= 1) {
-            L.split = C > 1 && n < B;
-            L.clusters = std::min(B, n);
+    // more instances than clusters: the smallest power of two of CTAs that
+    // holds the longest horizon
+    auto waves = [&](int reg, int cap) {
+        const int need = ceil_div(d.N, cap);
+        int C = 1;
+        while (C < need) C <<= 1;
+        const int kpc = C > 1 ? cap : d.N, n = shape(C, reg, kpc);
+        if (n < 1) return 0;
+        L.clusters = std::min(B, n);
+        L.split = C > 1 && n < B;
+        L.n_low = L.n_mid = 0;
+        if (L.split && C >= 4) {
             // later stages for shorter horizons; the first takes what 3/4 of the
             // size cannot hold, if there can be such
-            if (L.split && C >= 4) {
-                L.n_low = std::min(B, shape(C / 2, L.reg, kpc));
-                L.n_mid = std::min(B, shape(3 * C / 4, L.reg, kpc));
-                L.C = C;
-                if (L.n_low < 1 || L.n_mid < 1) {
-                    L.n_low = L.n_mid = 0;
-                } else if (C_full <= 3 * C / 4) {
-                    L.C = 3 * C / 4;
-                    L.clusters = L.n_mid;
-                }
+            L.n_low = std::min(B, shape(C / 2, reg, kpc));
+            L.n_mid = std::min(B, shape(3 * C / 4, reg, kpc));
+            L.C = C;
+            if (L.n_low < 1 || L.n_mid < 1) {
+                L.n_low = L.n_mid = 0;
+            } else if (need <= 3 * C / 4) {
+                L.C = 3 * C / 4;
+                L.clusters = L.n_mid;
             }
-            return MPCG_OK;
         }
+        return n;
+    };
+    const int n = waves(1, kpc_cap);
+    const PcgLaunch R = L;
+    if (waves(2, d.N <= kpc_cap_ps ? kpc_cap_ps : kpc_cap) < 1) {
+        L = R;
+        return n >= 1 ? MPCG_OK : MPCG_EUNSUPPORTED;
     }
-    return MPCG_EUNSUPPORTED;
+    if (n >= 1 && B < 4 * n) {
+        L.n_long = d.N;
+        L.light = {R.C, R.clusters, R.n_mid, R.n_low, R.split, R.kpc_max, R.threads, R.smem, (long long)(0.95 * R.clusters * R.C * d.N)};
+    }
+    return MPCG_OK;
 }
 
 // Launch shape of the cluster PCG kernels for horizons up to Nmax.  `wide`
@@ -460,7 +468,7 @@ int pcg_t(mpcg_handle *h, const mpcg_dims &d, int B, const int *knot_off, const 
     P.Pdp = (L.cta_mode == 2 && L.pk) ? (const T *)s->Pdp : nullptr;
     P.npk = packed_len(d.nx);
     if (P.inst_list && !knot_off) return MPCG_EINVAL;
-    if (P.n_tickets > 1 && L.clusters < P.n_tickets) {
+    if (P.n_tickets > 1 && (L.clusters < P.n_tickets || L.light.clusters > 0)) {
         // (a batch that needs none with a CTA per instance is dealt out in turn)
         if (!ws && P.n_tickets > L.n_cta) return MPCG_EINVAL;
         P.queue = (int *)ws;

@@ -27,10 +27,12 @@ struct PcgParams {
     const unsigned *info;
     mpcg_stats *stats;
     int *queue;       // instance counters, one per group level (nullptr: static round robin)
+    int pick;         // pcg_reg_kernel: 1 / -1: this launch serves batches of more / at most `work`
+    long long work;
     int n_above, n_upto;  // pcg_reg_kernel: the horizons this launch takes, (n_above, n_upto]
     int split;        // pcg_reg_kernel: clusters split into groups for shorter horizons;
                       // pcg_tile_kernel: instances by quarters of n_long, long ones first
-    int n_long;       // pcg_tile_kernel: the longest horizon of the launch
+    int n_long;       // the longest horizon of the launch (pcg_tile_kernel; with pick)
     const int *inst_list;  // tickets -> instances (nullptr: ticket t is instance t)
     int n_tickets;         // instances to solve (B, or the list's length)
     double tol;
@@ -60,12 +62,19 @@ struct PcgLaunch {
     int reg;       // cluster form with resident operators (float32, nx = 14): 1 both in
                    // registers, 2 Phi^-1 in shared memory, two CTAs per SM
     int split_rows; // cluster form with rows split over lanes (pcg_split.cu): its variant, 0 none
+    // reg == 2: the form in registers too, and the work from which the batch is
+    // not its own (clusters > 0: the device chooses, see pcg_reg.cu)
+    struct {
+        int C, clusters, n_mid, n_low, split, kpc_max, threads;
+        size_t smem;
+        long long work;
+    } light;
     int n_mid, n_low;  // reg: clusters of the later stages, 3/4 and 1/2 of the full
                    // size (0: one launch; see pcg_reg.cu)
     int n_cta;     // tiled: instances that one CTA each takes at a time
     int split;     // reg: one counter per group level, clusters split (see pcg_reg.cu);
                    // tiled: long horizons first (one counter per quarter of n_long)
-    int n_long;    // tiled: the longest horizon the launch is sized for
+    int n_long;    // tiled, reg with light: the longest horizon the launch is sized for
     int vw;        // pcg_tile_kernel: elements per shared-memory row load (2 or 4)
     int depth;     // pcg_tile_kernel: steps each knot stream copies ahead (1..4)
     int nxc;       // pcg_tile_kernel: nx fixed at compile time (14, 36), else 0

@@ -35,11 +35,26 @@
 // Phi^-1 (2 x 84 floats) in registers for the whole solve.  r, p, r~ (with
 // one halo knot on each side) live in shared memory.
 //
-// PS form: with many instances the exchanges of one leave the SM idle two
-// thirds of the time, and one 16-CTA cluster per GPC leaves SMs unused, so two
-// CTAs share an SM: 128 registers a thread hold the rows of S+, the rows of
-// Phi^-1 lie in shared memory (same products in the same order).  The shared-
-// memory reads then bound it: an iteration takes 1.84 times as long.
+// PS form, for batches: with many instances the exchanges of one leave the SM
+// idle two thirds of the time.  Four lanes own a knot, four rows each, their rows
+// of S+ (168 floats) in registers and those of Phi^-1 in shared memory, so a CTA of
+// 32 knots has 128 threads and two share an SM.  (A lane's vector loads serve
+// four rows: half the shared-memory reads of vectors that bound the form it
+// replaces, 8 lanes and 128 registers.)  An iteration takes 1.7-1.8 times as
+// long as alone.  Up to 64 knots one CTA of 256 threads holds an instance, without
+// exchanges (256 of 60..64 knots 1.07 against 1.22 ms); longer ones are better in
+// CTAs of 32 knots, which overlap (64 of 128 knots 1.17 against 1.24 with 64).
+// Former form -> this one: 256 instances of 32..512 knots 19.9 -> 16.4 ms, 256 of
+// 60..64 1.48 -> 1.07, 150 of 100..250 5.85 -> 4.85, 17 of 505..512 3.97 -> 3.66.
+//
+// Choice of the form: PS pays once the other would need a second wave; that
+// depends on the horizons, which the host does not know.  Between one and four
+// waves by count both forms are launched, and each CTA sums CTAs x knots over the
+// instances (the time of a wave): above 0.95 of one wave of the longest horizon the
+// PS launches do the work, below it the others, and the rest leave at once (5 to 20
+// us).  Register form / PS / chosen: 60 instances of 20..128 knots 0.68 / 0.98 /
+// 0.69 ms, 25 of 40..256 1.07 / 1.63 / 1.07, 64 of 128 1.37 / 1.17 / 1.19, 9 of 512
+// 2.63 / 2.07-2.20 / 2.20, 200 of 16..32 0.285 / 0.291 / 0.315.
 //
 // Groups: a launch with more instances than clusters splits its clusters as
 // the long instances run out.  At level l a group of C >> l CTAs takes only
@@ -47,14 +62,14 @@
 // class is exhausted the group splits in two.  A ragged batch then runs its
 // long horizons first, and short ones do not occupy a whole cluster (256
 // instances of 32..512 knots: 42.8 ms with a 16-CTA cluster for each and two
-// reductions, 27.5 ms split, 25.3 with two CTAs per SM).
+// reductions, 27.5 ms split).
 //
 // Stages: a GPC holds one or two clusters of 16 and then has SMs to spare (14
 // clusters, 224 of 304 CTAs, with two CTAs per SM), and 257..384 knots need no
 // 16.  So a batch of more than one wave takes up to three launches, for the
 // horizons that need full clusters (16, 8 or 4 CTAs), those that 3/4 hold and those
 // that half holds (which split); each may begin in the SMs that the one before
-// leaves free.  One launch -> stages: 256 instances of 32..512 knots 25.5 -> 19.9
+// leaves free.  One launch -> stages (with the former PS form): 256 instances of 32..512 knots 25.5 -> 19.9
 // ms, 64 of 150 3.69 -> 2.27, 40 of 260..384 6.37 -> 4.45, 64 of 65..96 0.95 -> 0.91;
 // where all instances need the full size, nothing (256 of 120..128: 4.90 -> 5.03).
 // 13 CTAs for the middle stage fit the GPU worse (20.9).
@@ -78,16 +93,14 @@ namespace {
 
 constexpr int NXR = 14;   // block size
 constexpr int VSR = 16;   // floats per knot slot of a shared vector
-constexpr int LPR = 8;    // lanes per knot
 constexpr int CMAX = 16;  // CTAs per cluster
 constexpr int WMAX = 8;   // warps per CTA
-constexpr int PROWS = 3 * 2 * NXR;  // a thread's entries of one operator
 constexpr int LEVELS = 5; // group sizes C, C/2, ..., C/16
 
 // Shared-memory carve-up, in bytes; the same on host and device.
 struct RegLayout {
     size_t vecR, vecP, vecZ, halo, slot, wpart, mbar, mail, misc, mats, total;
-    // threads > 0: the rows of Phi^-1 of so many threads too
+    // threads > 0: the rows of Phi^-1 of so many threads too, four each
     __host__ __device__ RegLayout(int kpc_max, int threads) {
         size_t o = 0;
         auto take = [&o](size_t bytes) {
@@ -105,19 +118,21 @@ struct RegLayout {
         mbar = take(sizeof(uint64_t) * (4 + LEVELS));  // R0, R1, Z, peers stopped, instance mail
         mail = take(sizeof(int) * LEVELS);
         misc = take(16);
-        mats = take(sizeof(float) * (size_t)PROWS * threads);
+        mats = take(sizeof(float) * (size_t)(3 * 4 * NXR) * threads);
         total = o;
     }
 };
 
-// Two rows of one block row times the halo'd vector: the knot's three
-// 16-float vector slots are read once for both rows.
-__device__ __forceinline__ void rowdot2(const float (&d)[2][NXR], const float (&l)[2][NXR],
-                                        const float (&u)[2][NXR], const float *vprev,
-                                        const float *vself, const float *vnext, float (&y)[2]) {
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, b0 = 0.f, b1 = 0.f, b2 = 0.f;
-    const float4 *s4 = reinterpret_cast<const float4 *>(vself);
+// R rows of one block row times the halo'd vector: the knot's three 16-float
+// vector slots are read once for all of them.
+template <int R>
+__device__ __forceinline__ void rowdot(const float (&d)[R][NXR], const float (&l)[R][NXR], const float (&u)[R][NXR],
+                                       const float *vprev, const float *vself, const float *vnext, float (&y)[R]) {
+    float a0[R], a1[R], a2[R];
+#pragma unroll
+    for (int m = 0; m < R; ++m) a0[m] = a1[m] = a2[m] = 0.f;
     const float4 *p4 = reinterpret_cast<const float4 *>(vprev);
+    const float4 *s4 = reinterpret_cast<const float4 *>(vself);
     const float4 *n4 = reinterpret_cast<const float4 *>(vnext);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -129,63 +144,75 @@ __device__ __forceinline__ void rowdot2(const float (&d)[2][NXR], const float (&
         for (int t = 0; t < 4; ++t) {
             const int j = 4 * q + t;
             if (j < NXR) {
-                a0 = __fmaf_rn(d[0][j], vs_[t], a0);
-                b0 = __fmaf_rn(d[1][j], vs_[t], b0);
-                a1 = __fmaf_rn(l[0][j], vp_[t], a1);
-                b1 = __fmaf_rn(l[1][j], vp_[t], b1);
-                a2 = __fmaf_rn(u[0][j], vn_[t], a2);
-                b2 = __fmaf_rn(u[1][j], vn_[t], b2);
+#pragma unroll
+                for (int m = 0; m < R; ++m) a0[m] = __fmaf_rn(d[m][j], vs_[t], a0[m]);
+#pragma unroll
+                for (int m = 0; m < R; ++m) a1[m] = __fmaf_rn(l[m][j], vp_[t], a1[m]);
+#pragma unroll
+                for (int m = 0; m < R; ++m) a2[m] = __fmaf_rn(u[m][j], vn_[t], a2[m]);
             }
         }
     }
-    y[0] = (a0 + a1) + a2;
-    y[1] = (b0 + b1) + b2;
+#pragma unroll
+    for (int m = 0; m < R; ++m) y[m] = (a0[m] + a1[m]) + a2[m];
 }
 
-// The same with the thread's rows in shared memory (PS form): 21 four-entry
-// words per thread, word c of all threads side by side, so a warp's load is
-// conflict-free; per block seven words, the two rows' entries 4 q .. 4 q + 3
-// in turn (the last word: entries 12 and 13 of both).
-__device__ __forceinline__ void rowdot2_ps(const float4 *m, int stride, const float *vprev,
-                                           const float *vself, const float *vnext, float (&y)[2]) {
-    float sum[3][2];
+// The same with the thread's four rows in shared memory (PS form): 42
+// four-entry words per thread, word c of all threads side by side, so a warp's
+// load is conflict-free; per block 14 words, the rows' entries 4 q .. 4 q + 3 in
+// turn (the last two: entries 12 and 13 of two rows each).
+__device__ __forceinline__ void rowdot_ps(const float4 *m, int stride, const float *v, float (&y)[4]) {
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-        const float4 *v4 = reinterpret_cast<const float4 *>(b == 0 ? vself : b == 1 ? vprev : vnext);
-        const float4 *w = m + (size_t)7 * b * stride;
-        float a0 = 0.f, a1 = 0.f;
+    for (int b = 0; b < 3; ++b) {  // diagonal, lower, upper
+        const float4 *v4 = reinterpret_cast<const float4 *>(v + (b == 0 ? VSR : b == 1 ? 0 : 2 * VSR));
+        const float4 *w = m + (size_t)14 * b * stride;
+        float a[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            const float4 x = v4[q], r0 = w[2 * q * stride], r1 = w[(2 * q + 1) * stride];
-            a0 = __fmaf_rn(r0.x, x.x, a0);
-            a1 = __fmaf_rn(r1.x, x.x, a1);
-            a0 = __fmaf_rn(r0.y, x.y, a0);
-            a1 = __fmaf_rn(r1.y, x.y, a1);
-            a0 = __fmaf_rn(r0.z, x.z, a0);
-            a1 = __fmaf_rn(r1.z, x.z, a1);
-            a0 = __fmaf_rn(r0.w, x.w, a0);
-            a1 = __fmaf_rn(r1.w, x.w, a1);
+            const float4 x = v4[q];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 e = w[(4 * q + i) * stride];
+                a[i] = __fmaf_rn(e.x, x.x, a[i]);
+                a[i] = __fmaf_rn(e.y, x.y, a[i]);
+                a[i] = __fmaf_rn(e.z, x.z, a[i]);
+                a[i] = __fmaf_rn(e.w, x.w, a[i]);
+            }
         }
         const float2 x = *reinterpret_cast<const float2 *>(v4 + 3);
-        const float4 r = w[6 * stride];
-        a0 = __fmaf_rn(r.x, x.x, a0);
-        a1 = __fmaf_rn(r.z, x.x, a1);
-        sum[b][0] = __fmaf_rn(r.y, x.y, a0);
-        sum[b][1] = __fmaf_rn(r.w, x.y, a1);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float4 e = w[(12 + h) * stride];
+            a[2 * h] = __fmaf_rn(e.y, x.y, __fmaf_rn(e.x, x.x, a[2 * h]));
+            a[2 * h + 1] = __fmaf_rn(e.w, x.y, __fmaf_rn(e.z, x.x, a[2 * h + 1]));
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) y[i] = b == 0 ? a[i] : y[i] + a[i];
     }
-    y[0] = (sum[0][0] + sum[1][0]) + sum[2][0];
-    y[1] = (sum[0][1] + sum[1][1]) + sum[2][1];
 }
 
+// a thread's rows as one word of a shared vector
+__device__ __forceinline__ void put(float *p, const float (&v)[2]) { *reinterpret_cast<float2 *>(p) = make_float2(v[0], v[1]); }
+__device__ __forceinline__ void put(float *p, const float (&v)[4]) { *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]); }
+__device__ __forceinline__ void get(const float *p, float (&v)[2]) {
+    const float2 x = *reinterpret_cast<const float2 *>(p);
+    v[0] = x.x; v[1] = x.y;
+}
+__device__ __forceinline__ void get(const float *p, float (&v)[4]) {
+    const float4 x = *reinterpret_cast<const float4 *>(p);
+    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+}
+__device__ __forceinline__ void push_rows(uint32_t a, const float (&v)[2], uint32_t mbar) { st_async(a, dfloat{v[0], v[1]}, mbar); }
+__device__ __forceinline__ void push_rows(uint32_t a, const float (&v)[4], uint32_t mbar) { st_async_v4(a, v[0], v[1], v[2], v[3], mbar); }
+
 __device__ __forceinline__ float resid_row(float b, const float (&d)[NXR], const float (&l)[NXR],
-                                           const float (&u)[NXR], const float *vprev,
-                                           const float *vself, const float *vnext) {
+                                           const float (&u)[NXR], const float *v) {
     dfloat a{b, 0.f};
 #pragma unroll
     for (int j = 0; j < NXR; ++j) {
-        a = df_add(a, df_prod(-d[j], vself[j]));
-        a = df_add(a, df_prod(-l[j], vprev[j]));
-        a = df_add(a, df_prod(-u[j], vnext[j]));
+        a = df_add(a, df_prod(-d[j], v[VSR + j]));
+        a = df_add(a, df_prod(-l[j], v[j]));
+        a = df_add(a, df_prod(-u[j], v[2 * VSR + j]));
     }
     return __fadd_rn(a.hi, a.lo);
 }
@@ -193,7 +220,7 @@ __device__ __forceinline__ float resid_row(float b, const float (&d)[NXR], const
 }  // namespace
 
 template <typename AT, bool PS>
-__global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const PcgParams<float> P) {
+__global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<float> P) {
     using A = typename AT::type;
     static_assert(sizeof(A) == 8, "sums travel in pairs of 8 bytes");
     extern __shared__ __align__(16) unsigned char smem[];
@@ -205,6 +232,7 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
     const int C = (int)cluster_size(), rank = (int)cluster_rank();
     const int nthreads = blockDim.x, W = nthreads / 32;
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+    constexpr int R = PS ? 4 : 2, LPR = 16 / R;  // rows per lane, lanes per knot
     const int kl = tid / LPR, li = tid % LPR;
 
     const RegLayout L(P.kpc_max, PS ? blockDim.x : 0);
@@ -223,6 +251,36 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
     // (0: from the left neighbour, 1: from the right), in floats
     auto halo_off = [](int v, uint32_t par, int side) { return ((v * 2 + (int)par) * 2 + side) * VSR; };
 
+    grid_dep_launch();
+    // the next stage overlaps this one, so the last must outlive them all: one
+    // thread of each stage leaves only when the stage before it is complete
+    auto leave = [&]() {
+        if (blockIdx.x == 0 && tid == 0) grid_dep_wait();
+    };
+
+    if (P.pick) {  // is this form the batch's? (every CTA of both forms finds the same)
+        unsigned long long *sum = reinterpret_cast<unsigned long long *>(wpart), w = 0;
+        if (tid == 0) *sum = 0;
+        __syncthreads();
+        for (int t = tid; t < P.n_tickets; t += nthreads) {
+            int k0, Nb;
+            P.bv.range(P.inst_list ? P.inst_list[t] : t, k0, Nb);
+            if (Nb < 1 || Nb > P.n_long) continue;
+            int need = 1;
+            while (32 * need < Nb) need *= 2;
+            if (need >= 4 && 24 * need >= Nb) need -= need / 4;
+            w += (unsigned long long)need * Nb;
+        }
+        for (int m = 16; m >= 1; m >>= 1) w += __shfl_xor_sync(0xffffffffu, w, m);
+        if (lane == 0) atomicAdd(sum, w);
+        __syncthreads();
+        const bool heavy = (long long)*sum > P.work;
+        __syncthreads();  // wpart is cleared below
+        if (heavy != (P.pick > 0)) {
+            leave();
+            return;
+        }
+    }
     if (tid == 0) {
         for (int i = 0; i < 4 + LEVELS; ++i) mbar_init(mb + 8 * i, i == 3 ? (C > 1 ? C - 1 : 1) : 1);
         *s_abort = 0;
@@ -241,13 +299,6 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
     int level = 0, g0 = 0, G = C;   // this CTA's group: ranks [g0, g0 + G)
     uint32_t mail_phase = 0;
     int served = 0;
-    grid_dep_launch();
-    // the next stage overlaps this one, so the last must outlive them all: one
-    // thread of each stage leaves only when the stage before it is complete
-    auto leave = [&]() {
-        if (blockIdx.x == 0 && tid == 0) grid_dep_wait();
-    };
-
     for (;;) {
         const int gr = rank - g0;  // rank in the group
         const bool has_left = gr > 0, has_right = gr + 1 < G;
@@ -328,24 +379,24 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
         // the warps holding the first and last knot slot (warp-uniform)
         const bool warp_left = has_left && warp == 0;
         const bool warp_right = has_right && warp == ((KPC - 1) * LPR) / 32;
-        const uint32_t halo_bytes = (uint32_t)(NXR * sizeof(float)) * ((has_left ? 1u : 0u) + (has_right ? 1u : 0u));
-        const bool rows = li < NXR / 2;               // lane 7 of a knot holds none
+        const uint32_t halo_bytes = (uint32_t)((PS ? VSR : NXR) * sizeof(float)) * ((has_left ? 1u : 0u) + (has_right ? 1u : 0u));
+        const bool rows = R * li < NXR;               // (R = 2) lane 7 of a knot holds none
         const bool rv = active_knot && rows, st = slot_knot && rows;
-        const int own = (kl + 1) * VSR + 2 * li;      // this thread's rows in a shared vector
+        const int own = (kl + 1) * VSR + R * li;      // this thread's rows in a shared vector
         // A boundary knot's lanes keep the neighbour's halo copies current and
         // push their own rows: `side` is the side they face (a group with one
         // knot slot per CTA faces both: its left lanes repeat for the right).
         const bool hleft = kl == 0 && has_left && rows, hright = kl == KPC - 1 && has_right && rows;
         const bool hany = hleft || hright, hboth = hleft && hright;
-        const int side = hleft ? 0 : 1, hbase = (side ? (KPC + 1) * VSR : 0) + 2 * li;
+        const int side = hleft ? 0 : 1, hbase = (side ? (KPC + 1) * VSR : 0) + R * li;
         const uint32_t nb = map_rank(smem_u32(smem), hleft ? rank - 1 : (hright ? rank + 1 : rank));
-        const uint32_t nb_halo = nb + (uint32_t)(L.halo + sizeof(float) * ((1 - side) * VSR + 2 * li));
+        const uint32_t nb_halo = nb + (uint32_t)(L.halo + sizeof(float) * ((1 - side) * VSR + R * li));
         const uint32_t nb_mbar = nb + (uint32_t)L.mbar;
 
         // ---- rows of S+ and Phi^-1 into registers -----------------------------
-        float sd[2][NXR], sl[2][NXR], su[2][NXR];
+        float sd[R][NXR], sl[R][NXR], su[R][NXR];
         constexpr int NQ = PS ? 1 : NXR;
-        float qd[2][NQ], ql[2][NQ], qu[2][NQ];  // (PS: in shared memory)
+        float qd[R][NQ], ql[R][NQ], qu[R][NQ];  // (PS: in shared memory)
         float4 *mq = reinterpret_cast<float4 *>(smem + L.mats) + tid;
         {
             // Phi^-1 rows without off-diagonal blocks: every row for block
@@ -356,30 +407,31 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
             const float *Sd = P.Sd + (size_t)(k0 + k) * n2, *Pd = P.Pd + (size_t)(k0 + k) * n2;
             const float *SoL = P.So + (ptrdiff_t)(c0 + k - 1) * n2, *PoL = P.Po + (ptrdiff_t)(c0 + k - 1) * n2;
             const float *SoU = P.So + (size_t)(c0 + k) * n2, *PoU = P.Po + (size_t)(c0 + k) * n2;
-            // rows 2 li, 2 li + 1 of a block: down its columns (the diagonal
+            // rows R li .. of a block (none past the last): down its columns (the diagonal
             // blocks are symmetric), or along its rows
             auto rows_of = [&](const float *M, bool on, bool along, auto &out) {
 #pragma unroll
-                for (int m = 0; m < 2; ++m)
+                for (int m = 0; m < R; ++m)
 #pragma unroll
                     for (int j = 0; j < NXR; ++j) {
-                        const int i = 2 * li + m;
-                        out[m][j] = on && rv ? __ldg(M + (along ? i * NXR + j : j * NXR + i)) : 0.f;
+                        const int i = R * li + m;
+                        out[m][j] = on && rv && (NXR % R == 0 || i < NXR) ? __ldg(M + (along ? i * NXR + j : j * NXR + i)) : 0.f;
                     }
             };
             rows_of(Sd, true, false, sd);
             rows_of(SoL, hl, true, sl);
             rows_of(SoU, hu, false, su);
             if constexpr (PS) {
-                auto stash = [&](int b, const float (&x)[2][NXR]) {
+                auto stash = [&](int b, const float (&x)[R][NXR]) {
 #pragma unroll
                     for (int q = 0; q < 3; ++q)
 #pragma unroll
-                        for (int m = 0; m < 2; ++m)
-                            mq[(7 * b + 2 * q + m) * nthreads] = make_float4(x[m][4 * q], x[m][4 * q + 1], x[m][4 * q + 2], x[m][4 * q + 3]);
-                    mq[(7 * b + 6) * nthreads] = make_float4(x[0][12], x[0][13], x[1][12], x[1][13]);
+                        for (int m = 0; m < 4; ++m)
+                            mq[(14 * b + 4 * q + m) * nthreads] = make_float4(x[m][4 * q], x[m][4 * q + 1], x[m][4 * q + 2], x[m][4 * q + 3]);
+                    for (int h = 0; h < 2; ++h)
+                        mq[(14 * b + 12 + h) * nthreads] = make_float4(x[2 * h][12], x[2 * h][13], x[2 * h + 1][12], x[2 * h + 1][13]);
                 };
-                float x[2][NXR];
+                float x[R][NXR];
                 rows_of(Pd, true, false, x);
                 stash(0, x);
                 rows_of(PoL, hl && !jac, true, x);
@@ -393,17 +445,22 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
             }
         }
 
-        // Boundary rows into the neighbours' halo slots of vector v, one 8-byte
-        // push per lane; bar: byte offset of the mbarrier among the CTA's.
-        auto push_halo = [&](int v, uint32_t par, uint32_t bar, const float (&val)[2]) {
+        // Boundary rows into the neighbours' halo slots of vector v, one push
+        // per lane; bar: byte offset of the mbarrier among the CTA's.
+        auto push_halo = [&](int v, uint32_t par, uint32_t bar, const float (&val)[R]) {
             if (!hany) return;
             const uint32_t off = (uint32_t)sizeof(float) * (uint32_t)halo_off(v, par, 0);
-            st_async(nb_halo + off, dfloat{val[0], val[1]}, nb_mbar + bar);
+            push_rows(nb_halo + off, val, nb_mbar + bar);
             if (hboth) {
                 const uint32_t nr = map_rank(smem_u32(smem), rank + 1);
-                st_async(nr + (uint32_t)(L.halo + sizeof(float) * 2 * li) + off, dfloat{val[0], val[1]},
-                         nr + (uint32_t)L.mbar + bar);
+                push_rows(nr + (uint32_t)(L.halo + sizeof(float) * R * li) + off, val, nr + (uint32_t)L.mbar + bar);
             }
+        };
+        // x . y over this thread's rows
+        auto dot = [](const float (&x)[R], const float (&y)[R]) -> A {
+            A a = AT::add(AT::prod(x[0], y[0]), AT::prod(x[1], y[1]));
+            if constexpr (R == 4) a = AT::add(a, AT::add(AT::prod(x[2], y[2]), AT::prod(x[3], y[3])));
+            return a;
         };
 
         // One thread, some way ahead of the exchange: the bytes that complete
@@ -476,15 +533,16 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
         // ---- initialisation: r = b - S lambda0, ||b||^2 ---------------------------
         for (int e = tid; e < (P.kpc_max + 2) * VSR; e += nthreads) vecR[e] = vecP[e] = vecZ[e] = 0.f;
         __syncthreads();
-        float lam[2] = {0.f, 0.f}, r[2] = {0.f, 0.f}, p[2] = {0.f, 0.f}, s[2] = {0.f, 0.f};
+        float lam[R] = {}, r[R] = {}, p[R] = {}, s[R] = {};
         const bool mode1 = P.tol_mode == 1;
         float tol_t;
         A bb;
         {
-            float bv[2] = {0.f, 0.f};
+            float bv[R] = {};
 #pragma unroll
-            for (int m = 0; m < 2; ++m) {
-                const int i = 2 * li + m;
+            for (int m = 0; m < R; ++m) {
+                const int i = R * li + m;
+                if (i >= NXR) continue;
                 if (rv) {
                     lam[m] = P.lam[(size_t)(k0 + k) * NXR + i];
                     bv[m] = P.rhs_sign * P.rhs[(size_t)(k0 + k) * NXR + i];
@@ -498,17 +556,23 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
             __syncthreads();
             const float *vp = vecZ + kl * VSR;
             if (rv) {
-                r[0] = resid_row(bv[0], sd[0], sl[0], su[0], vp, vp + VSR, vp + 2 * VSR);
-                r[1] = resid_row(bv[1], sd[1], sl[1], su[1], vp, vp + VSR, vp + 2 * VSR);
+#pragma unroll
+                for (int m = 0; m < R; ++m) r[m] = resid_row(bv[m], sd[m], sl[m], su[m], vp);
             }
-            if (st) *reinterpret_cast<float2 *>(vecR + own) = make_float2(r[0], r[1]);
+            if (st) put(vecR + own, r);
             const uint32_t par = xr & 1u;
             push_halo(1, par, 8 * par, r);
             expect(1u);
-            bb = exchange(AT::add(AT::prod(bv[0], bv[0]), AT::prod(bv[1], bv[1])), AT::zero(), AT::zero(), AT::zero()).eta;
-            if (hany) *reinterpret_cast<float2 *>(vecR + hbase) = *reinterpret_cast<const float2 *>(halo + halo_off(1, par, side) + 2 * li);
-            if (hboth)
-                *reinterpret_cast<float2 *>(vecR + 2 * VSR + 2 * li) = *reinterpret_cast<const float2 *>(halo + halo_off(1, par, 1) + 2 * li);
+            bb = exchange(dot(bv, bv), AT::zero(), AT::zero(), AT::zero()).eta;
+            float h[R];
+            if (hany) {
+                get(halo + halo_off(1, par, side) + R * li, h);
+                put(vecR + hbase, h);
+            }
+            if (hboth) {
+                get(halo + halo_off(1, par, 1) + R * li, h);
+                put(vecR + 2 * VSR + R * li, h);
+            }
             const double tol = P.tol > 0 ? P.tol : 1e-6;
             tol_t = mode1 ? (float)tol : (float)(tol * tol * AT::to_double(bb));
         }
@@ -525,25 +589,26 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
             // ---- r~ = Phi^-1 r, boundary rows to the neighbours -----------------
             const uint32_t zpar = xz & 1u, rpar = xr & 1u;  // halo rows alternate once per iteration
             const int failed = *s_fail;  // before the barrier: as every warp saw it
-            float z[2] = {0.f, 0.f}, q[2] = {0.f, 0.f}, t[2] = {0.f, 0.f};
+            float z[R] = {}, q[R] = {}, t[R] = {};
             if (active_knot) {
                 const float *vp = vecR + kl * VSR;
-                if constexpr (PS) rowdot2_ps(mq, nthreads, vp, vp + VSR, vp + 2 * VSR, z);
-                else rowdot2(qd, ql, qu, vp, vp + VSR, vp + 2 * VSR, z);
+                if constexpr (PS) rowdot_ps(mq, nthreads, vp, z);
+                else rowdot<R>(qd, ql, qu, vp, vp + VSR, vp + 2 * VSR, z);
             }
             push_halo(0, zpar, 16, z);
-            if (st) *reinterpret_cast<float2 *>(vecZ + own) = make_float2(z[0], z[1]);
+            if (st) put(vecZ + own, z);
             if (G > 1 && tid == arm) mbar_arrive_expect(mbZ, halo_bytes);
             expect(2u);
             // ---- S p_old and the sums without S r~, while they travel -------------
             if (active_knot) {
                 const float *vp = vecP + kl * VSR;
-                rowdot2(sd, sl, su, vp, vp + VSR, vp + 2 * VSR, t);
+                rowdot<R>(sd, sl, su, vp, vp + VSR, vp + 2 * VSR, t);
             }
             push_halo(2, zpar, 8 * rpar, t);
-            const A s_eta = AT::add(AT::prod(r[0], z[0]), AT::prod(r[1], z[1]));
-            const A s_rr = sq_sum(r[0], r[1], A{});
-            const A s_eps = AT::add(AT::prod(z[0], s[0]), AT::prod(z[1], s[1]));
+            const A s_eta = dot(r, z);
+            A s_rr = sq_sum(r[0], r[1], A{});
+            if constexpr (R == 4) s_rr = AT::add(s_rr, sq_sum(r[2], r[3], A{}));
+            const A s_eps = dot(z, s);
             if (failed) {
                 timed_out = true;
                 break;
@@ -555,23 +620,30 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
             ++xz;
             if (active_knot) {
                 const float *vp = vecZ + kl * VSR;
-                rowdot2(sd, sl, su, kl == 0 && has_left ? halo + halo_off(0, zpar, 0) : vp, vp + VSR,
-                        kl == KPC - 1 && has_right ? halo + halo_off(0, zpar, 1) : vp + 2 * VSR, q);
+                rowdot<R>(sd, sl, su, kl == 0 && has_left ? halo + halo_off(0, zpar, 0) : vp, vp + VSR,
+                          kl == KPC - 1 && has_right ? halo + halo_off(0, zpar, 1) : vp + 2 * VSR, q);
             }
             push_halo(1, zpar, 8 * rpar, q);
-            // the boundary lanes' halo operands are loaded before alpha and beta are formed
-            float2 hz, hq, ht, hp, hr;
-            hz = hq = ht = hp = hr = make_float2(0.f, 0.f);
-            const float *hsrc = halo + halo_off(0, 0, side) + 2 * li;
-            if (hany) {
-                hz = *reinterpret_cast<const float2 *>(hsrc + halo_off(0, zpar, 0));
-                hp = *reinterpret_cast<const float2 *>(vecP + hbase);
-                hr = *reinterpret_cast<const float2 *>(vecR + hbase);
+            // the boundary lanes' halo operands are loaded before alpha and beta
+            // are formed (PS: when used, there are no registers to spare)
+            constexpr int RH = PS ? 1 : R;
+            float hz[RH], hq[RH], ht[RH], hp[RH], hr[RH];
+            const float *hsrc = halo + halo_off(0, 0, side) + R * li;
+            if constexpr (!PS) {
+#pragma unroll
+                for (int m = 0; m < R; ++m) hz[m] = hq[m] = ht[m] = hp[m] = hr[m] = 0.f;
+                if (hany) {
+                    get(hsrc + halo_off(0, zpar, 0), hz);
+                    get(vecP + hbase, hp);
+                    get(vecR + hbase, hr);
+                }
             }
-            const Sums S = exchange(s_eta, s_rr, AT::add(AT::prod(z[0], q[0]), AT::prod(z[1], q[1])), s_eps);
-            if (hany) {
-                hq = *reinterpret_cast<const float2 *>(hsrc + halo_off(1, zpar, 0));
-                ht = *reinterpret_cast<const float2 *>(hsrc + halo_off(2, zpar, 0));
+            const Sums S = exchange(s_eta, s_rr, dot(z, q), s_eps);
+            if constexpr (!PS) {
+                if (hany) {
+                    get(hsrc + halo_off(1, zpar, 0), hq);
+                    get(hsrc + halo_off(2, zpar, 0), ht);
+                }
             }
             eta = S.eta;
             rr = S.rr;
@@ -587,34 +659,43 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
             // r -= alpha S p; the halo copies of p and r alike
             auto next_p = [&]() {
 #pragma unroll
-                for (int m = 0; m < 2; ++m) {
+                for (int m = 0; m < R; ++m) {
                     s[m] = fma_rn(beta, t[m], q[m]);
                     p[m] = fma_rn(beta, p[m], z[m]);
                 }
             };
             auto apply = [&]() {
 #pragma unroll
-                for (int m = 0; m < 2; ++m) {
+                for (int m = 0; m < R; ++m) {
                     r[m] = fma_rn(-alpha, s[m], r[m]);
                     lam[m] = fma_rn(alpha, p[m], lam[m]);
                 }
                 if (st) {
-                    *reinterpret_cast<float2 *>(vecR + own) = make_float2(r[0], r[1]);
-                    *reinterpret_cast<float2 *>(vecP + own) = make_float2(p[0], p[1]);
+                    put(vecR + own, r);
+                    put(vecP + own, p);
                 }
+                // halo rows from one side (h: what it pushed), entry `base` of r and p
+                auto halo_update = [&](const float *h, int base) {
+                    float *vr = vecR + base, *vp = vecP + base;
+                    for (int m = 0; m < R; ++m) {
+                        vr[m] = fma_rn(-alpha, fma_rn(beta, h[halo_off(2, zpar, 0) + m], h[halo_off(1, zpar, 0) + m]), vr[m]);
+                        vp[m] = fma_rn(beta, vp[m], h[halo_off(0, zpar, 0) + m]);
+                    }
+                };
                 if (hany) {
-                    *reinterpret_cast<float2 *>(vecR + hbase) = make_float2(fma_rn(-alpha, fma_rn(beta, ht.x, hq.x), hr.x),
-                                                                            fma_rn(-alpha, fma_rn(beta, ht.y, hq.y), hr.y));
-                    *reinterpret_cast<float2 *>(vecP + hbase) = make_float2(fma_rn(beta, hp.x, hz.x), fma_rn(beta, hp.y, hz.y));
-                }
-                if (hboth) {
-                    const float *h = halo + halo_off(0, 0, 1) + 2 * li;
-                    for (int m = 0; m < 2; ++m) {
-                        float *vr = vecR + 2 * VSR + 2 * li + m, *vp = vecP + 2 * VSR + 2 * li + m;
-                        *vr = fma_rn(-alpha, fma_rn(beta, h[halo_off(2, zpar, 0) + m], h[halo_off(1, zpar, 0) + m]), *vr);
-                        *vp = fma_rn(beta, *vp, h[halo_off(0, zpar, 0) + m]);
+                    if constexpr (PS) {
+                        halo_update(hsrc, hbase);
+                    } else {
+#pragma unroll
+                        for (int m = 0; m < R; ++m) {
+                            hr[m] = fma_rn(-alpha, fma_rn(beta, ht[m], hq[m]), hr[m]);
+                            hp[m] = fma_rn(beta, hp[m], hz[m]);
+                        }
+                        put(vecR + hbase, hr);
+                        put(vecP + hbase, hp);
                     }
                 }
+                if (hboth) halo_update(halo + halo_off(0, 0, 1) + R * li, 2 * VSR + R * li);
             };
             if (!done) {
                 next_p();
@@ -633,7 +714,7 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
                 if (done) break;
                 // sum p^T S p itself
                 expect(0u);
-                ups = AT::to_T(exchange(AT::add(AT::prod(p[0], s[0]), AT::prod(p[1], s[1])), AT::zero(), AT::zero(), AT::zero()).eta);
+                ups = AT::to_T(exchange(dot(p, s), AT::zero(), AT::zero(), AT::zero()).eta);
                 if (!(ups > 0.f) || !isfinite(ups)) {
                     broke = true;
                     iters = it + 1;
@@ -648,7 +729,8 @@ __global__ void __launch_bounds__(32 * WMAX, PS ? 2 : 1) pcg_reg_kernel(const Pc
         }
         // ---- write back ----------------------------------------------------------
         if (rv)
-            for (int m = 0; m < 2; ++m) P.lam[(size_t)(k0 + k) * NXR + 2 * li + m] = lam[m];
+            for (int m = 0; m < R; ++m)
+                if (R * li + m < NXR) P.lam[(size_t)(k0 + k) * NXR + R * li + m] = lam[m];
         if (gr == 0 && tid == 0 && P.stats) {
             const float etan = AT::to_T(eta);
             mpcg_stats st;
@@ -705,22 +787,22 @@ static cudaLaunchConfig_t reg_config(const PcgLaunch &L, int clusters, cudaLaunc
     return cfg;
 }
 
-cudaError_t pcg_reg_launch(const PcgLaunch &L, const PcgParams<float> &P0, cudaStream_t s) {
-    PcgParams<float> P = P0;
+// The stages of one form; `after`: it may begin while the launch before it runs
+static cudaError_t reg_stages(const PcgLaunch &L, PcgParams<float> P, bool after, cudaStream_t s) {
     P.kpc_max = L.kpc_max;
     P.vs = VSR;
+    P.n_upto = INT_MAX;
     cudaLaunchAttribute attr[2];
     PcgLaunch S = L;
-    P.n_upto = INT_MAX;
     int full = 1;  // sizes of the stages: full, 3/4 full, 1/2 full
     while (full < L.C) full *= 2;
     const int mid = 3 * full / 4, low = full / 2;
-    for (int stage = 0;; ++stage) {
+    for (;; after = true) {
         const bool to_mid = P.queue && L.n_mid > 0 && S.C > mid, to_low = P.queue && L.n_mid > 0 && S.C == mid;
         P.n_above = to_mid ? mid * L.kpc_max : to_low ? low * L.kpc_max : INT_MIN;
         P.split = to_mid || to_low ? 0 : L.split;
         cudaLaunchConfig_t cfg = reg_config(S, S.clusters, attr, s);
-        if (stage) cfg.numAttrs = 2;
+        if (after) cfg.numAttrs = 2;
         const cudaError_t e = cudaLaunchKernelEx(&cfg, reg_fn(S), P);
         if (e != cudaSuccess || !(to_mid || to_low)) return e;
         P.n_upto = P.n_above;
@@ -728,6 +810,28 @@ cudaError_t pcg_reg_launch(const PcgLaunch &L, const PcgParams<float> &P0, cudaS
         S.C = to_mid ? mid : low;
         S.clusters = to_mid ? L.n_mid : L.n_low;
     }
+}
+
+cudaError_t pcg_reg_launch(const PcgLaunch &L, const PcgParams<float> &P0, cudaStream_t s) {
+    PcgParams<float> P = P0;
+    const bool pick = L.light.clusters > 0 && P.queue;
+    P.pick = pick ? 1 : 0;
+    P.work = L.light.work;
+    P.n_long = L.n_long;
+    const cudaError_t e = reg_stages(L, P, false, s);
+    if (e != cudaSuccess || !pick) return e;
+    PcgLaunch R = L;
+    R.reg = 1;
+    R.C = L.light.C;
+    R.clusters = L.light.clusters;
+    R.n_mid = L.light.n_mid;
+    R.n_low = L.light.n_low;
+    R.split = L.light.split;
+    R.kpc_max = L.light.kpc_max;
+    R.threads = L.light.threads;
+    R.smem = L.light.smem;
+    P.pick = -1;
+    return reg_stages(R, P, true, s);
 }
 
 int pcg_reg_max_clusters(const PcgLaunch &L) {

@@ -136,17 +136,19 @@ def test_more_instances_than_clusters(B, N_lo, N_hi):
         assert oracle.relerr(lam[k0:k1], ref) < TOL_F32 and knot_err(lam[k0:k1], ref) < TOL_KNOT_F32, (b, n)
 
 
-@pytest.mark.parametrize("B,top,C", [(60, 512, 16), (60, 384, 12), (20, 257, 12), (70, 256, 8), (60, 192, 6),
-                                     (90, 128, 4), (90, 96, 3)])
+@pytest.mark.parametrize("B,top,C", [(60, 512, 16), (20, 512, 16), (60, 384, 12), (20, 257, 12), (70, 256, 8), (20, 256, 8),
+                                     (60, 192, 6), (90, 128, 4), (40, 128, 4), (90, 96, 3), (300, 96, 3), (100, 64, 1), (200, 33, 1)])
 def test_stages_of_a_ragged_batch(B, top, C):
-    """Horizons at the ends of every stage's range, one instance flagged, one
+    """Horizons at the ends of every stage's range, from batches that the
+    device leaves to the form in registers (40 of 128, 20 of 512) to those of
+    many waves; one instance flagged, one
     longer than a cluster of the launch holds; the launches of a captured graph give
     the same lambda, bit for bit."""
     import torch
     from paper_2309_08079_gb300.solver import LQTensors, make_opts, read_stats
     s = solver()
     edges = [n for n in (top, 385, 384, 257, 256, 193, 192, 129, 128, 97, 96, 65, 64, 48, 33, 32, 1) if n <= top]
-    Ns = edges + gen.batch_horizons(B - 1 - len(edges), 2, min(top, 130), 12).tolist() + [32 * C + 1]
+    Ns = edges + gen.batch_horizons(B - 1 - len(edges), 2, min(top, 130), 12).tolist() + [(32 if C > 1 else 64) * C + 1]
     items = [gen.kuka_lq(14, 7, int(n), 3500 + i) for i, n in enumerate(Ns)]
     items[2].Qd[0, 0] = 0.0
     batch = gen.concat_batch(items).astype(np.float32)
@@ -154,8 +156,7 @@ def test_stages_of_a_ragged_batch(B, top, C):
     sch, stats, ws = s.alloc_schur(lt), s.alloc_stats(lt.nb), s.alloc_workspace(lt)
     s.form(lt, sch)
     o = make_opts()
-    sh = s.pcg_shape(lt, sch, o, N=top)
-    assert sh["C"] == C and sh["clusters"] < B, sh
+    assert s.pcg_shape(lt, sch, o, N=top)["C"] == C
     lam = torch.full((lt.total, 14), 0.25, device="cuda")
     s.pcg_solve(lt, sch, lam, o, stats, ws, N=top)
     torch.cuda.synchronize()
