@@ -144,7 +144,7 @@ def measured_peaks():
 def cluster_kernel_sha() -> str:
     """sha256[:16] over the sources the cluster PCG kernel is compiled from."""
     h = hashlib.sha256()
-    for f in ("pcg.cu", "pcg_rows.cuh", "common.cuh", "launch.cuh"):
+    for f in ("pcg_reg.cu", "pcg_sums.cuh", "pcg_rows.cuh", "common.cuh", "launch.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2309_08079_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -152,7 +152,7 @@ def cluster_kernel_sha() -> str:
 def pcg_traffic_from_profile():
     """DRAM bytes per PCG launch from the committed ncu summary, if it was
     captured from the current kernel source (else None)."""
-    prof = os.path.join(ROOT, "profiles", "pcg_cluster_kernel_N512.md")
+    prof = os.path.join(ROOT, "profiles", "pcg_reg_kernel_N512.md")
     try:
         sha = cluster_kernel_sha()
         txt = open(prof).read()
@@ -173,22 +173,25 @@ def pcg_bytes_per_knot_iter(nx: int, esize: int = 4) -> int:
     return (2 * T + 7 * nx) * esize
 
 
-def latency_roofline(s, lt, sch, opts, iters_mean: float, launch_us: float, rounds: int = 2000) -> dict:
-    """The single-instance PCG kernel against its synchronisation floor: each
-    iteration of Algorithm 1 takes two cluster reductions, each at least the
-    time mpcg_bench_exchange measures for the launch shape the solve uses
-    (the same exchange code with no arithmetic), so the floor is
-    2 x exchange per iteration.  achieved / peak in PCG iterations per second."""
+def latency_roofline(s, lt, sch, opts, iters_mean: float, launch_us: float, rounds: int = 2000,
+                     per_iteration: int = 2) -> dict:
+    """The single-instance PCG kernel against its synchronisation floor: an
+    iteration takes `per_iteration` cluster reductions (two in Algorithm 1 as
+    it stands, one in the float32 nx = 14 kernel's recurrence), each at least
+    the time mpcg_bench_exchange measures for the launch shape the solve uses
+    (a reduction with no arithmetic), so the floor is that many exchanges per
+    iteration.  achieved / peak in PCG iterations per second."""
     sh = s.pcg_shape(lt, sch, opts)
     if sh["form"] != "cluster":
         return {"bound": "n/a", "note": f"kernel form {sh['form']}"}
     x = s.bench_exchange(sh["C"], sh["threads"] // 32, rounds=rounds)
-    floor_ns = 2.0 * x["ns"]
+    floor_ns = per_iteration * x["ns"]
     t_it_ns = launch_us * 1e3 / max(iters_mean, 1.0)
     return {"bound": "sync_latency", "achieved": 1e9 / t_it_ns, "peak": 1e9 / floor_ns,
             "unit": "PCG iterations/s", "frac": floor_ns / t_it_ns,
             "peak_source": f"measured: mpcg_bench_exchange on the solve's launch shape "
-                           f"(C={sh['C']} CTAs x {sh['threads'] // 32} warps), 2 exchanges per iteration",
+                           f"(C={sh['C']} CTAs x {sh['threads'] // 32} warps), "
+                           f"{per_iteration} exchange(s) per iteration",
             "exchange_ns": x["ns"], "exchange_cycles": x["cycles"], "ns_per_iteration": t_it_ns,
             "floor_ns_per_iteration": floor_ns, "shape": sh}
 
@@ -196,7 +199,7 @@ def latency_roofline(s, lt, sch, opts, iters_mean: float, launch_us: float, roun
 def profile_onchip():
     """SMEM-pipe share and barrier-stall share of the cluster kernel from the
     committed ncu summary, when it was taken from the current sources."""
-    prof = os.path.join(ROOT, "profiles", "pcg_cluster_kernel_N512.md")
+    prof = os.path.join(ROOT, "profiles", "pcg_reg_kernel_N512.md")
     try:
         txt = open(prof).read()
         m_sha = re.search(r"cluster kernel sources sha256\[:16\]:\s*([0-9a-f]+)", txt)
@@ -404,10 +407,10 @@ def run_ours(args, rank, world, local_rank):
         hbm, peak_note = 6800.0, "of fallback"
     achieved = alg_bytes / pcg_s / 1e9
     # the kernel's operators stay on chip (registers): what bounds it is the
-    # latency of its two cluster reductions per iteration, measured by the
+    # latency of its cluster reduction per iteration, measured by the
     # exchange microbenchmark on the same launch shape; HBM is secondary
-    roofline = latency_roofline(s, lt, sch, opts, float(np.mean(iters)), pcg_s * 1e6)
-    roofline.update({"traffic": pcg_traffic_from_profile(), "kernel": "pcg_cluster_kernel",
+    roofline = latency_roofline(s, lt, sch, opts, float(np.mean(iters)), pcg_s * 1e6, per_iteration=1)
+    roofline.update({"traffic": pcg_traffic_from_profile(), "kernel": "pcg_reg_kernel",
                      "launch_us": pcg_s * 1e6, "onchip_ncu": profile_onchip(),
                      "hbm": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                              "frac": achieved / hbm, "peak_source": peak_note,
@@ -611,8 +614,9 @@ def run_batched(s, dev, solves):
         runner = tuner.runner(lt, sch, master[0], opts)
 
     # Sync-latency floor of the cluster launches: the clusters keep each
-    # instance's operators on chip, so an instance solved on C CTAs holds C
-    # SMs for at least iterations x 2 exchanges at the latency
+    # instance's operators on chip, so an instance holds the SMs of the CTAs
+    # that its horizon needs (32 knots each; two CTAs of 128 threads share an
+    # SM) for at least iterations x 1 exchange at the latency
     # mpcg_bench_exchange measures on its launch shape; the floor is that
     # SM-time summed over the graph's solves and spread over every SM.
     n_sms = torch.cuda.get_device_properties(dev).multi_processor_count
@@ -630,7 +634,8 @@ def run_batched(s, dev, solves):
             key = (sh["C"], sh["threads"] // 32)
             if key not in xcache:
                 xcache[key] = s.bench_exchange(*key, rounds=1000)["ns"]
-            sm_ns += float(np.sum(iters[idx])) * 2.0 * xcache[key] * sh["C"]
+            need = np.array([min(sh["C"], next(x for x in (1, 2, 3, 4, 6, 8, 12, 16) if 32 * x >= n)) for n in Ns[idx]])
+            sm_ns += float(np.sum(iters[idx] * need)) * xcache[key] / (2.0 if sh["threads"] <= 128 else 1.0)
             shapes.append({"C": sh["C"], "threads": sh["threads"], "instances": int(len(idx))})
         if not shapes:
             return None, None, other
@@ -678,7 +683,7 @@ def run_batched(s, dev, solves):
             floor, shapes, other = None, None, []
         if floor is not None:
             roof = {"bound": "sync_latency", "frac": floor / gms, "floor_ms": floor, "shapes": shapes,
-                    "note": "SM-time of every cluster-launched instance at 2 measured exchanges "
+                    "note": "SM-time of every cluster-launched instance at 1 measured exchange "
                             "(mpcg_bench_exchange, its launch shape) per PCG iteration, spread over all "
                             "SMs, over the graph time (formation and recovery included); operators stay "
                             "on chip",
@@ -782,13 +787,13 @@ def run_backward(s, dev, reps=5):
     it_b = read_stats(bst)["iters"].astype(np.float64)
     alg = float(np.sum(it_f + it_b)) * c["N"] * pcg_bytes_per_knot_iter(c["nx"])
     # the batch's clusters keep their operators on chip: the floor is the
-    # reductions' latency, 2 exchanges per iteration on each cluster, the
+    # reductions' latency, one exchange per iteration on each cluster, the
     # instances spread over the co-resident clusters
     sh = s.pcg_shape(lt, sch, opts)
     lat = None
     if sh["form"] == "cluster":
         x = s.bench_exchange(sh["C"], sh["threads"] // 32, rounds=1000)
-        lat = float(np.sum(it_f + it_b)) * 2.0 * x["ns"] * 1e-6 / max(1, min(sh["clusters"], c["B"]))
+        lat = float(np.sum(it_f + it_b)) * x["ns"] * 1e-6 / max(1, min(sh["clusters"], c["B"]))
     # gradient of instance 0 against the oracle's analytic gradient
     it0 = batch.items[0].astype(np.float64)
     l0, x0, u0 = oracle.kkt_solve(it0)
@@ -818,7 +823,7 @@ def run_backward(s, dev, reps=5):
             "speedup_vs_loop": t_loop / (f + bw), "converged": ok, "grad_relerr_vs_oracle": gerr,
             "pcg_roofline": {"bound": "sync_latency", "frac": (lat / (f + bw)) if lat else None,
                              "floor_ms": lat, "shape": sh,
-                             "note": "forward + adjoint PCG iterations x 2 measured exchanges, spread over the "
+                             "note": "forward + adjoint PCG iterations x 1 measured exchange, spread over the "
                                      "co-resident clusters, over fwd + bwd time",
                              "hbm_equivalent_frac": alg / ((f + bw) / 1e3) / 1e9 / hbm, "peak_source": note}}
 
@@ -887,7 +892,8 @@ def run_sweep(s, dev, reps, flush):
         pus = np.array(pcg.ms()) * 1e3
         it = st["iters"].astype(np.float64)
         ach = float(np.mean(it)) * N * pcg_bytes_per_knot_iter(c["nx"]) / (np.mean(pus) * 1e-6) / 1e9
-        rl = latency_roofline(s, lt, sch, opts, float(np.mean(it)), float(np.median(pus)), rounds=1000)
+        rl = latency_roofline(s, lt, sch, opts, float(np.mean(it)), float(np.median(pus)), rounds=1000,
+                              per_iteration=1)
         rl["hbm"] = {"achieved_gbs": ach, "frac": ach / hbm, "peak_source": note}
         out[str(N)] = {"us_per_solve": pct(us), "pcg_us": float(np.median(pus)),
                        "iters": pct(it), "converged": bool(np.all(st["status"] == 0)), "roofline": rl}

@@ -122,16 +122,18 @@ typedef struct {
     int cluster;   /* CTAs per instance (1..16); 0 = automatic */
     int mode;      /* PCG kernel: 0 automatic; 1 a thread-block cluster per instance
                       (matrices held on chip, in registers for float32 nx = 14;
-                      the automatic choice whenever the horizon fits); 2 one CTA
+                      the automatic choice whenever the horizon fits, but for
+                      float32 nx = 36 beyond 8 knots per CTA); 2 one CTA
                       per instance reading the blocks from L2 (many instances at
                       once, any horizon that fits shared memory; the automatic
-                      choice beyond a cluster); 3 one CTA per instance streaming
+                      choice beyond the others); 3 one CTA per instance streaming
                       each knot's blocks through shared memory as TMA tiles
-                      (even nx and 16-byte-aligned block arrays, else as 2);
+                      (even nx and 16-byte-aligned block arrays, else as 2; the
+                      automatic choice runs float32 nx = 36 so with as many CTAs
+                      per instance as pay);
                       4 a cluster per instance with the matrices staged in
                       shared memory, 8 lanes x 2 rows per knot and up to 64
-                      knots per CTA (nx <= 16): half the SMs per instance of
-                      mode 1, for throughput */
+                      knots per CTA (nx <= 16) */
     /* Batched PCG only: solve just the instances listed (a DEVICE int
        array of n_instances distinct indices into the batch); NULL solves
        all B.  With a list, dims.N may be the largest horizon among the
@@ -232,14 +234,17 @@ int mpcg_form_schur(mpcg_handle *h, mpcg_dims dims, const mpcg_lq *lq, mpcg_schu
 int mpcg_form_precon(mpcg_handle *h, mpcg_dims dims, mpcg_schur *schur, void *stream);
 
 /*
- * mpcg_form_schur followed by mpcg_form_precon in one launch (nx <= 16): one
- * warp per knot k forms block row k of S+, gamma_k and Pd[k]; a CTA takes
- * consecutive knots and one extra warp that forms D_{k+1} and phi_k of the
- * knot after its last, so that Po[k] = -Pd[k+1] phi_k Pd[k] is formed from
+ * mpcg_form_schur followed by mpcg_form_precon, in one launch for nx <= 16
+ * with diagonal costs and, in float32, for (nx, nu) = (14, 7) and (36, 12)
+ * (the first with dense cost blocks too; the second writes schur->Sdp and Pdp
+ * as well when given).  A CTA takes
+ * consecutive knots and forms D_{k+1} and phi_k of the knot after its last
+ * as well, so that Po[k] = -Pd[k+1] phi_k Pd[k] is formed from
  * shared memory.  The outputs are those of the two calls up to rounding
  * (the same formulas in the same order; ~1 ulp per entry where the compiler
  * contracts other multiply-adds).
- * Dense cost blocks (lq->Q) and nx > 16 take the two calls' route.  Same
+ * Other shapes with dense cost blocks (lq->Q) or nx > 16 take the two calls'
+ * route.  Same
  * arguments and errors as mpcg_form_schur; schur->Pd and schur->Po are
  * required.
  */
@@ -480,8 +485,8 @@ int mpcg_selftest_drain(mpcg_handle *h, int mode, double limit_s, int *status,
  * the latency floor that the single-instance solve is measured against).
  * One cluster of C CTAs x W warps (1 <= C, W <= 16; else MPCG_EINVAL) runs
  * `rounds` (1..10^6) rounds of the two exchanges of a PCG iteration
- * (Algorithm 1's two reductions) exactly as the float32 cluster kernel
- * performs them -- halo pushes from the boundary warps, a shuffle sum per
+ * (Algorithm 1's two reductions) exactly as the general cluster kernel in
+ * float32 performs them (the nx = 14 kernel takes one per iteration) -- halo pushes from the boundary warps, a shuffle sum per
  * warp, warp 0 combining the warp sums and pushing the CTA sum into every
  * CTA with st.async, a bounded mbarrier wait, a CTA barrier and the sum of
  * the C partials -- with no other arithmetic.  DEVICE outputs: out[0] =

@@ -181,11 +181,16 @@ int choose_pcg_tile(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_schur 
     // Measured, 1 / 2 / 4 / 8 / 16 CTAs, ms: 160 instances of 64..256 knots
     // 238 / 152 / 136 / 208 / 336; 24 of 64..256 219 / 121 / 59 / 45 / 65; 300 of
     // 64..128 119 / 108 / 130 / 236 / 186; 60 of 20..60 20.7 / 14.0 / 11.0 / 10.6 / 12.6.
-    if (clusters && L.nxc == 36) {
+    // A batch that fills the GPU with a CTA each (packed blocks, no exchanges) is
+    // left to that: from 1.5 waves (220 of 64..256 209 ms against 252 with a CTA
+    // each, but 260 of 200..256 470 against 437, 1024 of 64..256 975 against 800),
+    // short horizons from 0.45 (60 of 20..60 above, but 90 of 60..64 25.3 against
+    // 22.6, 160 of 40..64 24.6 against 21.7, 152 of 30..40 13.0 against 9.9).
+    if (clusters && L.nxc == 36 && B <= (d.N > 64 ? 1.5 : 0.45) * n) {
         double cost[5], best = 0.0;
         int levels = 0;
         for (int C = 1; C <= kMaxCluster && (C == 1 || d.N >= 8 * C); C *= 2) {
-            const int m = shape(C);
+            const int m = std::min(shape(C), h->sms / C);  // CTAs that share an SM are no faster
             const double t = m < 1 ? 1e30 : (6.0 + 0.35 * L.kpc_max) * std::max(1.0, 0.6 * B / m);
             cost[levels++] = t;
             if (C == 1 || t < best) best = t;

@@ -207,8 +207,9 @@ class Solver:
                 "threads": shape[3], "depth": shape[4], "packed": bool(shape[5])}
 
     def bench_exchange(self, C_: int, W: int, rounds: int = 2000, stream=None) -> dict:
-        """Latency of one cluster reduction of the PCG kernels (both of
-        Algorithm 1's per-iteration reductions take one) on a C_ x W launch
+        """Latency of one cluster reduction of the PCG kernels (one per
+        iteration in those of float32 nx = 14, nx = 36 and float64 nx = 14, two
+        in the general one) on a C_ x W launch
         shape, from mpcg_bench_exchange: cycles and nanoseconds per
         exchange."""
         out = torch.zeros(3, dtype=torch.int64, device=self.device)

@@ -34,7 +34,7 @@ def _formed(Ns, seed, flagged=None):
 # of one knot each, and with unequal shares; more instances than clusters
 # (without a workspace too), and fewer
 @pytest.mark.parametrize("Ns,C", [
-    ([16, 9, 1, 2, 13, 16, 15] * 20, 2), ([33, 1, 3, 4, 5, 17, 40] * 6, 4),
+    ([70, 9, 1, 2, 13, 69, 15] * 20, 2), ([33, 1, 3, 4, 5, 17, 40] * 6, 4),
     ([67, 7, 8, 9, 1, 70, 31, 33] * 3, 8), ([130, 15, 16, 17, 5, 1, 131, 150, 2, 33], 16), ([257], 16)])
 @pytest.mark.parametrize("queue", [True, False])
 def test_solutions_at_every_cluster_size(Ns, C, queue):
