@@ -44,8 +44,8 @@
 // long as alone.  Up to 64 knots one CTA of 256 threads holds an instance, without
 // exchanges (256 of 60..64 knots 1.07 against 1.22 ms); longer ones are better in
 // CTAs of 32 knots, which overlap (64 of 128 knots 1.17 against 1.24 with 64).
-// Former form -> this one: 256 instances of 32..512 knots 19.9 -> 16.4 ms, 256 of
-// 60..64 1.48 -> 1.07, 150 of 100..250 5.85 -> 4.85, 17 of 505..512 3.97 -> 3.66.
+// Former form -> this one: 256 instances of 32..512 knots 19.9 -> 16.5 ms, 256 of
+// 60..64 1.48 -> 1.05, 150 of 100..250 5.85 -> 4.9, 17 of 505..512 3.97 -> 3.8.
 //
 // Choice of the form: PS pays once the other would need a second wave; that
 // depends on the horizons, which the host does not know.  Between one and four
@@ -92,7 +92,11 @@ namespace mpcg {
 namespace {
 
 constexpr int NXR = 14;   // block size
-constexpr int VSR = 16;   // floats per knot slot of a shared vector
+// Floats per knot slot of a shared vector (16 used): 20 puts the 16-byte words
+// of eight consecutive knots, one load of the PS form, on distinct banks (16: 22 %
+// of its shared-memory wavefronts were conflicts; 64 instances of 128 knots 1.21
+// against 1.12 ms, 256 of 60..64 1.08 against 1.05).
+constexpr int VSR = 20;
 constexpr int CMAX = 16;  // CTAs per cluster
 constexpr int WMAX = 8;   // warps per CTA
 constexpr int LEVELS = 5; // group sizes C, C/2, ..., C/16
@@ -123,7 +127,7 @@ struct RegLayout {
     }
 };
 
-// R rows of one block row times the halo'd vector: the knot's three 16-float
+// R rows of one block row times the halo'd vector: the knot's three
 // vector slots are read once for all of them.
 template <int R>
 __device__ __forceinline__ void rowdot(const float (&d)[R][NXR], const float (&l)[R][NXR], const float (&u)[R][NXR],
@@ -379,7 +383,7 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
         // the warps holding the first and last knot slot (warp-uniform)
         const bool warp_left = has_left && warp == 0;
         const bool warp_right = has_right && warp == ((KPC - 1) * LPR) / 32;
-        const uint32_t halo_bytes = (uint32_t)((PS ? VSR : NXR) * sizeof(float)) * ((has_left ? 1u : 0u) + (has_right ? 1u : 0u));
+        const uint32_t halo_bytes = (uint32_t)((PS ? 16 : NXR) * sizeof(float)) * ((has_left ? 1u : 0u) + (has_right ? 1u : 0u));
         const bool rows = R * li < NXR;               // (R = 2) lane 7 of a knot holds none
         const bool rv = active_knot && rows, st = slot_knot && rows;
         const int own = (kl + 1) * VSR + R * li;      // this thread's rows in a shared vector
