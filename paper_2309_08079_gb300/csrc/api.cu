@@ -96,8 +96,8 @@ int choose_pcg_cta(mpcg_handle *h, const mpcg_dims &d, int B, PcgLaunch &L) {
     return MPCG_OK;
 }
 
-// Launch shape of the tiled kernel, one CTA per instance or (`clusters`) more; MPCG_EUNSUPPORTED when
-// its TMA tiles cannot be used (odd nx: a block is not a 16-byte multiple;
+// Launch shape of the tiled kernel, one CTA per instance or (`clusters`) more;
+// MPCG_EUNSUPPORTED when its TMA tiles cannot be used (odd nx: a block is not a 16-byte multiple;
 // a block array not 16-byte aligned; nx > 64) or nothing fits in shared
 // memory.  Each knot stream's steps are bound by their own instruction
 // latency more than by the copies (measured: time falls with the stream
@@ -300,7 +300,8 @@ int choose_pcg_cluster(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opt
     // float32 nx = 36 and float64 nx = 14 while the operators stay on chip and
     // every instance has its own cluster (pcg_split.cu), as many CTAs as that
     // leaves (the products of a CTA shrink with its knots: N = 64 1.90 us per
-    // iteration at 4 knots per CTA, N = 128 2.94 at 8); float64 accumulation of float32 sums stays with the general form
+    // iteration at 4 knots per CTA, N = 128 2.94 at 8); float64 accumulation of
+    // float32 sums stays with the general form
     if (!wide && !L.dot) {
         const int fixed = o && o->cluster > 0 ? std::min(o->cluster, d.N) : 0;
         for (int C = fixed ? fixed : std::min(kMaxCluster, d.N); C >= (fixed ? fixed : 1) && C <= kMaxCluster; --C) {
@@ -321,9 +322,8 @@ int choose_pcg_cluster(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opt
     else return MPCG_EUNSUPPORTED;
     const int kpc_cap = kMaxThreads / L.lpk;  // knot slots per CTA
     // A single instance runs fastest at the largest cluster (each lane's rows
-    // per iteration grow with the knots per CTA: FP64 N = 128 4.9 ms at 16
-    // CTAs against 13.0 ms at 4; nx = 36 N = 64 2.0 against 4.3 ms).  Batches
-    // fill the CTAs (the autotuner tries the other packings).
+    // per iteration grow with the knots per CTA: FP64 nx = 14 N = 128 4.9 ms at
+    // 16 CTAs against 13.0 at 4, in this form).  Batches fill the CTAs (the autotuner tries the other packings).
     const int kpc_pref = B > 1 ? kpc_cap : 1;
     int C = (o && o->cluster > 0) ? o->cluster : std::min(kMaxCluster, ceil_div(d.N, kpc_pref));
     if (!(o && o->cluster > 0)) C = std::max(C, ceil_div(d.N, kpc_cap));
@@ -352,10 +352,10 @@ int choose_pcg_cluster(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opt
 }
 
 // Kernel choice (mode 0): a cluster per instance whenever the horizon fits
-// one (fastest for single solves; for float32 nx = 14 batches the
-// register-resident clusters match the tiled kernel), the tiled kernel for
-// larger batches of other shapes, one CTA per instance reading L2 for
-// horizons beyond both.
+// one (fastest for single solves, and at float32 nx = 14 for batches: 256
+// instances of 32..512 knots 16.5 ms against 30 tiled), the tiled kernel for
+// float32 nx = 36 beyond the lane-per-row form and for larger batches of
+// other shapes, one CTA per instance reading L2 for horizons beyond both.
 template <typename T>
 int choose_pcg(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opts *o, const mpcg_schur *s,
                PcgLaunch &L) {

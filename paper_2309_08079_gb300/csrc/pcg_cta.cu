@@ -1,7 +1,8 @@
 // One-CTA-per-instance PCG kernels (batched throughput forms of Algorithm 1):
 // pcg_cta_kernel reads the blocks of S+ and Phi^-1 from L2 each iteration;
 // pcg_tile_kernel streams them through shared memory with TMA bulk copies,
-// one pipeline per knot stream.
+// one pipeline per knot stream (float32 nx = 36 also with a cluster of CTAs per
+// instance).
 #include <type_traits>
 
 #include "pcg_sums.cuh"
@@ -256,8 +257,8 @@ __global__ void __launch_bounds__(512, 1) pcg_cta_kernel(const PcgParams<T> P) {
 }
 
 // ---------------------------------------------------------------------------
-// Tiled CTA-per-instance PCG (batched throughput form, opts.mode = 3).
-// One CTA owns an instance: r, p and a work vector w (S p, then Phi^-1 r)
+// Tiled PCG (batched throughput form, opts.mode = 3).
+// One CTA owns an instance (or, in a cluster, its share of the knots): r, p and a work vector w (S p, then Phi^-1 r)
 // live in shared memory for every knot, lambda in global memory.  The
 // CTA's lanes form knot streams of LPK lanes (two streams per warp when
 // LPK = 16); stream s owns a contiguous range of knots and walks it once per
