@@ -139,7 +139,9 @@ typedef struct {
        all B.  With a list, dims.N may be the largest horizon among the
        listed instances, which sizes the launch.  An entry >= B is skipped
        (nothing read or written for it, no stats); a negative entry ends
-       the list for the CTA or cluster that draws it. */
+       the list for the CTA or cluster that draws it, so a list may be
+       padded at its tail with negative entries.  (A launch that goes over
+       the list once per class of horizons ends that pass.) */
     const int *instances;
     int n_instances;
     /* Preconditioner applied by the PCG: 0 the symmetric stair Phi^-1 of

@@ -614,21 +614,25 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
         return gave_up;
     };
 
-    int served = 0, level = 0;
+    int served = 0, level = 0, ended = 0;
     bool failed = false;
     for (;;) {
         if (tid == 0 && rank == 0) {
             int b;
             for (;;) {
                 const int t = P.queue ? atomicAdd(P.queue + level, 1) : (int)(blockIdx.x / C + served * (gridDim.x / C));
-                if (t >= P.n_tickets) {
-                    b = -1;
-                    if (!P.split || level == 3) break;
+                const bool end = t >= P.n_tickets;
+                b = end ? -1 : P.inst_list ? P.inst_list[t] : t;
+                if (!P.split) break;
+                if (b < 0) {
+                    // A negative entry ends this pass over the list for one CTA,
+                    // so a cluster, in the place of C CTAs, takes C of them.
+                    if (!end && ++ended < C) continue;
+                    ended = 0;
+                    if (level == 3) break;
                     ++level;  // the next quarter of horizons
                     continue;
                 }
-                b = P.inst_list ? P.inst_list[t] : t;
-                if (!P.split || b < 0) break;
                 int k0, Nb;
                 P.bv.range(b, k0, Nb);
                 if (min(3, max(0, 3 - (4 * Nb - 1) / P.n_long)) == level) break;

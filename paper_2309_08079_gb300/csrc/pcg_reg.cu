@@ -315,10 +315,7 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
                                       : (int)(cluster_id_x() + (uint32_t)served++ * num_clusters_x());
                 if (t >= P.n_tickets) break;
                 b = P.inst_list ? P.inst_list[t] : t;
-                if (b < 0) {  // ends the list for this group
-                    b = -2;
-                    break;
-                }
+                if (b < 0) break;  // ends this pass over the list for the group, as its end does
                 int k0, Nb;
                 P.bv.range(b, k0, Nb);
                 if (Nb <= P.n_above || Nb > P.n_upto) {  // another stage's instance
@@ -355,7 +352,7 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
         }
         mail_phase ^= 1u;
         if (__syncthreads_or(fail)) timed_out = true;
-        const int b = timed_out ? -2 : mail[level];
+        const int b = mail[level];
         if (timed_out) {
             if (tid == 0) cluster_drain(rank, C, smem_u32(s_abort), mbS, DRAIN_LIMIT_NS, DRAIN_GRACE_NS);
             __syncthreads();
@@ -363,7 +360,7 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
             return;
         }
         if (b < 0) {
-            if (b == -2 || !P.split || G == 1) break;
+            if (!P.split || G == 1) break;
             G /= 2;  // this class is exhausted: two groups from here on
             if (rank - g0 >= G) g0 += G;
             ++level;

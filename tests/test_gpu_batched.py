@@ -191,3 +191,43 @@ def test_tiled_kernel_at_its_largest_horizon(nx, nu, lo_bound, hi_bound):
         with pytest.raises(MPCGError) as ei:
             s.pcg_shape(probe, psch, o, N=Nmax + 1)
         assert ei.value.code == MPCG_EUNSUPPORTED
+
+
+@pytest.mark.parametrize("nx,nu,mode,valid,pad", [(14, 7, 0, 20, 108), (14, 7, 0, 60, 400), (36, 12, 0, 20, 200),
+                                                  (36, 12, 3, 24, 400), (14, 7, 3, 24, 700)])
+def test_list_padded_with_negative_entries(nx, nu, mode, valid, pad):
+    """A list padded at its tail with at least as many negative entries as the
+    launch has clusters (CTAs): every listed instance is solved (the exact
+    solution of the S+ that was formed, at the usual bar), whichever class of
+    horizons it belongs to, and the others are left alone."""
+    import scipy.sparse.linalg as spla
+    import torch
+    from paper_2309_08079_gb300.solver import LQTensors, make_opts, read_stats
+    s = solver()
+    top = 512 if nx == 14 else 200
+    Ns = gen.batch_horizons(valid + 4, 8, top, 21)
+    Ns[:6] = [top, top // 2, top // 4, top // 8, 9, 1]
+    batch = gen.kuka_batch(nx, nu, Ns, 3700).astype(np.float32)
+    listed = np.random.default_rng(5).permutation(valid + 4)[:valid]
+    entries = np.concatenate([listed, np.full(pad, -1)])
+    inst = torch.tensor(entries, dtype=torch.int32, device="cuda")
+    lt = LQTensors.from_batch(batch)
+    sch = s.alloc_schur(lt)
+    s.form(lt, sch)
+    lam = torch.full((lt.total, nx), 0.25, device="cuda")
+    stats = s.alloc_stats(lt.nb)
+    stats.fill_(0xFF)
+    o = make_opts(mode=mode, instances=inst)
+    assert s.pcg_shape(lt, sch, o, N=top)["clusters"] <= pad
+    s.pcg_solve(lt, sch, lam, o, stats, s.alloc_workspace(lt), N=top)
+    torch.cuda.synchronize()
+    st = read_stats(stats)
+    lam, Sd, So, g = (t.cpu().double().numpy() for t in (lam, sch.Sd, sch.So, sch.gamma))
+    for b in range(valid + 4):
+        k0, k1 = batch.knot_off[b], batch.knot_off[b + 1]
+        if b not in listed:
+            assert st["status"][b] == -1 and np.all(lam[k0:k1] == 0.25), b
+            continue
+        S = oracle.block_tridiag_sparse(Sd[k0:k1], So[k0 - b:k1 - b - 1]).tocsc()
+        ref = spla.spsolve(S, -g[k0:k1].ravel()).reshape(-1, nx)
+        assert st["status"][b] == 0 and oracle.relerr(lam[k0:k1], ref) < TOL_F32, (b, Ns[b], st[b])
