@@ -654,8 +654,8 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
             float alpha = __fdividef(etan, ups);
             const bool done = !(fabsf(etan) <= 3.402823466e38f && rr <= 3.402823466e38f) ||
                               (mode1 ? etan < tol_t : rr <= tol_t) || it >= max_iter;
-            // the identity cancelled, or S+ is not positive on p (or not finite)
-            const bool direct = !(ups > 0.0625f * S.del && ups <= 3.402823466e38f);
+            // the identity cancelled, or S+ may not be positive on p (or not finite)
+            const bool direct = !(ups > 0.f && ups > 0.0625f * fabsf(S.del) && ups <= 3.402823466e38f);
             // p = r~ + beta p, S p = S r~ + beta S p_old, lambda += alpha p,
             // r -= alpha S p; the halo copies of p and r alike
             auto next_p = [&]() {

@@ -426,8 +426,8 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
                 eta = S.eta;
                 rr = S.rr;
                 const bool done = !(fabs(etan) <= big && rr <= big) || (mode1 ? etan < tol_t : rr <= tol_t) || it >= max_iter;
-                // the identity cancelled, or S+ is not positive on p (or not finite)
-                const bool direct = !(ups > T(0.0625) * S.del && ups <= big);
+                // the identity cancelled, or S+ may not be positive on p (or not finite)
+                const bool direct = !(ups > T(0) && ups > T(0.0625) * fabs(S.del) && ups <= big);
                 if (lane == 0) {
                     scal[0] = alpha;
                     scal[1] = beta;

@@ -180,3 +180,53 @@ def test_stages_of_a_ragged_batch(B, top, C):
         S = oracle.block_tridiag_sparse(Sd[k0:k1], So[k0 - b:k1 - b - 1]).tocsc()
         ref = spla.spsolve(S, -gam[k0:k1].ravel()).reshape(n, 14)
         assert st["status"][b] == 0 and oracle.relerr(lam[k0:k1], ref) < TOL_F32, (b, n)
+
+
+@pytest.mark.parametrize("nx,nu,N,seed,scale,shift,precon", [
+    (14, 7, 6, 9, 2.0, 0.42199, 2), (14, 7, 40, 0, 3.0, 0.42199, 2), (36, 12, 6, 19, 3.0, 0.39835, 2),
+    (14, 7, 16, 2, 1.0, 0.05, 0), (36, 12, 16, 0, 1.0, 0.05, 0)])
+@pytest.mark.parametrize("dtype", ["float32", "float64"])
+def test_breakdown_after_the_first_iteration(nx, nu, N, seed, scale, shift, precon, dtype):
+    """S+ made indefinite so that p^T S p turns negative in a later iteration, by
+    a small share of |r~^T S r~| where the preconditioner is not symmetric:
+    MPCG_BREAKDOWN in the iteration of Algorithm 1.  (Smallest |p^T S p| over
+    the sum of the identity's terms: 8e-3, against 1e-6 of rounding.)"""
+    import torch
+    from paper_2309_08079_gb300.solver import LQTensors, make_opts, read_stats
+    t = getattr(torch, dtype)
+    lq = gen.kuka_lq(nx, nu, N, seed)
+    Sd, So, g = oracle.schur_blocks(lq)
+    Pd, Po = oracle.precon_blocks(Sd, So)
+    Po = scale * Po
+    rng = np.random.default_rng(seed)
+    for k in range(N):
+        if rng.random() < 0.5:
+            Sd[k] -= shift * np.trace(Sd[k]) / nx * np.eye(nx)
+    S, P = oracle.block_tridiag_sparse(Sd, So), oracle.block_tridiag_sparse(Pd, Po).toarray()
+    if precon == 2:  # even block rows keep their diagonal block alone
+        for k in range(0, N, 2):
+            rows = slice(k * nx, (k + 1) * nx)
+            P[rows, :k * nx] = 0.0
+            P[rows, (k + 1) * nx:] = 0.0
+    r = -g.ravel()
+    z = P @ r
+    p, eta = z.copy(), r @ z
+    for it in range(1, 10):
+        Sp = S @ p
+        if not p @ Sp > 0:
+            break
+        r = r - eta / (p @ Sp) * Sp
+        z = P @ r
+        eta, p = r @ z, z + (r @ z) / eta * p
+    assert p @ Sp < 0 and it >= 2
+    s = solver()
+    lt = LQTensors.from_numpy(lq, dtype=t)
+    sch = s.alloc_schur(lt)
+    s.form(lt, sch)
+    for dst, src in ((sch.Sd, Sd), (sch.So, So), (sch.Pd, Pd), (sch.Po, Po), (sch.gamma, g)):
+        dst.copy_(torch.as_tensor(src))
+    for C in (1 if N <= 8 else 4, 16):
+        lam = torch.zeros(N, nx, dtype=t, device="cuda")
+        st = read_stats(s.pcg_solve(lt, sch, lam, make_opts(mode=1, cluster=C, precon=precon)))
+        assert st["status"][0] == 2 and st["iters"][0] == it, (C, it, st)
+        assert torch.isfinite(lam).all()
