@@ -646,10 +646,10 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
                     get(hsrc + halo_off(2, zpar, 0), ht);
                 }
             }
+            const float etan = AT::to_T(S.eta);
+            const float beta = beta_from(etan, inv_eta, AT::to_T(eta));  // 0 in the first iteration
             eta = S.eta;
             rr = S.rr;
-            const float etan = AT::to_T(S.eta);
-            const float beta = __fmul_rn(etan, inv_eta);  // 0 in the first iteration
             ups = __fmaf_rn(beta, __fmaf_rn(beta, ups, S.eps + S.eps), S.del);
             float alpha = __fdividef(etan, ups);
             const bool done = !(fabsf(etan) <= 3.402823466e38f && rr <= 3.402823466e38f) ||

@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
                 // ---- alpha, beta and the exit tests, in T from the extended sums ---------
                 const Sums S = collect(1u);
                 const T etan = AT::to_T(S.eta);
-                const T beta = etan * inv_eta;  // 0 in the first iteration
+                const T beta = beta_from(etan, inv_eta, AT::to_T(eta));  // 0 in the first iteration
                 ups = fma_rn(beta, fma_rn(beta, ups, S.eps + S.eps), S.del);
                 const T alpha = quot(etan, ups);
                 eta = S.eta;

@@ -37,6 +37,19 @@ __device__ __forceinline__ void load_pair(const double *p, double &a, double &b)
     b = v.y;
 }
 
+// beta = eta / eta_old, with the reciprocal inv of eta_old taken ahead of the
+// reduction that brings eta; the quotient itself where the reciprocal overflows
+// (eta_old subnormal).  In double one correction step takes the product to
+// the rounded quotient; in float the product is as close as __fdividef.
+__device__ __forceinline__ float beta_from(float eta, float inv, float eta_old) {
+    return fabsf(inv) <= 3.402823466e38f ? __fmul_rn(eta, inv) : __fdiv_rn(eta, eta_old);
+}
+__device__ __forceinline__ double beta_from(double eta, double inv, double eta_old) {
+    if (!(fabs(inv) <= 1.7976931348623157e308)) return eta / eta_old;
+    const double b = __dmul_rn(eta, inv);
+    return __fma_rn(__fma_rn(-b, eta_old, eta), inv, b);
+}
+
 // Every lane of a warp waits (bounded) for the phase of `parity`; true in all
 // lanes if any of them gave up.
 __device__ __forceinline__ bool warp_wait(uint32_t mbar, uint32_t parity, const volatile int *abort_flag) {

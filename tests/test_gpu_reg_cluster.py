@@ -230,3 +230,30 @@ def test_breakdown_after_the_first_iteration(nx, nu, N, seed, scale, shift, prec
         st = read_stats(s.pcg_solve(lt, sch, lam, make_opts(mode=1, cluster=C, precon=precon)))
         assert st["status"][0] == 2 and st["iters"][0] == it, (C, it, st)
         assert torch.isfinite(lam).all()
+
+
+@pytest.mark.parametrize("nx,nu,dtype,scale,small", [(14, 7, "float32", 85, 20), (36, 12, "float32", 85, 20),
+                                                     (14, 7, "float64", 900, 60)])
+def test_small_scale(nx, nu, dtype, scale, small):
+    """S+ times 2^scale, Phi^-1 as much smaller, gamma 2^-small: r^T r~ and p^T S p
+    leave the normal range before the solve ends (no vector does), and 1 / (r^T
+    r~) overflows.  As the unscaled problem does, it converges, and the
+    residual meets the tolerance to a tenth."""
+    import torch
+    from paper_2309_08079_gb300.solver import LQTensors, make_opts, read_stats
+    t = getattr(torch, dtype)
+    N, tol = 64, 1e-3 if dtype == "float32" else 1e-6
+    s = solver()
+    lt = LQTensors.from_numpy(gen.kuka_lq(nx, nu, N, 31).astype(dtype), dtype=t)
+    sch = s.alloc_schur(lt)
+    s.form(lt, sch)
+    Sd, So, g = (x.cpu().double().numpy() for x in (sch.Sd, sch.So, sch.gamma))
+    for x, e in ((sch.Sd, scale), (sch.So, scale), (sch.Pd, -scale), (sch.Po, -scale), (sch.gamma, -small)):
+        x.mul_(2.0 ** e)
+    for C in (2 if nx == 14 else 8, 16):
+        lam = torch.zeros(N, nx, dtype=t, device="cuda")
+        st = read_stats(s.pcg_solve(lt, sch, lam, make_opts(mode=1, cluster=C, tol=tol)))
+        assert st["status"][0] == 0 and 0 < st["eta"][0] < (2.0 ** -128 if dtype == "float32" else 2.0 ** -1024), st
+        y = np.ldexp(lam.cpu().double().numpy().ravel(), scale + small)
+        res = oracle.block_tridiag_sparse(Sd, So) @ y + g.ravel()
+        assert np.linalg.norm(res) < 1.1 * tol * np.linalg.norm(g)
