@@ -168,7 +168,9 @@ typedef struct {
        0 float pairs ("double-float": exact products by FMA, TwoSum
        additions, ~44 significant bits; the default), 1 float64 (products
        and every partial sum in FP64 instructions; slower on GB300, whose
-       FP64 pipe is a small fraction of its FP32 rate).  1 runs in the
+       FP64 pipe is a small fraction of its FP32 rate).  The kernels with one
+       reduction per iteration hold the value of p^T S p that they carry in the
+       same way.  1 runs in the
        cluster kernel and in the tiled kernel for nx = 14 and 36; the L2
        CTA kernel (mode 2) and other tiled shapes return
        MPCG_EUNSUPPORTED.  float64 always accumulates in float64.  Other

@@ -10,17 +10,18 @@
 // so alpha needs only sums that are known once r~ and S r~ are: one reduction
 // of (r^T r~, ||r||^2, r~^T S r~, r~^T S p_old) serves both scalars.  The
 // identity uses only the symmetry of S+ (not orthogonality of the residuals,
-// nor symmetry of Phi^-1), and S p = S r~ + beta S p_old takes S p_old from a
-// fresh product of the stored p each iteration, so no error is carried from
-// one iteration to the next: emulated in float32 on the Kuka-shaped problems
+// nor symmetry of Phi^-1).  S p = S r~ + beta S p_old takes S p_old from a
+// fresh product of the stored p each iteration; p_old^T S p_old is carried, in
+// float pairs, with most of it taken anew in each iteration (curvature in
+// pcg_sums.cuh).  Emulated in float32 on the Kuka-shaped problems
 // (N = 32..512, cold and warm), iteration counts equal Algorithm 1's and
 // lambda differs from it by what another summation order changes (1e-6 warm).
 // The Chronopoulos-Gear form, which carries S p by recurrence, is 3 to 10
 // times further off.  The price is a third product, 84 FMAs per lane, which
 // runs while the boundary rows of r~ travel to the neighbour CTAs.  Where the
-// identity cancels (p^T S p below 1/16 of r~^T S r~; 0.29 was the smallest
-// share seen on the emulated problems) the sum p^T S p is taken directly with
-// one more reduction.  Measured on GB300 at fixed iteration counts: 1.75 us
+// identity cancels (p^T S p below about 1/32 of its terms; 0.29 of r~^T S r~ was the
+// smallest share seen on the emulated problems) or too much of the carried
+// error is passed on, the sum p^T S p is taken directly with one more reduction.  Measured on GB300 at fixed iteration counts: 1.75 us
 // per iteration at N = 512 (16 CTAs x 32 knots) and 1.50 at N = 128 (16 x 8)
 // against 2.23 and 1.98 with two reductions.  Of the 1.75 us, by leaving parts
 // out one at a time: the three products 0.2-0.3 each (bound by the shared-
@@ -229,8 +230,8 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
     static_assert(sizeof(A) == 8, "sums travel in pairs of 8 bytes");
     extern __shared__ __align__(16) unsigned char smem[];
     struct Sums {
-        A eta;               // r^T r~
-        float rr, del, eps;  // ||r||^2, r~^T S r~, r~^T S p_old
+        A eta, del, eps;  // r^T r~, r~^T S r~, (r~ + g / 2 p_old)^T S p_old
+        float rr;         // ||r||^2
     };
 
     const int C = (int)cluster_size(), rank = (int)cluster_rank();
@@ -526,8 +527,8 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
             const float xf = AT::to_T(x);
             r.eta = bcast(x, 0);
             r.rr = __shfl_sync(0xffffffffu, xf, 8);
-            r.del = __shfl_sync(0xffffffffu, xf, 16);
-            r.eps = __shfl_sync(0xffffffffu, xf, 24);
+            r.del = bcast(x, 16);
+            r.eps = bcast(x, 24);
             return r;
         };
 
@@ -581,8 +582,8 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
 
         // Scalars of the iteration (alpha, beta, exit tests) are taken in
         // float from the extended sums.
-        A eta = AT::zero();
-        float ups = 0.f, inv_eta = 0.f, rr = 0.f;
+        A eta = AT::zero(), acc = AT::zero();  // acc: p^T S p
+        float inv_eta = 0.f, rr = 0.f, g = 0.f;  // g: the last beta
         int iters = 0;
         bool broke = false;
         int it = 0;
@@ -609,7 +610,10 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
             const A s_eta = dot(r, z);
             A s_rr = sq_sum(r[0], r[1], A{});
             if constexpr (R == 4) s_rr = AT::add(s_rr, sq_sum(r[2], r[3], A{}));
-            const A s_eps = dot(z, s);
+            float w[R];
+#pragma unroll
+            for (int m = 0; m < R; ++m) w[m] = __fmaf_rn(0.5f * g, p[m], z[m]);
+            const A s_eps = dot(w, s);
             if (failed) {
                 timed_out = true;
                 break;
@@ -650,12 +654,12 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
             const float beta = beta_from(etan, inv_eta, AT::to_T(eta));  // 0 in the first iteration
             eta = S.eta;
             rr = S.rr;
-            ups = __fmaf_rn(beta, __fmaf_rn(beta, ups, S.eps + S.eps), S.del);
-            float alpha = __fdividef(etan, ups);
+            const float old = AT::to_T(acc);
+            acc = curvature(S.del, S.eps, acc, beta, g);
+            float ups = AT::to_T(acc), alpha = __fdividef(etan, ups);
             const bool done = !(fabsf(etan) <= 3.402823466e38f && rr <= 3.402823466e38f) ||
                               (mode1 ? etan < tol_t : rr <= tol_t) || it >= max_iter;
-            // the identity cancelled, or S+ may not be positive on p (or not finite)
-            const bool direct = !(ups > 0.f && ups > 0.0625f * fabsf(S.del) && ups <= 3.402823466e38f);
+            const bool direct = doubtful(ups, AT::to_T(S.del), AT::to_T(S.eps), old, beta, g);
             // p = r~ + beta p, S p = S r~ + beta S p_old, lambda += alpha p,
             // r -= alpha S p; the halo copies of p and r alike
             auto next_p = [&]() {
@@ -703,6 +707,7 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
                 if (!direct) apply();
             }
             inv_eta = __fdividef(1.f, etan);
+            g = beta;
             iters = it;
             __syncthreads();
             if (done || direct) {
@@ -715,7 +720,8 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
                 if (done) break;
                 // sum p^T S p itself
                 expect(0u);
-                ups = AT::to_T(exchange(dot(p, s), AT::zero(), AT::zero(), AT::zero()).eta);
+                acc = exchange(dot(p, s), AT::zero(), AT::zero(), AT::zero()).eta;
+                ups = AT::to_T(acc);
                 if (!(ups > 0.f) || !isfinite(ups)) {
                     broke = true;
                     iters = it + 1;

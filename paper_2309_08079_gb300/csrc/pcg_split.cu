@@ -54,8 +54,8 @@ struct SplitLayout {
         vecP = take(vec_bytes);
         vecZ = take(2 * vec_bytes);                  // by parity of the r~ exchange
         halo = take((size_t)2 * 2 * 2 * nx * esz);   // (S r~, S p) x parity x side
-        slot = take(16 * 2 * 2 * SPLIT_CMAX);        // parity x pair of sums x source CTA
-        wpart = take(16 * 2 * SPLIT_WMAX);           // pair x warp
+        slot = take(16 * 2 * 2 * SPLIT_CMAX + 8 * 2 * SPLIT_CMAX);  // parity x pair of sums x source CTA; the fifth: parity x source
+        wpart = take(8 * 5 * SPLIT_WMAX);            // pair x warp; the fifth
         scal = take(48);
         mbar = take(sizeof(uint64_t) * 6);           // R0, R1, Z, T, peers stopped, instance mail
         mail = take(sizeof(int));
@@ -92,9 +92,12 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
     static_assert(!PS || Q == 1, "whole rows");
     constexpr uint32_t R0 = 0, Z = 16, TT = 24, STOP = 32, MAIL = 40;  // mbarriers
     extern __shared__ __align__(16) unsigned char smem[];
+    // float64: p_old^T S p_old as a fifth sum (2 % of the time, an FP64 addition more per
+    // level); float32: carried, with the predicted beta g in eps (the fifth would take 7 %)
+    constexpr bool FIFTH = sizeof(T) == 8;
     struct Sums {
-        A eta;           // r^T r~
-        T rr, del, eps;  // ||r||^2, r~^T S r~, r~^T S p_old
+        A eta, del, eps, old;  // r^T r~, r~^T S r~, (r~ + g / 2 p_old)^T S p_old, (FIFTH) p_old^T S p_old
+        T rr;                  // ||r||^2
     };
     const int C = (int)cluster_size(), rank = (int)cluster_rank();
     const int nthreads = blockDim.x, W = nthreads / 32 - 1;  // row warps
@@ -120,7 +123,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
         for (int m = 0; m < 6; ++m) mbar_init(mb + 8 * m, 8 * m == (int)STOP ? (C > 1 ? C - 1 : 1) : 1);
         *s_abort = 0;
         *s_fail = 0;
-        for (int m = 0; m < 4 * SPLIT_WMAX; ++m) wpart[m] = AT::zero();
+        for (int m = 0; m < 5 * SPLIT_WMAX; ++m) wpart[m] = AT::zero();
         fence_mbar_init();
     }
     cluster_sync_all();  // peers may push only after every mbarrier is initialised
@@ -273,60 +276,82 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
             push(y, (uint32_t)(L.halo + sizeof(T) * halo_off(v, par, 1)), (uint32_t)(L.halo + sizeof(T) * halo_off(v, par, 0)), bar);
         };
 
-        // ---- sums over the cluster of four accumulators per row thread -----------------
-        // A row warp reduces its own by recursive halving (lanes 8u hold sum u),
-        // leaves them and goes on.
-        auto contribute = [&](A v0, A v1, A v2, A v3) {
-            const bool h16 = lane & 16, h8 = lane & 8;
-            const A a = AT::add_tree(h16 ? v2 : v0, AT::shfl_xor(h16 ? v0 : v2, 16));
-            const A c = AT::add_tree(h16 ? v3 : v1, AT::shfl_xor(h16 ? v1 : v3, 16));
-            A x = AT::add_tree(h8 ? c : a, AT::shfl_xor(h8 ? a : c, 8));
+        // ---- sums over the cluster of four (FIFTH: five) accumulators per row thread -----
+        // A row warp reduces its own by recursive halving (lanes 8u hold sum u, lane 4
+        // the fifth), leaves them and goes on.
+        auto contribute = [&](A v0, A v1, A v2, A v3, A v4) {
+            A x;
+            if constexpr (FIFTH) {
+                x = warp_sums5<AT>(v0, v1, v2, v3, v4);
+                if (lane == 4) wpart[4 * SPLIT_WMAX + warp] = x;
+            } else {
+                x = halve<AT>(halve<AT>(v0, v2, 16), halve<AT>(v1, v3, 16), 8);
 #pragma unroll
-            for (int m = 4; m >= 1; m >>= 1) x = AT::add_tree(x, AT::shfl_xor(x, m));
+                for (int m = 4; m >= 1; m >>= 1) x = AT::add_tree(x, AT::shfl_xor(x, m));
+            }
             const int u = lane >> 3;
             if ((lane & 7) == 0) wpart[(u >> 1) * 2 * SPLIT_WMAX + 2 * warp + (u & 1)] = x;
             named_bar_arrive(1, nthreads);
         };
-        // The sums warp adds the warps' (lanes 0-15 the first pair of sums, 16-31
-        // the second), pushes the CTA's to every CTA and adds those of all.
+        // The sums warp adds the warps', pushes the CTA's to every CTA (lanes 0-15 the
+        // first pair of sums, 16-31 the second, 0-15 the fifth) and adds those of all.
         auto collect = [&](uint32_t nh) -> Sums {
             const uint32_t par = xr & 1u, bar = mb + R0 + 8 * par;
             const int c16 = lane & 15, pr = lane >> 4, w8 = lane & 7;
-            const bool h8 = lane & 8;
+            const uint32_t fifth_off = (uint32_t)L.slot + (uint32_t)(16 * 2 * 2 * SPLIT_CMAX + 8 * SPLIT_CMAX * (int)par);
             const uint32_t slot_off = (uint32_t)L.slot + (uint32_t)((((int)par * 2 + pr) * SPLIT_CMAX) * 16);
-            if (C > 1 && lane == 0) mbar_arrive_expect(bar, (uint32_t)C * 32u + nh * halo_bytes);
+            if (C > 1 && lane == 0) mbar_arrive_expect(bar, (uint32_t)C * (FIFTH ? 40u : 32u) + nh * halo_bytes);
             const uint32_t pb = map_rank(smem_u32(smem), c16 < C ? c16 : 0);
             named_bar_sync(1, nthreads);
-            const A *w = wpart + pr * 2 * SPLIT_WMAX + 2 * w8;
-            A y0, y1;
-            load_pair(w, y0, y1);
-            if (W > 8) {
-                A z0, z1;
-                load_pair(w + 16, z0, z1);
-                y0 = AT::add_tree(y0, z0);
-                y1 = AT::add_tree(y1, z1);
-            }
+            A x, y0, y1, y2 = AT::zero();
+            if constexpr (FIFTH) {  // sum lane / 8 of row warp lane % 8: three additions for all five
+                static_assert(!FIFTH || MAXT <= 288, "at most 8 row warps");
+                const int u = lane >> 3;
+                x = fold5<AT>(wpart[(u >> 1) * 2 * SPLIT_WMAX + 2 * w8 + (u & 1)], wpart[4 * SPLIT_WMAX + w8]);
+                y0 = bcast(x, 16 * pr);
+                y1 = bcast(x, 16 * pr + 8);
+                y2 = bcast(x, 4);
+            } else {
+                const A *w = wpart + pr * 2 * SPLIT_WMAX + 2 * w8;
+                load_pair(w, y0, y1);
+                if (W > 8) {
+                    A z0, z1;
+                    load_pair(w + 16, z0, z1);
+                    y0 = AT::add_tree(y0, z0);
+                    y1 = AT::add_tree(y1, z1);
+                }
 #pragma unroll
-            for (int m = 4; m >= 1; m >>= 1) {
-                y0 = AT::add_tree(y0, AT::shfl_xor(y0, m));
-                y1 = AT::add_tree(y1, AT::shfl_xor(y1, m));
+                for (int m = 4; m >= 1; m >>= 1) {
+                    y0 = AT::add_tree(y0, AT::shfl_xor(y0, m));
+                    y1 = AT::add_tree(y1, AT::shfl_xor(y1, m));
+                }
+                x = lane & 8 ? y1 : y0;
             }
-            A x = h8 ? y1 : y0;
             if (C > 1) {
-                if (c16 < C) push_pair(pb + slot_off + 16u * (uint32_t)rank, y0, y1, pb + (uint32_t)L.mbar + R0 + 8 * par);
+                const uint32_t pbar = pb + (uint32_t)L.mbar + R0 + 8 * par;
+                if (c16 < C) push_pair(pb + slot_off + 16u * (uint32_t)rank, y0, y1, pbar);
+                if (FIFTH && lane < C) st_async(pb + fifth_off + 8u * (uint32_t)rank, y2, pbar);
                 if (warp_wait(bar, (xr >> 1) & 1u, s_abort)) *s_fail = 1;
-                y0 = y1 = AT::zero();
-                if (c16 < C) load_pair(reinterpret_cast<const A *>(smem + slot_off + 16 * c16), y0, y1);
-                x = AT::add_tree(h8 ? y1 : y0, AT::shfl_xor(h8 ? y0 : y1, 8));
+                y0 = y1 = y2 = AT::zero();
+                if (c16 < C) {
+                    load_pair(reinterpret_cast<const A *>(smem + slot_off + 16 * c16), y0, y1);
+                    if (FIFTH) y2 = *reinterpret_cast<const A *>(smem + fifth_off + 8 * c16);
+                }
+                x = halve<AT>(y0, y1, 8);
+                if constexpr (FIFTH) {
+                    x = fold5<AT>(x, AT::add_tree(y2, AT::shfl_xor(y2, 8)));
+                } else {
 #pragma unroll
-                for (int m = 4; m >= 1; m >>= 1) x = AT::add_tree(x, AT::shfl_xor(x, m));
+                    for (int m = 4; m >= 1; m >>= 1) x = AT::add_tree(x, AT::shfl_xor(x, m));
+                }
             }
             Sums r;
+            r.old = FIFTH ? bcast(x, 4) : AT::zero();
             const T xf = AT::to_T(x);
             r.eta = bcast(x, 0);
             r.rr = __shfl_sync(0xffffffffu, xf, 8);
-            r.del = __shfl_sync(0xffffffffu, xf, 16);
-            r.eps = __shfl_sync(0xffffffffu, xf, 24);
+            r.del = bcast(x, 16);
+            r.eps = bcast(x, 24);
             return r;
         };
 
@@ -365,7 +390,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
             tol_t = mode1 ? (T)tol : (T)(tol * tol * AT::to_double(bb));
         } else {
             push_halo(0, ipar, r, R0 + 8 * ipar);
-            contribute(one ? AT::prod(bv, bv) : AT::zero(), AT::zero(), AT::zero(), AT::zero());
+            contribute(one ? AT::prod(bv, bv) : AT::zero(), AT::zero(), AT::zero(), AT::zero(), AT::zero());
         }
         ++xr;
         __syncthreads();
@@ -375,7 +400,8 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
         __syncthreads();
 
         const T big = sizeof(T) == 4 ? (T)3.402823466e38f : (T)1.7976931348623157e308;
-        T ups = T(0), inv_eta = T(0), rr = T(0);  // the sums warp's
+        A acc = AT::zero();                     // p^T S p; this and the next two the sums warp's
+        T inv_eta = T(0), rr = T(0), g = T(0);  // g (every warp's): the last beta (FIFTH: 0)
         int iters = 0;
         bool broke = false, late = false;  // late: this warp gave up waiting for S p rows
         for (int it = 0; !timed_out; ++it) {
@@ -383,7 +409,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
             if (late) *s_fail = 1;  // read after the second barrier from here
             T *vz = vecZ(zpar);
             T z = T(0), qv = T(0), t = T(0), hz = T(0), hp = T(0), hr = T(0);
-            A s_eta = AT::zero(), s_rr = AT::zero(), s_eps = AT::zero();
+            A s_eta = AT::zero(), s_rr = AT::zero(), s_eps = AT::zero(), s_old = AT::zero();
             // ---- r~ = Phi^-1 r, boundary rows to the neighbours -----------------------
             if (!sums) {
                 z = rowdot(true, vecR);
@@ -392,7 +418,8 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
                 if (Q == 1 || one) {
                     s_eta = AT::prod(r, z);
                     s_rr = sq_sum(r, T(0), A{});
-                    s_eps = AT::prod(z, s);
+                    s_eps = AT::prod(FIFTH ? z : fma_rn(T(0.5) * g, p, z), s);
+                    if (FIFTH) s_old = AT::prod(p, s);
                 }
             } else {
                 if (C > 1 && lane == 0) {
@@ -408,7 +435,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
                     if (warp_wait(mb + Z, xz & 1u, s_abort)) *s_fail = 1;
                 qv = rowdot(false, vz);
                 push_halo(0, zpar, qv, R0 + 8 * rpar);
-                contribute(s_eta, s_rr, Q == 1 || one ? AT::prod(z, qv) : AT::zero(), s_eps);
+                contribute(s_eta, s_rr, Q == 1 || one ? AT::prod(z, qv) : AT::zero(), s_eps, s_old);
                 t = rowdot(false, vecP);
                 push_halo(1, zpar, t, TT);
                 if (hany) {
@@ -421,13 +448,14 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
                 const Sums S = collect(1u);
                 const T etan = AT::to_T(S.eta);
                 const T beta = beta_from(etan, inv_eta, AT::to_T(eta));  // 0 in the first iteration
-                ups = fma_rn(beta, fma_rn(beta, ups, S.eps + S.eps), S.del);
-                const T alpha = quot(etan, ups);
+                if (FIFTH) acc = S.old;
+                const T old = AT::to_T(acc);
+                acc = curvature(S.del, S.eps, acc, beta, g);
+                const T ups = AT::to_T(acc), alpha = quot(etan, ups);
                 eta = S.eta;
                 rr = S.rr;
                 const bool done = !(fabs(etan) <= big && rr <= big) || (mode1 ? etan < tol_t : rr <= tol_t) || it >= max_iter;
-                // the identity cancelled, or S+ may not be positive on p (or not finite)
-                const bool direct = !(ups > T(0) && ups > T(0.0625) * fabs(S.del) && ups <= big);
+                const bool direct = doubtful(ups, AT::to_T(S.del), AT::to_T(S.eps), old, beta, g);
                 if (lane == 0) {
                     scal[0] = alpha;
                     scal[1] = beta;
@@ -445,6 +473,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
             T alpha = scal[0];
             const int f = *flags;
             if (f & 1) break;
+            if (!FIFTH) g = beta;
             // p = r~ + beta p, S p = S r~ + beta S p_old, lambda += alpha p,
             // r -= alpha S p; the halo copies of p and r alike
             s = fma_rn(beta, t, qv);
@@ -452,14 +481,14 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
             if (f & 2) {  // sum p^T S p itself
                 __syncthreads();  // flags and scalars are read
                 if (sums) {
-                    const T ud = AT::to_T(collect(0u).eta);
+                    acc = collect(0u).eta;
+                    const T ud = AT::to_T(acc);
                     if (lane == 0) {
                         scal[0] = AT::div(AT::to_T(eta), ud);
                         *flags = !(ud > T(0)) || !(ud <= big);
                     }
-                    ups = ud;
                 } else {
-                    contribute(Q == 1 || one ? AT::prod(p, s) : AT::zero(), AT::zero(), AT::zero(), AT::zero());
+                    contribute(Q == 1 || one ? AT::prod(p, s) : AT::zero(), AT::zero(), AT::zero(), AT::zero(), AT::zero());
                 }
                 ++xr;
                 __syncthreads();

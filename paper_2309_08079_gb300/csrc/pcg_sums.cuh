@@ -50,6 +50,77 @@ __device__ __forceinline__ double beta_from(double eta, double inv, double eta_o
     return __fma_rn(__fma_rn(-b, eta_old, eta), inv, b);
 }
 
+// p^T S p for p = r~ + beta p_old, without a reduction of its own.  With the last
+// beta, g, in the place of the one that r^T r~ will give, each thread adds up
+//     eps = (r~ + g / 2 p_old)^T S p_old,
+// and then
+//     p^T S p = r~^T S r~ + beta (2 eps + (beta - g) p_old^T S p_old),
+// so that the carried p_old^T S p_old enters with beta - g in place of beta: its error
+// is passed on times |beta (beta - g)| (p_old^T S p_old) / (p^T S p), 0.1-0.2 at the
+// median and 0.3-0.55 at the 95th percentile of the iterations (Kuka-shaped,
+// N = 32 and 128, nx = 36), where plain beta passes it on times 1 on average and
+// up to 10 in a row.  Relative error of alpha, rms of 48 iterations whose solution is
+// white noise, this form / summed itself / carried plainly in float: nx = 14,
+// N = 64 5.1e-7 / 4.8e-7 / 2.9e-6, N = 512 4.1e-7 / 4.0e-7 / 2.0e-6; nx = 36, N = 64
+// 4.0e-7 / 5.3e-7 / 3.0e-6.  Rounded once, by the compensated Horner scheme
+// (Graillat, Langlois, Louvet) in float pairs, in double arithmetic else.
+// Against the plain float form it takes 3 % (N = 512) to 5 % (batches); a fifth sum
+// in place of the prediction, the same accuracy, 9 %.
+__device__ __forceinline__ dfloat curvature(dfloat del, dfloat eps, dfloat old, float beta, float g) {
+    auto step = [](float b, float x, float xl, float a, float al, float &lo) {  // a + b x
+        const float p = __fmul_rn(b, x), s = __fadd_rn(p, a), t = __fsub_rn(s, p);
+        const float e = __fadd_rn(__fsub_rn(p, __fsub_rn(s, t)), __fsub_rn(a, t));
+        lo = __fmaf_rn(b, xl, __fadd_rn(__fadd_rn(e, __fmaf_rn(b, x, -p)), al));
+        return s;
+    };
+    float l1, l2;
+    const float s1 = step(__fsub_rn(beta, g), old.hi, old.lo, eps.hi + eps.hi, eps.lo + eps.lo, l1);
+    const float s2 = step(beta, s1, l1, del.hi, del.lo, l2), hi = __fadd_rn(s2, l2);
+    return dfloat{hi, __fsub_rn(l2, __fsub_rn(hi, s2))};
+}
+__device__ __forceinline__ double curvature(double del, double eps, double old, double beta, double g) {
+    return __fma_rn(beta, __fma_rn(beta - g, old, eps + eps), del);
+}
+
+// Is that p^T S p not to be trusted, and to be summed itself?  It is not positive or
+// not finite, its three terms cancel to less than about 1/32 of their size, or
+// more than 0.9 of the error of p_old^T S p_old is passed on (so that no more than
+// ten iterations' worth of errors can gather).
+__device__ __forceinline__ bool doubtful(float ups, float del, float eps, float old, float beta, float g) {
+    const float b = fabsf(beta), passed = b * (fabsf(beta - g) * fabsf(old)), m = __fmaf_rn(b, 2.f * fabsf(eps), fabsf(del)) + passed;
+    return !(ups > 0.f && ups > 0.03125f * m && passed <= 0.9f * ups && ups <= 3.402823466e38f);
+}
+// In double p_old^T S p_old is a sum of its own in each iteration (g = 0), and nothing
+// is carried (error of alpha 1.2e-15, 1.1e-15 summed itself, 7.0e-15 carried).  The terms are compared by their exponents, since an FP64
+// instruction takes an issue slot of 64 cycles.
+__device__ __forceinline__ bool doubtful(double ups, double del, double eps, double old, double beta, double) {
+    auto ex = [](double x) { return (__double2hiint(x) >> 20) & 2047; };
+    const int eb = ex(beta) - 1023, lead = max(ex(del), max(ex(eps) + 1, ex(old) + eb) + eb);
+    return !(ups > 0.0 && ex(ups) >= lead - 4 && ups <= 1.7976931348623157e308);
+}
+
+// Sums over a warp of five accumulators per lane by recursive halving, each lane
+// giving away half of its sums per level: lanes 8u end with sum u, lane 4 with
+// the fifth.  fold5: the last three levels, with sum lane / 8 in x and the fifth in
+// e (each over lanes lane % 8).
+template <class AT, typename A>
+__device__ __forceinline__ A halve(A p0, A p1, int m) {
+    const bool h = threadIdx.x & m;
+    return AT::add_tree(h ? p1 : p0, AT::shfl_xor(h ? p0 : p1, m));
+}
+template <class AT, typename A>
+__device__ __forceinline__ A fold5(A x, A e) {
+    x = halve<AT>(x, e, 4);
+    x = AT::add_tree(x, AT::shfl_xor(x, 2));
+    return AT::add_tree(x, AT::shfl_xor(x, 1));
+}
+template <class AT, typename A>
+__device__ __forceinline__ A warp_sums5(A v0, A v1, A v2, A v3, A v4) {
+    const A x = halve<AT>(halve<AT>(v0, v2, 16), halve<AT>(v1, v3, 16), 8);
+    const A e = AT::add_tree(v4, AT::shfl_xor(v4, 16));
+    return fold5<AT>(x, AT::add_tree(e, AT::shfl_xor(e, 8)));
+}
+
 // Every lane of a warp waits (bounded) for the phase of `parity`; true in all
 // lanes if any of them gave up.
 __device__ __forceinline__ bool warp_wait(uint32_t mbar, uint32_t parity, const volatile int *abort_flag) {
