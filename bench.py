@@ -196,6 +196,21 @@ def latency_roofline(s, lt, sch, opts, iters_mean: float, launch_us: float, roun
             "floor_ns_per_iteration": floor_ns, "shape": sh}
 
 
+def cluster_batch_floor_ms(iters, Ns, exchange_ns, n_sms: int, shape: dict) -> float:
+    """Synchronisation floor of a batch in the float32 nx = 14 clusters, whichever
+    of their forms the device takes (Solver.pcg_shape reports the one with two
+    CTAs per SM): an instance holds the CTAs that its horizon needs (32 knots
+    each, never more than the reported C), two to an SM, for at least one
+    exchange of that group per iteration, exchange_ns(CTAs, warps); a group of
+    one CTA has none.  The SM-time of all instances spread over the SMs, or the
+    longest instance's exchanges alone if that is more."""
+    need = np.array([min(shape["C"], next(x for x in (1, 2, 3, 4, 6, 8, 12, 16) if 32 * x >= n)) for n in Ns])
+    W = min(4, shape["threads"] // 32)
+    x = {int(c): 0.0 if c == 1 else exchange_ns(int(c), W) for c in np.unique(need)}
+    t = np.asarray(iters, dtype=np.float64) * np.array([x[int(c)] for c in need])
+    return float(max(np.sum(t * need) / 2.0 / n_sms, np.max(t))) * 1e-6
+
+
 def profile_onchip():
     """SMEM-pipe share and barrier-stall share of the cluster kernel from the
     committed ncu summary, when it was taken from the current sources."""
@@ -613,33 +628,30 @@ def run_batched(s, dev, solves):
         tuned = tuner.tune(lt, sch, master[0], opts)
         runner = tuner.runner(lt, sch, master[0], opts)
 
-    # Sync-latency floor of the cluster launches: the clusters keep each
-    # instance's operators on chip, so an instance holds the SMs of the CTAs
-    # that its horizon needs (32 knots each; two CTAs of 128 threads share an
-    # SM) for at least iterations x 1 exchange at the latency
-    # mpcg_bench_exchange measures on its launch shape; the floor is that
-    # SM-time summed over the graph's solves and spread over every SM.
+    # Sync-latency floor of the cluster launches, which keep each instance's
+    # operators on chip (cluster_batch_floor_ms)
     n_sms = torch.cuda.get_device_properties(dev).multi_processor_count
     xcache = {}
+
+    def exchange_ns(C, W):
+        if (C, W) not in xcache:
+            xcache[C, W] = s.bench_exchange(C, W, rounds=1000)["ns"]
+        return xcache[C, W]
 
     def cluster_floor_ms(groups, iters):
         """(floor over the cluster groups, their shapes, the instances of
         the other groups, which stream their operators from HBM)."""
-        sm_ns, shapes, other = 0.0, [], []
+        floor, shapes, other = 0.0, [], []
         for o_g, N_g, idx in groups:
             sh = s.pcg_shape(lt, sch, o_g, N=N_g)
             if sh["form"] != "cluster":
                 other.extend(int(i) for i in idx)
                 continue
-            key = (sh["C"], sh["threads"] // 32)
-            if key not in xcache:
-                xcache[key] = s.bench_exchange(*key, rounds=1000)["ns"]
-            need = np.array([min(sh["C"], next(x for x in (1, 2, 3, 4, 6, 8, 12, 16) if 32 * x >= n)) for n in Ns[idx]])
-            sm_ns += float(np.sum(iters[idx] * need)) * xcache[key] / (2.0 if sh["threads"] <= 128 else 1.0)
+            floor += cluster_batch_floor_ms(iters[idx], Ns[idx], exchange_ns, n_sms, sh)
             shapes.append({"C": sh["C"], "threads": sh["threads"], "instances": int(len(idx))})
         if not shapes:
             return None, None, other
-        return sm_ns / n_sms * 1e-6, shapes, other
+        return floor, shapes, other
 
     # capture the repeated solves in one graph, once per PCG kernel form
     per_mode = {}
@@ -684,9 +696,10 @@ def run_batched(s, dev, solves):
         if floor is not None:
             roof = {"bound": "sync_latency", "frac": floor / gms, "floor_ms": floor, "shapes": shapes,
                     "note": "SM-time of every cluster-launched instance at 1 measured exchange "
-                            "(mpcg_bench_exchange, its launch shape) per PCG iteration, spread over all "
-                            "SMs, over the graph time (formation and recovery included); operators stay "
-                            "on chip",
+                            "(mpcg_bench_exchange, the CTAs its horizon needs, two to an SM) per PCG "
+                            "iteration, spread over all SMs, over the graph time (formation and recovery "
+                            "included); operators stay on chip; shapes: as pcg_shape reports them (the first "
+                            "launch of the form with two CTAs per SM)",
                     "hbm_equivalent_frac": hbm_frac, "peak_source": note}
             if other:
                 # a mixed plan: the tiled (or L2) groups stream their operators
@@ -787,13 +800,13 @@ def run_backward(s, dev, reps=5):
     it_b = read_stats(bst)["iters"].astype(np.float64)
     alg = float(np.sum(it_f + it_b)) * c["N"] * pcg_bytes_per_knot_iter(c["nx"])
     # the batch's clusters keep their operators on chip: the floor is the
-    # reductions' latency, one exchange per iteration on each cluster, the
-    # instances spread over the co-resident clusters
+    # reductions' latency
     sh = s.pcg_shape(lt, sch, opts)
     lat = None
     if sh["form"] == "cluster":
-        x = s.bench_exchange(sh["C"], sh["threads"] // 32, rounds=1000)
-        lat = float(np.sum(it_f + it_b)) * x["ns"] * 1e-6 / max(1, min(sh["clusters"], c["B"]))
+        lat = cluster_batch_floor_ms(it_f + it_b, [c["N"]] * c["B"],
+                                     lambda C, W: s.bench_exchange(C, W, rounds=1000)["ns"],
+                                     torch.cuda.get_device_properties(dev).multi_processor_count, sh)
     # gradient of instance 0 against the oracle's analytic gradient
     it0 = batch.items[0].astype(np.float64)
     l0, x0, u0 = oracle.kkt_solve(it0)
@@ -823,8 +836,9 @@ def run_backward(s, dev, reps=5):
             "speedup_vs_loop": t_loop / (f + bw), "converged": ok, "grad_relerr_vs_oracle": gerr,
             "pcg_roofline": {"bound": "sync_latency", "frac": (lat / (f + bw)) if lat else None,
                              "floor_ms": lat, "shape": sh,
-                             "note": "forward + adjoint PCG iterations x 1 measured exchange, spread over the "
-                                     "co-resident clusters, over fwd + bwd time",
+                             "note": "forward + adjoint PCG iterations x 1 measured exchange (the CTAs an "
+                                     "instance needs, two to an SM; the longest instance's if more), over fwd + "
+                                     "bwd time; shape: as pcg_shape reports it (the form with two CTAs per SM)",
                              "hbm_equivalent_frac": alg / ((f + bw) / 1e3) / 1e9 / hbm, "peak_source": note}}
 
 

@@ -278,7 +278,11 @@ int mpcg_pcg_solve(mpcg_handle *h, mpcg_dims dims, const mpcg_schur *schur, void
  * streams the packed diagonal blocks (schur->Sdp, Pdp), else 0.  `shape` is
  * a HOST int[6]; the schur pointers matter only through their alignment
  * (the tiled kernel needs 16-byte-aligned blocks) and whether the packed
- * copies are given.  B = 1 for a single instance.
+ * copies are given.  B = 1 for a single instance.  A float32 nx = 14 batch of
+ * more instances than clusters takes up to six launches: reported is the first
+ * (the longest horizons) of the form with two CTAs per SM, and where the device
+ * chooses between that form and the one in registers (up to four waves of the
+ * latter), the work may be the other's.
  */
 int mpcg_pcg_shape(mpcg_handle *h, mpcg_dims dims, int B, const mpcg_schur *schur,
                    const mpcg_opts *opts, int *shape);

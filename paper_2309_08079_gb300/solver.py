@@ -195,7 +195,9 @@ class Solver:
     def pcg_shape(self, lq: LQTensors, schur: SchurTensors, opts=None, N: Optional[int] = None) -> dict:
         """The launch shape pcg_solve uses for these arguments (nothing is
         launched): kernel form, CTAs per cluster, clusters in the grid,
-        threads per CTA."""
+        threads per CTA.  Of a float32 nx = 14 batch with more instances than
+        clusters the first launch of the form with two CTAs per SM; the device
+        may give the work to the form in registers."""
         ss = schur.struct()
         o = opts if opts is not None else make_opts()
         dims = lq.dims()

@@ -72,3 +72,25 @@ def test_summary_collects_the_secondary_figures_last():
 def test_percentiles():
     p = bench.pct(np.arange(1, 11, dtype=float))
     assert p["p50"] == pytest.approx(5.5) and p["max"] == 10.0 and p["p10"] < p["p90"]
+
+
+def test_batch_floor_takes_the_group_of_each_instance():
+    """A lower bound for every form of the batch: the exchange of the CTAs an
+    instance needs (not of the reported cluster), two CTAs to an SM, none for
+    one CTA; never less than the longest instance alone."""
+    asked = []
+
+    def exchange(C, W):
+        asked.append((C, W))
+        return 100.0 * C
+    shape = {"C": 16, "threads": 128, "clusters": 14}
+    # 128 instances of 4 CTAs: 128 * 10 * 400 ns * 4 / 2 over 100 SMs, above 10 * 400 ns
+    assert bench.cluster_batch_floor_ms([10] * 128, [128] * 128, exchange, 100, shape) == pytest.approx(128 * 10 * 400 * 2 / 100 * 1e-6)
+    assert asked == [(4, 4)]
+    # few instances: the longest one
+    assert bench.cluster_batch_floor_ms([10, 7], [512, 20], exchange, 152, shape) == pytest.approx(16000e-6)
+    assert bench.cluster_batch_floor_ms([50], [32], exchange, 152, shape) == 0.0
+    # the reported cluster caps the group, its warps the exchange
+    asked.clear()
+    bench.cluster_batch_floor_ms([10], [512], exchange, 152, {"C": 12, "threads": 64, "clusters": 1})
+    assert asked == [(12, 2)]
