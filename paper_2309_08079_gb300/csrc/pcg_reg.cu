@@ -654,12 +654,12 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
             const float beta = beta_from(etan, inv_eta, AT::to_T(eta));  // 0 in the first iteration
             eta = S.eta;
             rr = S.rr;
-            const float old = AT::to_T(acc);
+            const A old = acc;
             acc = curvature(S.del, S.eps, acc, beta, g);
             float ups = AT::to_T(acc), alpha = __fdividef(etan, ups);
             const bool done = !(fabsf(etan) <= 3.402823466e38f && rr <= 3.402823466e38f) ||
                               (mode1 ? etan < tol_t : rr <= tol_t) || it >= max_iter;
-            const bool direct = doubtful(ups, AT::to_T(S.del), AT::to_T(S.eps), old, beta, g);
+            const bool direct = doubtful(ups, S.del, S.eps, old, beta, g);
             // p = r~ + beta p, S p = S r~ + beta S p_old, lambda += alpha p,
             // r -= alpha S p; the halo copies of p and r alike
             auto next_p = [&]() {

@@ -449,13 +449,13 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
                 const T etan = AT::to_T(S.eta);
                 const T beta = beta_from(etan, inv_eta, AT::to_T(eta));  // 0 in the first iteration
                 if (FIFTH) acc = S.old;
-                const T old = AT::to_T(acc);
+                const A old = acc;
                 acc = curvature(S.del, S.eps, acc, beta, g);
                 const T ups = AT::to_T(acc), alpha = quot(etan, ups);
                 eta = S.eta;
                 rr = S.rr;
                 const bool done = !(fabs(etan) <= big && rr <= big) || (mode1 ? etan < tol_t : rr <= tol_t) || it >= max_iter;
-                const bool direct = doubtful(ups, AT::to_T(S.del), AT::to_T(S.eps), old, beta, g);
+                const bool direct = doubtful(ups, S.del, S.eps, old, beta, g);
                 if (lane == 0) {
                     scal[0] = alpha;
                     scal[1] = beta;

@@ -86,13 +86,23 @@ __device__ __forceinline__ double curvature(double del, double eps, double old, 
 // not finite, its three terms cancel to less than about 1/32 of their size, or
 // more than 0.9 of the error of p_old^T S p_old is passed on (so that no more than
 // ten iterations' worth of errors can gather).
-__device__ __forceinline__ bool doubtful(float ups, float del, float eps, float old, float beta, float g) {
-    const float b = fabsf(beta), passed = b * (fabsf(beta - g) * fabsf(old)), m = __fmaf_rn(b, 2.f * fabsf(eps), fabsf(del)) + passed;
+__device__ __forceinline__ bool doubtful(float ups, dfloat del, dfloat eps, dfloat old, float beta, float g) {
+    const float b = fabsf(beta), passed = b * (fabsf(beta - g) * fabsf(old.hi)),
+                m = __fmaf_rn(b, 2.f * fabsf(eps.hi), fabsf(del.hi)) + passed;
     return !(ups > 0.f && ups > 0.03125f * m && passed <= 0.9f * ups && ups <= 3.402823466e38f);
 }
+// (float32 with double sums: an FP64 instruction, conversions among them, takes an
+// issue slot of 64 cycles, so the terms are compared by their high words)
+__device__ __forceinline__ float high(double x) {  // |x| to a relative 2^-20, in float's range
+    const int h = __double2hiint(x) & 0x7fffffff, lo = 0x38100000, hi = 0x47efffff;
+    return h < lo ? 0.f : __int_as_float((min(h, hi) - 0x38000000) << 3);
+}
+__device__ __forceinline__ bool doubtful(float ups, double del, double eps, double old, float beta, float g) {
+    return doubtful(ups, dfloat{high(del), 0.f}, dfloat{high(eps), 0.f}, dfloat{high(old), 0.f}, beta, g);
+}
 // In double p_old^T S p_old is a sum of its own in each iteration (g = 0), and nothing
-// is carried (error of alpha 1.2e-15, 1.1e-15 summed itself, 7.0e-15 carried).  The terms are compared by their exponents, since an FP64
-// instruction takes an issue slot of 64 cycles.
+// is carried (error of alpha 1.2e-15, 1.1e-15 summed itself, 7.0e-15 carried).  The
+// terms are compared by their exponents.
 __device__ __forceinline__ bool doubtful(double ups, double del, double eps, double old, double beta, double) {
     auto ex = [](double x) { return (__double2hiint(x) >> 20) & 2047; };
     const int eb = ex(beta) - 1023, lead = max(ex(del), max(ex(eps) + 1, ex(old) + eb) + eb);
