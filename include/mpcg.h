@@ -282,7 +282,8 @@ int mpcg_pcg_solve(mpcg_handle *h, mpcg_dims dims, const mpcg_schur *schur, void
  * more instances than clusters takes up to six launches: reported is the first
  * (the longest horizons) of the form with two CTAs per SM, and where the device
  * chooses between that form and the one in registers (up to four waves of the
- * latter), the work may be the other's.
+ * latter), the work may be the other's.  A float32 nx = 36 batch reported with
+ * several CTAs per instance may run with one, where its horizons favour that.
  */
 int mpcg_pcg_shape(mpcg_handle *h, mpcg_dims dims, int B, const mpcg_schur *schur,
                    const mpcg_opts *opts, int *shape);

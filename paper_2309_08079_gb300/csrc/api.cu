@@ -172,6 +172,7 @@ int choose_pcg_tile(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_schur 
     int n = shape(1);  // what one CTA cannot hold stays refused
     if (n < 1) return MPCG_EUNSUPPORTED;
     L.n_cta = n;
+    const PcgLaunch one = L;
     // `clusters` (float32 nx = 36): as many CTAs per instance as pays.  One
     // iteration of an instance takes about 6 us + 0.35 us per knot of a CTA
     // (measured alone at 16..224 knots: 12.1, 15.7 at 32, 25 at 64, 51 at 128,
@@ -197,6 +198,11 @@ int choose_pcg_tile(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_schur 
         }
         while (cost[levels - 1] > 1.2 * best) --levels;
         n = shape(1 << (levels - 1));
+        // The horizons may still favour a CTA each: the device chooses.  (Up to one
+        // wave of CTAs equal horizons do so most.)
+        const int m = std::min(n, h->sms / L.C);
+        if (L.C > 1 && (B > L.n_cta || !tile_clusters_pay_when_equal(d.N, B, L.C, m, L.n_cta, one.pk)))
+            L.one = {std::min(B, L.n_cta), one.kpc_max, one.threads, one.depth, one.pk, m, one.smem};
     }
     L.clusters = std::max(1, std::min(B, n));
     // a batch of more than one wave starts its long horizons first
@@ -469,8 +475,9 @@ int pcg_t(mpcg_handle *h, const mpcg_dims &d, int B, const int *knot_off, const 
     if (P.precon < 0 || P.precon > 2) return MPCG_EINVAL;
     P.inst_list = (o && o->instances && o->n_instances > 0) ? o->instances : nullptr;
     P.n_tickets = P.inst_list ? o->n_instances : B;
-    P.Sdp = (L.cta_mode == 2 && L.pk) ? (const T *)s->Sdp : nullptr;
-    P.Pdp = (L.cta_mode == 2 && L.pk) ? (const T *)s->Pdp : nullptr;
+    const bool packed = L.cta_mode == 2 && (L.pk || L.one.pk);
+    P.Sdp = packed ? (const T *)s->Sdp : nullptr;
+    P.Pdp = packed ? (const T *)s->Pdp : nullptr;
     P.npk = packed_len(d.nx);
     if (P.inst_list && !knot_off) return MPCG_EINVAL;
     if (P.n_tickets > 1 && (L.clusters < P.n_tickets || L.light.clusters > 0)) {

@@ -27,7 +27,10 @@ struct PcgParams {
     const unsigned *info;
     mpcg_stats *stats;
     int *queue;       // instance counters, one per group level (nullptr: static round robin)
-    int pick;         // pcg_reg_kernel: 1 / -1: this launch serves batches of more / at most `work`
+    int pick;         // pcg_reg_kernel: 1 / -1: this launch serves batches of more / at most `work`;
+                      // pcg_tile_kernel: batches that clusters / one CTA each serve faster
+    int pick_C, pick_m, pick_n;  // pcg_tile_kernel, with pick: CTAs per cluster, clusters and CTAs at a time
+    int pick_packed;             // ... does the form with one CTA stream packed blocks?
     long long work;
     int n_above, n_upto;  // pcg_reg_kernel: the horizons this launch takes, (n_above, n_upto]
     int split;        // pcg_reg_kernel: clusters split into groups for shorter horizons;
@@ -72,6 +75,12 @@ struct PcgLaunch {
     int n_mid, n_low;  // reg: clusters of the later stages, 3/4 and 1/2 of the full
                    // size (0: one launch; see pcg_reg.cu)
     int n_cta;     // tiled: instances that one CTA each takes at a time
+    // tiled with C > 1: the form with one CTA per instance, where the device chooses
+    // by the horizons (clusters > 0), and the clusters at a time of this one
+    struct {
+        int clusters, kpc_max, threads, depth, pk, m;
+        size_t smem;
+    } one;
     int split;     // reg: one counter per group level, clusters split (see pcg_reg.cu);
                    // tiled: long horizons first (one counter per quarter of n_long)
     int n_long;    // tiled, reg with light: the longest horizon the launch is sized for
@@ -136,6 +145,9 @@ template <typename T>
 size_t pcg_tile_smem_bytes(int nmax, int vs, int W, int NS, int nx, int depth, int npk, bool cluster);
 template <typename T> cudaError_t pcg_tile_launch(const PcgLaunch &, const PcgParams<T> &, cudaStream_t);
 template <typename T> int pcg_tile_max_clusters(const PcgLaunch &, int sms);
+// nx = 36, B instances of N knots each: clusters of C CTAs, m at a time, rather than one
+// CTA each, n at a time?
+bool tile_clusters_pay_when_equal(int N, int B, int C, int m, int n, bool packed);
 template <typename T> size_t pcg_cta_smem_bytes(int nmax, int vs, int W);
 template <typename T> cudaError_t pcg_cta_launch(const PcgLaunch &, const PcgParams<T> &, cudaStream_t);
 template <typename T> int pcg_cta_max_blocks(const PcgLaunch &);

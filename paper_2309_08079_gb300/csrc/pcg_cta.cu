@@ -503,6 +503,39 @@ constexpr int tile_max_threads() { return NXC == 36 ? 256 : 512; }
 // of 64..256 219 -> 45, 24 of 64..128 62 -> 22; alone at N = 256 41.2 (pcg.cu, 16
 // CTAs) -> 28.6.  Packed diagonal blocks cost more loads than they save here
 // (136 -> 192), a ring of three steps ahead gives nothing.
+//
+// Which form a batch takes depends on its horizons, which the host does not know:
+// where equal horizons would favour one CTA per instance, both are launched and
+// every CTA finds the same answer from sum N_i and sum N_i^2 (the other form's leave
+// at once).  Per iteration of the longest horizon N, with iterations growing as
+// the horizon: nb = sum N_i / N instances of S = sum N_i^2 / N knots in waves of
+// tile_cost(a, b) each (whole waves for equal horizons), and never faster than
+// the blocks stream (the more instances at a time, the less of them the L2 holds).
+// Measured, us per iteration, clusters / one CTA: 152 of 200
+// knots 114 / 88, 80 of 72 43 / 30, 100 of 256 94 / 110, 60 of 160 41 / 65; 160 of
+// 64..256 knots 136 / 238 ms.
+__host__ __device__ inline float tile_cost(float start, float knots, float nb, float S, float at_a_time, float share, float ragged) {
+    const float t = start + 0.35f * knots, x = (start * nb + 0.35f * S * share) / (at_a_time * t);
+    const float waves = x + ragged * (ceilf(x) - x);
+    return t * (waves > 1.f ? waves : 1.f);
+}
+// count, sum and sum of squares of the horizons -> clusters of C CTAs, m at a
+// time, rather than one CTA each, n at a time?
+__host__ __device__ inline bool tile_clusters_pay(int N, float count, float sum, float sum2, int C, int m, int n, bool packed) {
+    const float nb = sum / N, S = sum2 / N, u = (nb / count - 0.6f) / 0.4f, ragged = u > 0.f ? u : 0.f;
+    const float tc = tile_cost(8.f, (float)ceil_div(N, C), nb, S, (float)m, 1.f / C, ragged), bc = (C == 2 ? 4.2e-3f : 3.7e-3f) * S;
+    const float t1 = tile_cost(6.f, (float)N, nb, S, (float)n, 1.f, ragged), b1 = (packed ? 2.85e-3f : 3.5e-3f) * S;
+    return (tc > bc ? tc : bc) <= (t1 > b1 ? t1 : b1);
+}
+bool tile_clusters_pay_when_equal(int N, int B, int C, int m, int n, bool packed) {
+    return tile_clusters_pay(N, (float)B, (float)B * N, (float)B * N * N, C, m, n, packed);
+}
+// one definition for both forms (the compiler may contract differently where it
+// is inlined, and both have to come to the same answer)
+__device__ __noinline__ bool tile_pick(int N, float count, float sum, float sum2, int C, int m, int n, int packed) {
+    return tile_clusters_pay(N, count, sum, sum2, C, m, n, packed != 0);
+}
+
 template <typename T, int LPK, int RPT, int VW, int NXC = 0, typename AT = Acc<T>, bool PK = false, bool CL = false>
 __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(const PcgParams<T> P) {
     // PK: the diagonal blocks arrive packed (upper triangle by columns) and
@@ -537,6 +570,29 @@ __global__ void __launch_bounds__(tile_max_threads<NXC>(), 1) pcg_tile_kernel(co
     int *s_misc = reinterpret_cast<int *>(smem + Lo.misc);
     const uint32_t mbs = smem_u32(&mbar[(size_t)s * RM]);  // this stream's barriers
 
+    if constexpr (NXC == 36) {
+        if (P.pick) {  // is this form the batch's?  (in wpart: cleared here, written before it is read below)
+            unsigned long long *sum = reinterpret_cast<unsigned long long *>(smem + Lo.wpart);
+            if (tid < 2) sum[tid] = 0;
+            __syncthreads();
+            unsigned long long k = 0, k2 = 0;  // k: the count above bit 40
+            for (int t = tid; t < P.n_tickets; t += nthreads) {
+                int k0, Nb;
+                P.bv.range(P.inst_list ? P.inst_list[t] : t, k0, Nb);
+                if (Nb < 1 || Nb > P.n_long) continue;
+                k += (1ull << 40) + (unsigned)Nb;
+                k2 += (unsigned long long)Nb * Nb;
+            }
+            atomicAdd(sum, k);
+            atomicAdd(sum + 1, k2);
+            __syncthreads();
+            const unsigned long long all = sum[0];
+            const bool pay = tile_pick(P.n_long, (float)(all >> 40), (float)(all & ((1ull << 40) - 1)), (float)sum[1], P.pick_C,
+                                       P.pick_m, P.pick_n, P.pick_packed);
+            if (pay != (P.pick > 0)) return;
+            __syncthreads();
+        }
+    }
     for (int e = tid; e < NS * RM; e += nthreads) mbar_init(smem_u32(&mbar[e]), 1);
     if (tid == 0) fence_mbar_init();
     __syncthreads();
@@ -1088,9 +1144,29 @@ cudaError_t pcg_tile_launch(const PcgLaunch &L, const PcgParams<T> &P0, cudaStre
     P.depth = L.depth;
     P.split = P.queue ? L.split : 0;
     P.n_long = L.n_long;
+    P.pick = L.one.clusters > 0 ? 1 : 0;
+    P.pick_C = L.C;
+    P.pick_m = L.one.m;
+    P.pick_n = L.n_cta;
+    P.pick_packed = L.one.pk;
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = tile_config(L, L.clusters, attr, s);
-    return cudaLaunchKernelEx(&cfg, pcg_tile_fn<T>(L), P);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, pcg_tile_fn<T>(L), P);
+    if (e != cudaSuccess || !P.pick) return e;
+    PcgLaunch O = L;
+    O.C = 1;
+    O.clusters = L.one.clusters;
+    O.kpc_max = L.one.kpc_max;
+    O.threads = L.one.threads;
+    O.depth = L.one.depth;
+    O.pk = L.one.pk;
+    O.smem = L.one.smem;
+    P.pick = -1;
+    P.kpc_max = O.kpc_max;
+    P.depth = O.depth;
+    P.split = P.queue && O.clusters < P.n_tickets;
+    const cudaLaunchConfig_t cfg1 = tile_config(O, O.clusters, attr, s);
+    return cudaLaunchKernelEx(&cfg1, pcg_tile_fn<T>(O), P);
 }
 
 // Co-resident clusters (CTAs when L.C == 1) on the device (0: cannot run).

@@ -85,3 +85,52 @@ def test_capped_iterate(N, precon):
     if precon == 0:
         lo, it, _ = oracle.pcg(Sd, So, *oracle.precon_blocks(Sd, So), -g, lam0=lam0, tol=1e-30, max_iter=m)
         assert it == m and oracle.relerr(got[0][0], lo.reshape(N, 36)) < 1e-3
+
+
+def _capped(s, lt, sch, mode, m=4, lam0=0.25):
+    import torch
+    from paper_2309_08079_gb300.solver import make_opts
+    lam = torch.full((lt.total, 36), lam0, device="cuda")
+    s.pcg_solve(lt, sch, lam, make_opts(mode=mode, tol=1e-30, max_iter=m), s.alloc_stats(lt.nb), s.alloc_workspace(lt))
+    return lam
+
+
+def _median_ms(f):
+    import torch
+    f()
+    t = []
+    for _ in range(9):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        f()
+        b.record()
+        b.synchronize()
+        t.append(a.elapsed_time(b))
+    return sorted(t)[4]
+
+
+@pytest.mark.parametrize("Ns,one", [([200] * 152, True), ([72] * 100, True), ([100] * 120, True), ([256, 64, 80, 90] * 40, False),
+                                    ([160] * 60, False)])
+def test_batch_takes_the_form_that_its_horizons_favour(Ns, one):
+    """Equal horizons that fill the GPU run with a CTA per instance: the bits of
+    mode 3 (which has no other form), eagerly, from a captured graph and with a
+    padded list, and within 1.1 of its time (clusters took 1.3).  Ragged ones,
+    and few, run with clusters: other bits (another order of sums), less time."""
+    import torch
+    from paper_2309_08079_gb300.solver import make_opts
+    s, batch, lt, sch = _formed(Ns, 5300)
+    assert s.pcg_shape(lt, sch, make_opts())["C"] > 1
+    want, got = _capped(s, lt, sch, 3), _capped(s, lt, sch, 0)
+    assert torch.equal(got, want) == one
+    assert oracle.relerr(got.cpu().double().numpy(), want.cpu().double().numpy()) < 1e-4
+    g = torch.cuda.CUDAGraph()
+    stats, ws, lam = s.alloc_stats(lt.nb), s.alloc_workspace(lt), torch.empty_like(got)
+    o = make_opts(tol=1e-30, max_iter=4)
+    with torch.cuda.graph(g):
+        lam.fill_(0.25)
+        s.pcg_solve(lt, sch, lam, o, stats, ws)
+    for _ in range(2):
+        g.replay()
+    assert torch.equal(lam, got)
+    t0, t3 = (_median_ms(lambda: _capped(s, lt, sch, mode, 40)) for mode in (0, 3))
+    assert t0 < (1.1 if one else 0.95) * t3, (t0, t3)
