@@ -307,20 +307,31 @@ int choose_pcg_cluster(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opt
     // every instance has its own cluster (pcg_split.cu), as many CTAs as that
     // leaves (the products of a CTA shrink with its knots: N = 64 1.90 us per
     // iteration at 4 knots per CTA, N = 128 2.94 at 8); float64 accumulation of
-    // float32 sums stays with the general form
+    // float32 sums stays with the general form.  A given number of CTAs that leaves
+    // fewer clusters than instances: while the waves over the general form's, which
+    // packs more clusters on an SM, are made up for by its speed (nx = 36 about 4.5
+    // times; float64 1.3 at 4 CTAs to 2 at 16).  40 instances, 60 iterations, this /
+    // general: float64 of 32 knots at 4, 8, 16 CTAs 746 / 680, 844 / 553, 1442 / 519 us;
+    // nx = 36 of 16 knots 262 / 606, 274 / 579, 389 / 591.
+    PcgLaunch in_turn{};
     if (!wide && !L.dot) {
         const int fixed = o && o->cluster > 0 ? std::min(o->cluster, d.N) : 0;
         for (int C = fixed ? fixed : std::min(kMaxCluster, d.N); C >= (fixed ? fixed : 1) && C <= kMaxCluster; --C) {
             PcgLaunch Ls{};
             const int n = pcg_split_shape<T>(nx, d.N, C, Ls);
             if (n < 1 && !fixed && Ls.C == 0) break;  // not its shape at this many knots per CTA, nor below
-            if (n >= B || (fixed && n >= 1)) {
+            if (n >= B) {
                 L = Ls;
-                L.clusters = std::min(B, n);
+                L.clusters = B;
                 return MPCG_OK;
+            }
+            if (fixed && n >= 1) {
+                in_turn = Ls;
+                in_turn.clusters = n;
             }
         }
     }
+    const double speed = sizeof(T) == 4 ? 5.0 : 1.3;
     if (wide) { L.lpk = 8; L.rpt = 2; }
     else if (nx <= 16) { L.lpk = 16; L.rpt = 1; }
     else if (nx <= 32) { L.lpk = 32; L.rpt = 1; }
@@ -346,6 +357,10 @@ int choose_pcg_cluster(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opt
         if (pcg_smem_bytes<T>(L.kpc_max, L.vs, C, W, nx, 1, L.dot) <= (size_t)h->smem_optin) L.stage = 1;
         L.smem = pcg_smem_bytes<T>(L.kpc_max, L.vs, C, W, nx, L.stage, L.dot);
         const int active = pcg_max_clusters<T>(L);
+        if (in_turn.clusters > 0 && (active < 1 || ceil_div(B, in_turn.clusters) <= speed * ceil_div(B, active))) {
+            L = in_turn;
+            return MPCG_OK;
+        }
         if (active >= 1) {
             L.clusters = std::max(1, std::min(B, active));
             return MPCG_OK;

@@ -298,3 +298,29 @@ def test_steps_are_as_exact_as_with_a_direct_sum(nx, nu, N, dtype, dot):
                 rms[mode] += float(((v * r[m + 1]).sum() / (v * r[m]).sum()) ** 2) / (3 * M)
     assert np.sqrt(rms[1]) < 2.0 * np.sqrt(rms[3]), {k: np.sqrt(v) for k, v in rms.items()}
     print({k: np.sqrt(v) for k, v in rms.items()})
+
+
+@pytest.mark.parametrize("nx,nu,dtype,N,C,at_once", [(14, 7, "float64", 32, 4, True), (14, 7, "float64", 32, 16, True),
+                                                     (36, 12, "float32", 16, 8, False), (14, 7, "float64", 32, 2, True)])
+def test_fixed_cluster_batches_run_at_once_where_that_is_faster(nx, nu, dtype, N, C, at_once):
+    """40 instances with a given number of CTAs: in float64 the general kernel,
+    which holds them all at once, unless the lane-per-row kernel does; at nx =
+    36 the latter in several waves.  The solutions are those of the formed S+."""
+    import torch
+    from paper_2309_08079_gb300.solver import LQTensors, make_opts, read_stats
+    s = solver()
+    Ns = [N] * 39 + [N - 3]
+    batch = gen.kuka_batch(nx, nu, Ns, 3900).astype(dtype)
+    lt = LQTensors.from_batch(batch, dtype=getattr(torch, dtype))
+    sch = s.alloc_schur(lt)
+    s.form(lt, sch)
+    o = make_opts(cluster=C, tol=1e-6 if dtype == "float32" else 1e-13)
+    sh = s.pcg_shape(lt, sch, o)
+    assert sh["C"] == C and (sh["clusters"] == 40) == at_once, sh
+    lam = torch.zeros(lt.total, nx, dtype=lt.dtype, device="cuda")
+    st = read_stats(s.pcg_solve(lt, sch, lam, o))
+    lam, Sd, So, g = (x.cpu().double().numpy() for x in (lam, sch.Sd, sch.So, sch.gamma))
+    for b in (0, 17, 39):
+        k0, k1 = batch.knot_off[b], batch.knot_off[b + 1]
+        ref = spla.spsolve(oracle.block_tridiag_sparse(Sd[k0:k1], So[k0 - b:k1 - b - 1]).tocsc(), -g[k0:k1].ravel())
+        assert st["status"][b] == 0 and oracle.relerr(lam[k0:k1].ravel(), ref) < (TOL_F32 if dtype == "float32" else 1e-9), b
