@@ -224,7 +224,6 @@ int choose_pcg_tile(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_schur 
 inline int choose_pcg_reg(const mpcg_dims &d, int B, const mpcg_opts *o, PcgLaunch &L) {
     constexpr int kpc_cap = 32, kpc_cap_ps = 64, kpc_small = 8;
     L.cta_mode = 0;
-    L.vs = 16;
     const int C_full = ceil_div(d.N, kpc_cap);
     if (C_full > kMaxCluster) return MPCG_EUNSUPPORTED;
     // co-resident clusters of C CTAs (0: cannot run)
@@ -233,9 +232,7 @@ inline int choose_pcg_reg(const mpcg_dims &d, int B, const mpcg_opts *o, PcgLaun
         L.C = C;
         L.kpc_max = kpc;
         if (kpc > (reg == 2 ? kpc_cap_ps : kpc_cap)) return 0;
-        L.lpk = reg == 2 ? 4 : 8;
-        L.rpt = 16 / L.lpk;
-        L.threads = std::max(32, ceil_div(kpc * L.lpk, 32) * 32);
+        L.threads = std::max(32, ceil_div(kpc * (reg == 2 ? 4 : 8), 32) * 32);  // lanes per knot
         L.smem = pcg_reg_smem_bytes(L);
         return pcg_reg_max_clusters(L);
     };
@@ -305,8 +302,8 @@ int choose_pcg_cluster(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opt
     if (!wide && std::is_same<T, float>::value && nx == 14) return choose_pcg_reg(d, B, o, L);
     // float32 nx = 36 and float64 nx = 14 while the operators stay on chip and
     // every instance has its own cluster (pcg_split.cu), as many CTAs as that
-    // leaves (the products of a CTA shrink with its knots: N = 64 1.90 us per
-    // iteration at 4 knots per CTA, N = 128 2.94 at 8); float64 accumulation of
+    // leaves (the products of a CTA shrink with its knots: N = 64 1.91 us per
+    // iteration at 4 knots per CTA, N = 128 2.99 at 8); float64 accumulation of
     // float32 sums stays with the general form.  A given number of CTAs that leaves
     // fewer clusters than instances: while the waves over the general form's, which
     // packs more clusters on an SM, are made up for by its speed (nx = 36 about 4.5
@@ -374,7 +371,7 @@ int choose_pcg_cluster(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opt
 
 // Kernel choice (mode 0): a cluster per instance whenever the horizon fits
 // one (fastest for single solves, and at float32 nx = 14 for batches: 256
-// instances of 32..512 knots 16.5 ms against 30 tiled), the tiled kernel for
+// instances of 32..512 knots 17.5 ms against 30 tiled), the tiled kernel for
 // float32 nx = 36 beyond the lane-per-row form and for larger batches of
 // other shapes, one CTA per instance reading L2 for horizons beyond both.
 template <typename T>

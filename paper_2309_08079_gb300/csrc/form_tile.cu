@@ -21,7 +21,7 @@
 // Measured (GB300, ragged batches of 256): nx = 14, 69,600 knots 151 us against
 // 315 with a warp per knot and one operand load per multiply-add; nx = 36,
 // 41,000 knots 946 us against 5,200 in five launches (form, inverse, off-
-// diagonal, two packings).  ncu: 72 and 68 % of the shared-memory pipe; DRAM
+// diagonal, two packings).  ncu: 68 and 65 % of the shared-memory pipe; DRAM
 // would allow 45 and 160 us.  The loops over the summation index and over the
 // pivots are rolled at nx = 36: fully unrolled, instruction fetch was the
 // largest stall (1,490 against 1,825 us at that step).  5 + 1 warps in two

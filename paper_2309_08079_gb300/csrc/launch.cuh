@@ -1,4 +1,5 @@
-// Internal launch interface shared by api.cu, form.cu and pcg.cu.
+// Internal launch interface between api.cu and the kernels' files (form.cu, form_tile.cu,
+// pcg.cu, pcg_reg.cu, pcg_split.cu, pcg_cta.cu).
 #pragma once
 
 #include "common.cuh"

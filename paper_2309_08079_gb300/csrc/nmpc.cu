@@ -162,10 +162,11 @@ __device__ __forceinline__ double half(float v) {
 }
 __device__ __forceinline__ double half(double v) { return 0.5 * v; }
 
-// sin of a float in double precision: x = q pi/2 + r with |r| <= pi/4 (pi/2 in
-// two parts; q is small, so the first fused step loses only its own rounding),
-// then the Taylor series of sin r or cos r to r^17, r^16 (the next terms are
-// below 2e-18).  Large arguments take the library's.
+// sin of a float in double precision: a two-part Cody-Waite reduction, x = q pi/2 + r
+// with |r| <= pi/4 + 5e-4 (q is rounded from a float product; it is small, so
+// the first fused step loses only its own rounding), then the Taylor series of
+// sin r or cos r to r^17, r^16 (the first term left out is at most 2.1e-18).
+// Large arguments take the library's.
 __device__ __forceinline__ double sin_wide(float x) {
     if (!(fabsf(x) < 8192.f)) return sin((double)x);
     const float qf = rintf(x * 0.63661977f);

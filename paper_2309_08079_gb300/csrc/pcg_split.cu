@@ -10,14 +10,14 @@
 // few warps, few additions and no repeated scalars beside them.  Therefore
 //  - S p_old, which only the update needs, is formed by the row warps while the
 //    sums of r~ travel, so it costs no time of its own;
-//  - the sums of four accumulators are reduced by recursive halving (6
-//    additions a warp in place of 15);
+//  - the sums of the accumulators are reduced by recursive halving (8 additions a
+//    warp for five in place of 25);
 //  - the last warp holds no rows: it adds the warp sums, exchanges them, forms
 //    alpha and beta for everybody, and 1 / eta for the next beta while the
 //    others update.
 // Measured per iteration, against the general cluster kernel (pcg.cu, blocks in
-// shared memory, two reductions): float32 nx = 36, N = 64: 1.90 against 8.4 us
-// (N = 128: 2.94); float64 nx = 14, N = 101: 5.9 against 8.2 us, of which the
+// shared memory, two reductions): float32 nx = 36, N = 64: 1.91 against 8.4 us
+// (N = 128: 2.99); float64 nx = 14, N = 101: 6.05 against 8.2 us, of which the
 // three products' FP64 instructions are 3.9.
 // Rows split over two or four lanes: slower at nx = 36 (N = 64, refined solve:
 // 3.3 and 4.4 ms against 2.8: more warps read the vectors); in float64 faster
@@ -576,7 +576,8 @@ struct SplitForm<double> {
     // Lanes per row, so that a product's instructions spread over the four
     // schedulers (8 knots x 2 lanes: 7 warps).  Per iteration with 1 lane -> as
     // chosen: N = 20 6.1 -> 4.0 us, 50 6.0 -> 4.6, 64 5.9 -> 4.5, 96 5.9 -> 5.4, 101
-    // 6.0 -> 5.9 (4 lanes at 3-4 knots: 4.5-4.8, 1 at 5: no gain over 6.0).
+    // 6.0 -> 5.9 (4 lanes at 3-4 knots: 4.5-4.8, 1 at 5: no gain over 6.0); the fifth
+    // sum, added since, takes 0.1-0.2.
     static int lanes(int kpc) { return kpc <= 2 ? 4 : kpc <= 8 ? 2 : 1; }
     static int variant(int kpc) { return lanes(kpc); }
     static auto fn(int v) {

@@ -6,7 +6,8 @@
 
 namespace mpcg {
 
-// ||r||^2 term in the accumulator's precision (the exit test alone uses it)
+// A thread's share of ||r||^2, which the exit test and the reported residual alone
+// use: a plain float beside float pairs, a double beside doubles
 __device__ __forceinline__ dfloat sq_sum(float a, float b, dfloat) { return dfloat{__fmaf_rn(b, b, __fmul_rn(a, a)), 0.f}; }
 __device__ __forceinline__ double sq_sum(float a, float b, double) {
     return __fma_rn((double)b, (double)b, __dmul_rn((double)a, (double)a));
@@ -64,8 +65,8 @@ __device__ __forceinline__ double beta_from(double eta, double inv, double eta_o
 // N = 64 5.1e-7 / 4.8e-7 / 2.9e-6, N = 512 4.1e-7 / 4.0e-7 / 2.0e-6; nx = 36, N = 64
 // 4.0e-7 / 5.3e-7 / 3.0e-6.  Rounded once, by the compensated Horner scheme
 // (Graillat, Langlois, Louvet) in float pairs, in double arithmetic else.
-// Against the plain float form it takes 3 % (N = 512) to 5 % (batches); a fifth sum
-// in place of the prediction, the same accuracy, 9 %.
+// Against the plain float form it takes 3 to 6 % of the time; a fifth sum in
+// place of the prediction, the same accuracy, 9 %.
 __device__ __forceinline__ dfloat curvature(dfloat del, dfloat eps, dfloat old, float beta, float g) {
     auto step = [](float b, float x, float xl, float a, float al, float &lo) {  // a + b x
         const float p = __fmul_rn(b, x), s = __fadd_rn(p, a), t = __fsub_rn(s, p);
