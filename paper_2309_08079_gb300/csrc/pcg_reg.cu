@@ -586,7 +586,8 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
         // Scalars of the iteration (alpha, beta, exit tests) are taken in
         // float from the extended sums.
         A eta = AT::zero(), acc = AT::zero();  // acc: p^T S p
-        float inv_eta = 0.f, rr = 0.f, g = 0.f;  // g: the last beta
+        float rr = 0.f, g = 0.f;  // g: the last beta
+        EtaRecip<float> recip;
         int iters = 0;
         bool broke = false;
         int it = 0;
@@ -654,12 +655,12 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
                 }
             }
             const float etan = AT::to_T(S.eta);
-            const float beta = beta_from(etan, inv_eta, AT::to_T(eta));  // 0 in the first iteration
+            const float beta = recip.beta(etan, 0.f);  // 0 in the first iteration
             eta = S.eta;
             rr = S.rr;
             const A old = acc;
             acc = curvature(S.del, S.eps, acc, beta, g);
-            float ups = AT::to_T(acc), alpha = __fdividef(etan, ups);
+            float ups = rounded(acc, 0.f), alpha = __fdividef(etan, ups);
             const bool done = !(fabsf(etan) <= 3.402823466e38f && rr <= 3.402823466e38f) ||
                               (mode1 ? etan < tol_t : rr <= tol_t) || it >= max_iter;
             const bool direct = doubtful(ups, S.del, S.eps, old, beta, g);
@@ -709,7 +710,7 @@ __global__ void __launch_bounds__(32 * WMAX, 1) pcg_reg_kernel(const PcgParams<f
                 next_p();
                 if (!direct) apply();
             }
-            inv_eta = __fdividef(1.f, etan);
+            recip.set(etan);
             g = beta;
             iters = it;
             __syncthreads();

@@ -400,8 +400,9 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
         __syncthreads();
 
         const T big = sizeof(T) == 4 ? (T)3.402823466e38f : (T)1.7976931348623157e308;
-        A acc = AT::zero();                     // p^T S p; this and the next two the sums warp's
-        T inv_eta = T(0), rr = T(0), g = T(0);  // g (every warp's): the last beta (FIFTH: 0)
+        A acc = AT::zero();     // p^T S p; this, rr and recip the sums warp's
+        T rr = T(0), g = T(0);  // g (every warp's): the last beta (FIFTH: 0)
+        EtaRecip<T> recip;
         int iters = 0;
         bool broke = false, late = false;  // late: this warp gave up waiting for S p rows
         for (int it = 0; !timed_out; ++it) {
@@ -426,7 +427,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
                     mbar_arrive_expect(mb + Z, halo_bytes);
                     mbar_arrive_expect(mb + TT, halo_bytes);
                 }
-                if (it > 0) inv_eta = quot(T(1), AT::to_T(eta));
+                if (it > 0) recip.set(AT::to_T(eta));
             }
             __syncthreads();
             if (!sums) {
@@ -447,11 +448,11 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_split_kernel(const PcgParams<T> P
                 // ---- alpha, beta and the exit tests, in T from the extended sums ---------
                 const Sums S = collect(1u);
                 const T etan = AT::to_T(S.eta);
-                const T beta = beta_from(etan, inv_eta, AT::to_T(eta));  // 0 in the first iteration
+                const T beta = recip.beta(etan, AT::to_T(eta));  // 0 in the first iteration
                 if (FIFTH) acc = S.old;
                 const A old = acc;
                 acc = curvature(S.del, S.eps, acc, beta, g);
-                const T ups = AT::to_T(acc), alpha = quot(etan, ups);
+                const T ups = rounded(acc, T(0)), alpha = quot(etan, ups);
                 eta = S.eta;
                 rr = S.rr;
                 const bool done = !(fabs(etan) <= big && rr <= big) || (mode1 ? etan < tol_t : rr <= tol_t) || it >= max_iter;
