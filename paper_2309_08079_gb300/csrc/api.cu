@@ -171,7 +171,7 @@ int choose_pcg_tile(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_schur 
     };
     int n = shape(1);  // what one CTA cannot hold stays refused
     if (n < 1) return MPCG_EUNSUPPORTED;
-    L.n_cta = n;
+    L.n_cta = L.no_queue = n;
     const PcgLaunch one = L;
     // `clusters` (float32 nx = 36): as many CTAs per instance as pays.  One
     // iteration of an instance takes about 6 us + 0.35 us per knot of a CTA
@@ -356,6 +356,7 @@ int choose_pcg_cluster(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opt
         const int active = pcg_max_clusters<T>(L);
         if (in_turn.clusters > 0 && (active < 1 || ceil_div(B, in_turn.clusters) <= speed * ceil_div(B, active))) {
             L = in_turn;
+            L.no_queue = active;  // the general form holds them at once, without a workspace
             return MPCG_OK;
         }
         if (active >= 1) {
@@ -493,8 +494,8 @@ int pcg_t(mpcg_handle *h, const mpcg_dims &d, int B, const int *knot_off, const 
     P.npk = packed_len(d.nx);
     if (P.inst_list && !knot_off) return MPCG_EINVAL;
     if (P.n_tickets > 1 && (L.clusters < P.n_tickets || L.light.clusters > 0)) {
-        // (a batch that needs none with a CTA per instance is dealt out in turn)
-        if (!ws && P.n_tickets > L.n_cta) return MPCG_EINVAL;
+        // (a batch that needs none in another form is dealt out in turn)
+        if (!ws && P.n_tickets > L.no_queue) return MPCG_EINVAL;
         P.queue = (int *)ws;
         if (ws) {
             rc = err_cuda(cudaMemsetAsync(ws, 0, 3 * QUEUE_LEVELS * sizeof(int), st));  // a counter per stage and level

@@ -75,6 +75,8 @@ struct PcgLaunch {
     } light;
     int n_mid, n_low;  // reg: clusters of the later stages, 3/4 and 1/2 of the full
                    // size (0: one launch; see pcg_reg.cu)
+    int no_queue;  // instances that need no queue in another form of the launch, and so
+                   // no workspace in this one either (they are dealt out in turn)
     int n_cta;     // tiled: instances that one CTA each takes at a time
     // tiled with C > 1: the form with one CTA per instance, where the device chooses
     // by the horizons (clusters > 0), and the clusters at a time of this one

@@ -324,3 +324,30 @@ def test_fixed_cluster_batches_run_at_once_where_that_is_faster(nx, nu, dtype, N
         k0, k1 = batch.knot_off[b], batch.knot_off[b + 1]
         ref = spla.spsolve(oracle.block_tridiag_sparse(Sd[k0:k1], So[k0 - b:k1 - b - 1]).tocsc(), -g[k0:k1].ravel())
         assert st["status"][b] == 0 and oracle.relerr(lam[k0:k1].ravel(), ref) < (TOL_F32 if dtype == "float32" else 1e-9), b
+
+
+@pytest.mark.parametrize("N,C", [(16, 8), (16, 4), (5, 2)])
+def test_fixed_cluster_batch_without_a_workspace(N, C):
+    """nx = 36, 40 (80) instances with a given number of CTAs: the general kernel
+    holds them all at once and needs no workspace, so the lane-per-row kernel,
+    which takes them in turn, needs none either; the same bits as with one."""
+    import ctypes
+
+    import torch
+    from paper_2309_08079_gb300.solver import LQTensors, make_opts, read_stats
+    s = solver()
+    B = 80 if N == 5 else 40
+    lt = LQTensors.from_batch(gen.kuka_batch(36, 12, [N] * B, 3950).astype(np.float32))
+    sch = s.alloc_schur(lt)
+    s.form(lt, sch)
+    o, ss = make_opts(cluster=C), sch.struct()
+    assert s.pcg_shape(lt, sch, o)["clusters"] < B
+    out = []
+    for ws in (s.alloc_workspace(lt), None):
+        lam, st = torch.zeros(lt.total, 36, device="cuda"), s.alloc_stats(B)
+        assert s.lib.mpcg_pcg_solve_batched(s.h, lt.dims(), lt.nb, lt.knot_off.data_ptr(), ctypes.byref(ss), lam.data_ptr(),
+                                            ctypes.byref(o), st.data_ptr(), None if ws is None else ws.data_ptr(),
+                                            torch.cuda.current_stream().cuda_stream) == 0
+        assert (read_stats(st)["status"] == 0).all()
+        out.append(lam)
+    assert torch.equal(*out)
