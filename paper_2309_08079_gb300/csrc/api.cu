@@ -302,7 +302,7 @@ int choose_pcg_cluster(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opt
     if (!wide && std::is_same<T, float>::value && nx == 14) return choose_pcg_reg(d, B, o, L);
     // float32 nx = 36 and float64 nx = 14 while the operators stay on chip and
     // every instance has its own cluster (pcg_split.cu), as many CTAs as that
-    // leaves (the products of a CTA shrink with its knots: N = 64 1.91 us per
+    // leaves (the products of a CTA shrink with its knots: N = 64 1.89 us per
     // iteration at 4 knots per CTA, N = 128 2.99 at 8); float64 accumulation of
     // float32 sums stays with the general form.  A given number of CTAs that leaves
     // fewer clusters than instances: while the waves over the general form's, which
@@ -372,7 +372,7 @@ int choose_pcg_cluster(mpcg_handle *h, const mpcg_dims &d, int B, const mpcg_opt
 
 // Kernel choice (mode 0): a cluster per instance whenever the horizon fits
 // one (fastest for single solves, and at float32 nx = 14 for batches: 256
-// instances of 32..512 knots 17.5 ms against 30 tiled), the tiled kernel for
+// instances of 32..512 knots 17.1 ms against 30 tiled), the tiled kernel for
 // float32 nx = 36 beyond the lane-per-row form and for larger batches of
 // other shapes, one CTA per instance reading L2 for horizons beyond both.
 template <typename T>

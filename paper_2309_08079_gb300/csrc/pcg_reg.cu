@@ -22,12 +22,12 @@
 // identity cancels (p^T S p below about 1/32 of its terms; 0.29 of r~^T S r~ was the
 // smallest share seen on the emulated problems) or too much of the carried
 // error is passed on, the sum p^T S p is taken directly with one more
-// reduction.  Measured on GB300 at fixed iteration counts: 1.84 us per
-// iteration at N = 512 (16 CTAs x 32 knots) and 1.60 at N = 128 (16 x 8) against
-// 2.23 and 1.98 with two reductions.  Of the 1.84 us, by leaving parts out one
+// reduction.  Measured on GB300 at fixed iteration counts: 1.83 us per
+// iteration at N = 512 (16 CTAs x 32 knots) and 1.57 at N = 128 (16 x 8) against
+// 2.23 and 1.98 with two reductions.  Of the 1.83 us, by leaving parts out one
 // at a time: the three products 0.2-0.3 each (bound by the shared-memory reads
 // of the vectors, 128 bytes per clock), the warp sums 0.11, the CTA sums 0.11,
-// the sums over CTAs 0.06, p^T S p in float pairs 0.07; the rest is the transport
+// the sums over CTAs 0.06, p^T S p in float pairs 0.06; the rest is the transport
 // (0.12 one way) and the CTA barriers.
 //
 // Launch shape: clusters of C <= 16 CTAs; a group of G CTAs (the whole
@@ -49,7 +49,7 @@
 // Former form -> this one: 256 instances of 32..512 knots 19.9 -> 16.5 ms, 256 of
 // 60..64 1.48 -> 1.05, 150 of 100..250 5.85 -> 4.9, 17 of 505..512 3.97 -> 3.8.
 // (These times, and those below, are of a p^T S p in plain float; in pairs batches
-// take 3 to 6 % more: 17.5, 1.11, 5.1 and 4.0 ms.)
+// take 3 to 5 % more: 17.1, 1.10, 5.05 and 4.0 ms.)
 //
 // Choice of the form: PS pays once the other would need a second wave; that
 // depends on the horizons, which the host does not know.  Between one and four

@@ -16,7 +16,7 @@
 //    alpha and beta for everybody, and 1 / eta for the next beta while the
 //    others update.
 // Measured per iteration, against the general cluster kernel (pcg.cu, blocks in
-// shared memory, two reductions): float32 nx = 36, N = 64: 1.91 against 8.4 us
+// shared memory, two reductions): float32 nx = 36, N = 64: 1.89 against 8.4 us
 // (N = 128: 2.99); float64 nx = 14, N = 101: 6.05 against 8.2 us, of which the
 // three products' FP64 instructions are 3.9.
 // Rows split over two or four lanes: slower at nx = 36 (N = 64, refined solve:

@@ -85,7 +85,7 @@ __device__ __forceinline__ double rounded(double a, double) { return a; }
 // N = 64 5.1e-7 / 4.8e-7 / 2.9e-6, N = 512 4.1e-7 / 4.0e-7 / 2.0e-6; nx = 36, N = 64
 // 4.0e-7 / 5.3e-7 / 3.0e-6.  Rounded once, by the compensated Horner scheme
 // (Graillat, Langlois, Louvet) in float pairs, in double arithmetic else.
-// Against the plain float form it takes 3 to 6 % of the time; a fifth sum in
+// Against the plain float form it takes 2 to 5 % of the time; a fifth sum in
 // place of the prediction, the same accuracy, 9 %.
 __device__ __forceinline__ dfloat curvature(dfloat del, dfloat eps, dfloat old, float beta, float g) {
     auto step = [](float b, float x, float xl, float a, float al, float &lo) {  // a + b x
